@@ -34,8 +34,8 @@
 // k_sift_cov:     64 descriptors per step in shared memory, transposed;
 //                 every thread accumulates 64 of the 128 x 128 products with
 //                 dp4a, flushed into 64-bit sums.
-// k_sift_axes:    one CTA: mean, covariance, power iterations, projection
-//                 weights.
+// k_sift_axes:    one cluster of four CTAs: mean, covariance, power
+//                 iterations, projection weights.
 // k_sift_project: phi of every pixel of one scale of the four images.
 #include <algorithm>
 
@@ -246,75 +246,136 @@ __global__ void __launch_bounds__(kCovThreads) k_sift_cov(SiftJob J, size_t coun
     flush();
 }
 
-// Dot product of two 128-vectors in shared memory as in the power
-// iteration: threads 0-3 each accumulate the indices of one residue mod 4 in
-// index order by fused multiply-adds; thread 0 combines (s0 + s1) + (s2 + s3)
-// into *out.  Called by the whole CTA (two barriers).
-__device__ __forceinline__ void dot128_cta(const double* a, const double* b, double* part, double* out) {
-    const int i = threadIdx.x;
-    if (i < 4) {
-        double t = 0.0;
-#pragma unroll 8
-        for (int k = i; k < kDesc; k += 4) t = __fma_rn(a[k], b[k], t);
-        part[i] = t;
-    }
-    __syncthreads();
-    if (i == 0) *out = __dadd_rn(__dadd_rn(part[0], part[1]), __dadd_rn(part[2], part[3]));
-    __syncthreads();
+// The principal axes, by one cluster of kAxesCtas CTAs.  The FP64 pipe bounds
+// it: a warp's DFMA holds its SM sub-partition for 64 clocks however many lanes
+// are active, and the definition fixes the order of every sum, so an iteration
+// is a chain of 32 dependent DFMAs for the matrix rows, 32 for each deflation
+// dot product and 32 for the norm.  One thread per (row, residue mod 4) chain:
+// 512 chains are 16 warps, one per sub-partition of four SMs, so the rows take
+// one chain's time (2080 clocks) instead of the four that one SM needs.  A
+// thread keeps its 32 covariance entries and the earlier axes' entries of its
+// residue in registers; each row's sum goes to all four CTAs through
+// distributed shared memory, one cluster barrier per iteration.  The dot
+// products are computed by every warp for itself (its own sub-partition would
+// idle otherwise), so they need no barrier.  5573 -> 3169 us (one CTA before).
+constexpr int kAxesCtas = 4;
+constexpr int kChain = kDesc / 4;  // terms of one residue's sum
+
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// One CTA of 128 threads: thread i owns row i of the covariance, kept
-// column-major in shared memory (Ct[j][i] = C(i, j)) so that a warp reads 32
-// consecutive doubles at every step of its rows.  Every dot product of the
-// iteration is four partial sums over the indices mod 4 in index order by
-// fused multiply-adds, combined as (s0 + s1) + (s2 + s3).
-__global__ void __launch_bounds__(kDesc) k_sift_axes(SiftJob J, double count) {
-    extern __shared__ double Ct[];  // [128][128], column-major covariance
-    __shared__ double mean[kDesc], v[kDesc], wv[kDesc], ax[3][kDesc], part[4], bc;
-    const int i = threadIdx.x;
-    mean[i] = __ddiv_rn((double)J.s1[i], count);
+// Stores v at the address that p has in the shared memory of CTA `rank`.
+__device__ __forceinline__ void store_remote(double* p, int rank, double v) {
+    asm volatile(
+        "{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %0, %1;\n\tst.shared::cluster.f64 [a], %2;\n\t}" ::"r"(
+            (unsigned)__cvta_generic_to_shared(p)),
+        "r"(rank), "d"(v)
+        : "memory");
+}
+
+// (s0 + s1) + (s2 + s3) of the partial sums of four neighbouring lanes (lane
+// mod 4 = the residue), on every lane.
+__device__ __forceinline__ double combine4(double s) {
+    s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, 1));
+    return __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, 2));
+}
+
+// Axis c by the power iteration.  cov: this thread's row at its residue; ax /
+// axr: the earlier axes, whole in shared memory / at this thread's residue.
+template <int c>
+__device__ __forceinline__ void power_axis(const double (&cov)[kChain], const double (&axr)[2][kChain],
+                                           double (*ax)[kDesc], double* v, double (*raw)[kDesc], double (*upd)[kDesc]) {
+    const int i = threadIdx.x, r = i & 3;
+    const int row = (int)blockIdx.x * (kDesc / kAxesCtas) + (i >> 2);
+    v[i] = 1.0;
     __syncthreads();
-    for (int j = 0; j < kDesc; ++j)
-        Ct[j * kDesc + i] = __dsub_rn(__ddiv_rn((double)J.s2[i * kDesc + j], count), __dmul_rn(mean[i], mean[j]));
-    __syncthreads();
-    for (int c = 0; c < 3; ++c) {
-        v[i] = 1.0;
-        __syncthreads();
-        for (int it = 0; it < kPowerIters; ++it) {
-            double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-#pragma unroll 4
-            for (int k = 0; k < kDesc; k += 4) {
-                s0 = __fma_rn(Ct[(k + 0) * kDesc + i], v[k + 0], s0);
-                s1 = __fma_rn(Ct[(k + 1) * kDesc + i], v[k + 1], s1);
-                s2 = __fma_rn(Ct[(k + 2) * kDesc + i], v[k + 2], s2);
-                s3 = __fma_rn(Ct[(k + 3) * kDesc + i], v[k + 3], s3);
-            }
-            wv[i] = __dadd_rn(__dadd_rn(s0, s1), __dadd_rn(s2, s3));
-            __syncthreads();
-            for (int e = 0; e < c; ++e) {
-                dot128_cta(ax[e], wv, part, &bc);
-                wv[i] = __dsub_rn(wv[i], __dmul_rn(bc, ax[e][i]));
-                __syncthreads();
-            }
-            dot128_cta(wv, wv, part, &bc);
-            const double nr = __dsqrt_rn(bc);
-            v[i] = nr > 0.0 ? __ddiv_rn(wv[i], nr) : 0.0;
+    double vi = 0.0;
+    for (int it = 0; it < kPowerIters; ++it) {
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < kChain; ++k) s = __fma_rn(cov[k], v[4 * k + r], s);
+        s = combine4(s);
+        // the buffers alternate: a CTA writes one again only after the next
+        // barrier, which every CTA reaches when it has read it
+        double* w = raw[it & 1];
+        store_remote(w + row, r, s);
+        cluster_barrier();
+        double wi = w[i];
+#pragma unroll
+        for (int e = 0; e < c; ++e) {
+            double t = 0.0;
+#pragma unroll
+            for (int k = 0; k < kChain; ++k) t = __fma_rn(axr[e][k], w[4 * k + r], t);
+            wi = __dsub_rn(wi, __dmul_rn(combine4(t), ax[e][i]));
+            w = upd[e];
+            w[i] = wi;
             __syncthreads();
         }
-        if (i == 0) {
-            int big = 0;
-            for (int k = 1; k < kDesc; ++k)
-                if (fabs(v[k]) > fabs(v[big])) big = k;
-            bc = v[big] < 0.0 ? -1.0 : 1.0;
-        }
-        __syncthreads();
-        ax[c][i] = __dmul_rn(bc, v[i]);
-        J.axes[c * kDesc + i] = ax[c][i];
+        double t = 0.0;
+#pragma unroll
+        for (int k = 0; k < kChain; ++k) t = __fma_rn(w[4 * k + r], w[4 * k + r], t);
+        const double nr = __dsqrt_rn(combine4(t));
+        vi = nr > 0.0 ? __ddiv_rn(wi, nr) : 0.0;
+        v[i] = vi;
         __syncthreads();
     }
-    // single-precision projection weights and biases fl(a_c . mean), the
-    // bias a sequential sum
-    for (int c = 0; c < 3; ++c) J.proj[c * kDesc + i] = (float)ax[c][i];
+    // the largest component (the first of equals) made positive; magnitudes
+    // order like their bit patterns
+    if (i < 32) {
+        unsigned long long best = 0ull;
+        int big = 0;
+        for (int k = i; k < kDesc; k += 32) {
+            const unsigned long long m = (unsigned long long)__double_as_longlong(v[k]) & 0x7fffffffffffffffull;
+            if (k == i || m > best) {
+                best = m;
+                big = k;
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long om = __shfl_xor_sync(0xffffffffu, best, o);
+            const int ob = __shfl_xor_sync(0xffffffffu, big, o);
+            if (om > best || (om == best && ob < big)) {
+                best = om;
+                big = ob;
+            }
+        }
+        if (i == 0) raw[0][0] = v[big] < 0.0 ? -1.0 : 1.0;
+    }
+    __syncthreads();
+    ax[c][i] = __dmul_rn(raw[0][0], vi);
+    // no CTA writes raw[0] again (the next axis) before all have read the sign
+    cluster_barrier();
+}
+
+__global__ void __cluster_dims__(kAxesCtas, 1, 1) __launch_bounds__(kDesc) k_sift_axes(SiftJob J, double count) {
+    __shared__ double mean[kDesc], v[kDesc], ax[3][kDesc], raw[2][kDesc], upd[2][kDesc];
+    const int i = threadIdx.x, r = i & 3;
+    const int row = (int)blockIdx.x * (kDesc / kAxesCtas) + (i >> 2);
+    mean[i] = __ddiv_rn((double)J.s1[i], count);
+    __syncthreads();
+    double cov[kChain], axr[2][kChain];
+#pragma unroll
+    for (int k = 0; k < kChain; ++k)
+        cov[k] = __dsub_rn(__ddiv_rn((double)J.s2[row * kDesc + 4 * k + r], count),
+                           __dmul_rn(mean[row], mean[4 * k + r]));
+    cluster_barrier();  // every CTA of the cluster runs before the first remote store
+    power_axis<0>(cov, axr, ax, v, raw, upd);
+#pragma unroll
+    for (int k = 0; k < kChain; ++k) axr[0][k] = ax[0][4 * k + r];
+    power_axis<1>(cov, axr, ax, v, raw, upd);
+#pragma unroll
+    for (int k = 0; k < kChain; ++k) axr[1][k] = ax[1][4 * k + r];
+    power_axis<2>(cov, axr, ax, v, raw, upd);
+    if (blockIdx.x != 0) return;  // the last cluster barrier is behind every remote store
+    // axes, single-precision projection weights and biases fl(a_c . mean),
+    // the bias a sequential sum
+    for (int c = 0; c < 3; ++c) {
+        J.axes[c * kDesc + i] = ax[c][i];
+        J.proj[c * kDesc + i] = (float)ax[c][i];
+    }
     if (i < 3) {
         double b = 0.0;
         for (int k = 0; k < kDesc; ++k) b = __dadd_rn(b, __dmul_rn(ax[i][k], mean[k]));
@@ -405,10 +466,6 @@ extern "C" int sff_sift_features(const uint8_t* const* rgb_dev4, int32_t pitch_b
     cudaStream_t st = (cudaStream_t)stream;
     const dim3 g((width + 127) / 128, height, 4);
     const dim3 gd((width + kDescThreads / 4 - 1) / (kDescThreads / 4), height, 4);
-    // the attribute is per device: set it on the current one at every call
-    if (cudaFuncSetAttribute(k_sift_axes, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kDesc * kDesc * (int)sizeof(double)) != cudaSuccess)
-        return SFF_ERR_CUDA;
     for (int s = 0; s < params->num_scales; ++s) {
         J.s = s;
         J.n = 1 << s;
@@ -420,7 +477,7 @@ extern "C" int sff_sift_features(const uint8_t* const* rgb_dev4, int32_t pitch_b
             const size_t count = 4 * (size_t)width * height;
             const int blocks = (int)std::min<size_t>((count + kCovPix - 1) / kCovPix, 152 * 4);
             SFF_LAUNCH(k_sift_cov, dim3(blocks), kCovThreads, 0, st, J, count);
-            SFF_LAUNCH(k_sift_axes, dim3(1), kDesc, kDesc * kDesc * sizeof(double), st, J, (double)count);
+            SFF_LAUNCH(k_sift_axes, dim3(kAxesCtas), kDesc, 0, st, J, (double)count);
         }
         SFF_LAUNCH(k_sift_project, g, 128, 0, st, J);
     }
