@@ -426,7 +426,7 @@ int sff_emit_seeds_noalloc(const int16_t* fwd_dev, const int32_t* fwd_cost_dev,
  * operation follows this fixed order, fused multiply-adds only there, so
  * results are reproducible bit for bit. */
 
-/* Scratch of sff_sift_features: about 650 bytes per pixel; 0 for invalid sizes. */
+/* Scratch of sff_sift_features: about 516 bytes per pixel; 0 for invalid sizes. */
 size_t sff_sift_workspace_bytes(int32_t width, int32_t height);
 
 /* phi of the four images at every scale.  rgb_dev4: host array of 4 device

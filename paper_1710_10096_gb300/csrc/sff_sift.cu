@@ -28,9 +28,8 @@
 // results are reproducible bit for bit on any IEEE machine.
 //
 // k_sift_grey:    smoothed grey image of one scale (4 images, blockIdx.z).
-// k_sift_grad:    magnitude and orientation sector per pixel.
-// k_sift_desc:    the quantised descriptor, four threads per pixel with 32
-//                 sums each in registers; the norms handed along in bin order.
+// k_sift_desc:    gradients, cell sums and quantised descriptors of a tile of
+//                 pixels, one thread per pixel.
 // k_sift_cov:     64 descriptors per step in shared memory, transposed;
 //                 every thread accumulates 64 of the 128 x 128 products with
 //                 dp4a, flushed into 64-bit sums.
@@ -45,7 +44,11 @@ namespace sff {
 namespace {
 
 constexpr int kDesc = 128;
-constexpr int kDescThreads = 128;  // threads of k_sift_desc: 32 pixels, four threads each
+// k_sift_desc: pixels per CTA (of one residue class mod n), the samples and
+// the cell positions that their descriptors read
+constexpr int kTileW = 32, kTileH = 16;
+constexpr int kSampW = kTileW + 11, kSampH = kTileH + 11;
+constexpr int kCellW = kTileW + 9, kCellH = kTileH + 9;
 constexpr int kCovPix = 64;       // descriptors per step of k_sift_cov
 constexpr int kCovThreads = 256;
 constexpr int kCovFlush = 16384;  // descriptors between flushes of the 32-bit partial sums
@@ -55,8 +58,6 @@ struct SiftJob {
     const uint8_t* rgb[4];
     int pitch, w, h, s, n;
     uint8_t* grey;           // [4][H][W]
-    float* mag;              // [4][H][W]
-    uint8_t* bin;            // [4][H][W]
     uint8_t* desc;           // [4][H][W][128]
     unsigned long long* s1;  // [128] sums
     unsigned long long* s2;  // [128][128] sums of products
@@ -97,101 +98,146 @@ __global__ void k_sift_grey(SiftJob J) {
     J.grey[((size_t)v * J.h + y) * J.w + x] = (uint8_t)((c[0] + 2 * c[1] + c[2] + 2) >> 2);
 }
 
-// Sector k of a direction: the rays of the sector boundaries are 45 degrees
-// apart; the direction lies in [ray k, ray k+1) exactly when its cross
-// product with ray k is >= 0 and with ray k+1 is < 0.
+// Sector k of a direction: [45 k, 45 k + 45) degrees, by sign and magnitude
+// after a half turn of the lower half-plane (any sector for a zero gradient,
+// whose magnitude is 0).
 __device__ __forceinline__ int sector_of(int dx, int dy) {
-    constexpr int rx[9] = {1, 1, 0, -1, -1, -1, 0, 1, 1}, ry[9] = {0, 1, 1, 1, 0, -1, -1, -1, 0};
-    int k = 0;
-#pragma unroll
-    for (int t = 7; t >= 0; --t)
-        if (rx[t] * dy - ry[t] * dx >= 0 && rx[t + 1] * dy - ry[t + 1] * dx < 0) k = t;
-    return k;
-}
-
-__global__ void k_sift_grad(SiftJob J) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y, v = blockIdx.z;
-    if (x >= J.w) return;
-    const uint8_t* g = J.grey + (size_t)v * J.h * J.w;
-    const int dx = (int)g[(size_t)y * J.w + min(x + J.n, J.w - 1)] - (int)g[(size_t)y * J.w + max(x - J.n, 0)];
-    const int dy = (int)g[(size_t)min(y + J.n, J.h - 1) * J.w + x] - (int)g[(size_t)max(y - J.n, 0) * J.w + x];
-    const size_t o = ((size_t)v * J.h + y) * J.w + x;
-    J.mag[o] = __fsqrt_rn((float)(dx * dx + dy * dy));
-    J.bin[o] = (uint8_t)sector_of(dx, dy);
-}
-
-// Sum of squares of the 128 values of a pixel's four-thread group in bin
-// order: thread r of the group holds bins 32 r .. 32 r + 31 and continues
-// the running sum of threads 0 .. r - 1, so the sum is the sequential one.
-// Every lane of the warp calls it.
-__device__ __forceinline__ float group_sum_sq(const float (&h)[32], int r, int lane) {
-    float ss = 0.0f;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        if (r == q) {
-#pragma unroll
-            for (int b = 0; b < 32; ++b) ss = __fadd_rn(ss, __fmul_rn(h[b], h[b]));
-        }
-        ss = __shfl_sync(0xffffffffu, ss, (lane & ~3) | q);
+    const bool lower = dy < 0 || (dy == 0 && dx < 0);
+    if (lower) {
+        dx = -dx;
+        dy = -dy;
     }
-    return ss;
+    const int k = dx > 0 ? (dy < dx ? 0 : 1) : (-dx < dy ? 2 : 3);
+    return lower ? k + 4 : k;
 }
 
-// The descriptor of one pixel per four threads: thread r of the group holds
-// the 32 sums of cell row r (bins 32 r .. 32 r + 31 in descriptor order) in
-// registers.  A bin's sum adds +0 for the samples of the other sectors,
-// which leaves it bit-identical to adding only its own samples.  Threads
-// past the image's edge compute on the last column and store nothing, so
-// that every lane takes part in the shuffles.
-__global__ void __launch_bounds__(kDescThreads, 7) k_sift_desc(SiftJob J) {
-    const int lane = threadIdx.x & 31, r = threadIdx.x & 3;
-    const int x = blockIdx.x * (kDescThreads / 4) + (threadIdx.x >> 2), y = blockIdx.y, v = blockIdx.z;
-    const bool valid = x < J.w;
-    const int xs = valid ? x : J.w - 1;
-    const size_t plane = (size_t)v * J.h * J.w;
-    const float* mag = J.mag + plane;
-    const uint8_t* bin = J.bin + plane;
-    float h[32];
+// Correctly rounded a / b for many a: with y = RN(1 / b), a faithful quotient
+// q and the exact remainder r = a - q b, RN(q + r y) = RN(a / b) (Markstein,
+// "Computation of elementary functions on the IBM RISC System/6000
+// processor", 1990, theorem on division).  q is faithful here because it is
+// rounded once from a (y + lo) with y + lo within 2^-47 of 1 / b.  Needs 0 <=
+// a <= 2^20 b with a and b in the normal range's middle (nothing below
+// underflows): magnitudes are 0 or at least 1 and at most 9 x 361 per bin.
+struct Divisor {
+    float b, y, lo;
+};
+__device__ __forceinline__ Divisor divisor_of(float b) {
+    Divisor d;
+    d.b = b > 0.0f ? b : 1.0f;  // an all-zero descriptor stays all zero
+    d.y = __frcp_rn(d.b);
+    d.lo = __fmul_rn(__fmaf_rn(-d.b, d.y, 1.0f), d.y);
+    return d;
+}
+__device__ __forceinline__ float quotient(float a, const Divisor& d) {
+    const float q = __fmaf_rn(a, d.y, __fmul_rn(a, d.lo));
+    return __fmaf_rn(__fmaf_rn(-q, d.b, a), d.y, q);
+}
+
+// Descriptors of a tile of kTileW x kTileH pixels whose coordinates share a
+// residue mod n, one thread per pixel.  A cell's 8 sums depend only on its
+// position, so they are computed once per position (kCellW x kCellH of them,
+// two per pixel) and read by the 16 descriptors that contain the cell; the
+// samples are n apart, hence the residue classes.  A bin's sum adds +0 for the
+// samples of the other sectors, which leaves it bit-identical to adding only
+// its own.  The thread reads its 128 values from shared memory three times
+// (norm, clipped norm, result): holding them would leave 12 warps per SM.  The
+// two halves of a position are separate planes, so that a warp's 16-byte
+// reads are conflict-free.  Bound by issue: per value 2 + 7 + 11 operations.
+// 1242 x 375, four images, four scales: 5127 us (each pixel's cells computed by
+// four threads, IEEE divide routine, separate gradient kernel of 55 us) ->
+// 929 us.
+__global__ void __launch_bounds__(kTileW * kTileH, 3) k_sift_desc(SiftJob J) {
+    __shared__ float4 cell[2][kCellW * kCellH];
+    __shared__ float mag[kSampW * kSampH];
+    __shared__ uint8_t bin[kSampW * kSampH];
+    const int n = J.n, t = threadIdx.x;
+    // residue (a, b) and tile
+    const int a = (int)blockIdx.x % n, b = (int)blockIdx.y % n;
+    const int x0 = a + n * kTileW * ((int)blockIdx.x / n), y0 = b + n * kTileH * ((int)blockIdx.y / n);
+    if (x0 >= J.w || y0 >= J.h) return;  // CTA-uniform
+    const size_t plane = (size_t)blockIdx.z * J.h * J.w;
+    const uint8_t* g = J.grey + plane;
+    // sample i of a row is image column x0 + n (i - 6), clamped
+    for (int k = t; k < kSampW * kSampH; k += kTileW * kTileH) {
+        const int x = clampi(x0 + n * (k % kSampW - 6), 0, J.w - 1), y = clampi(y0 + n * (k / kSampW - 6), 0, J.h - 1);
+        const uint8_t* row = g + (size_t)y * J.w;
+        const int dx = (int)row[min(x + n, J.w - 1)] - (int)row[max(x - n, 0)];
+        const int dy = (int)g[(size_t)min(y + n, J.h - 1) * J.w + x] - (int)g[(size_t)max(y - n, 0) * J.w + x];
+        mag[k] = __fsqrt_rn((float)(dx * dx + dy * dy));
+        bin[k] = (uint8_t)sector_of(dx, dy);
+    }
+    __syncthreads();
+    for (int k = t; k < kCellW * kCellH; k += kTileW * kTileH) {
+        const int o = (k / kCellW) * kSampW + k % kCellW;
+        float h[8];
 #pragma unroll
-    for (int b = 0; b < 32; ++b) h[b] = 0.0f;
+        for (int q = 0; q < 8; ++q) h[q] = 0.0f;
 #pragma unroll
-    for (int sj = 0; sj < 3; ++sj) {
-        const int qy = clampi(y + (r * 3 + sj - 6) * J.n, 0, J.h - 1);
-        const float* mrow = mag + (size_t)qy * J.w;
-        const uint8_t* brow = bin + (size_t)qy * J.w;
+        for (int j = 0; j < 3; ++j)
 #pragma unroll
-        for (int cx = 0; cx < 4; ++cx)
+            for (int i = 0; i < 3; ++i) {
+                const float m = mag[o + j * kSampW + i];
+                const int s = bin[o + j * kSampW + i];
 #pragma unroll
-            for (int si = 0; si < 3; ++si) {
-                const int qx = clampi(xs + (cx * 3 + si - 6) * J.n, 0, J.w - 1);
-                const float m = mrow[qx];
-                const int k = brow[qx];
-#pragma unroll
-                for (int b = 0; b < 8; ++b) h[cx * 8 + b] = __fadd_rn(h[cx * 8 + b], k == b ? m : 0.0f);
+                for (int q = 0; q < 8; ++q) h[q] = __fadd_rn(h[q], s == q ? m : 0.0f);
             }
+        cell[0][k] = make_float4(h[0], h[1], h[2], h[3]);
+        cell[1][k] = make_float4(h[4], h[5], h[6], h[7]);
     }
-    const float nr = __fsqrt_rn(group_sum_sq(h, r, lane));
-    if (nr > 0.0f) {
+    __syncthreads();
+    const int px = t % kTileW, py = t / kTileW;
+    const int x = x0 + n * px, y = y0 + n * py;
+    if (x >= J.w || y >= J.h) return;
+    const float4* c0 = &cell[0][py * kCellW + px];  // position of cell (0, 0); cells are 3 apart
+    constexpr int kHalf = kCellW * kCellH;
+    float ss = 0.0f;
+#pragma unroll 1
+    for (int j = 0; j < 4; ++j)
 #pragma unroll
-        for (int b = 0; b < 32; ++b) {
-            h[b] = __fdiv_rn(h[b], nr);
-            if (h[b] > 0.2f) h[b] = 0.2f;
+        for (int i = 0; i < 8; ++i) {
+            const float4 v = c0[3 * j * kCellW + 3 * (i >> 1) + (i & 1) * kHalf];
+            ss = __fadd_rn(ss, __fmul_rn(v.x, v.x));
+            ss = __fadd_rn(ss, __fmul_rn(v.y, v.y));
+            ss = __fadd_rn(ss, __fmul_rn(v.z, v.z));
+            ss = __fadd_rn(ss, __fmul_rn(v.w, v.w));
         }
-    }
-    const float nr2 = __fsqrt_rn(group_sum_sq(h, r, lane));
-    uint32_t word[8];
+    const Divisor d1 = divisor_of(__fsqrt_rn(ss));
+    ss = 0.0f;
+#pragma unroll 1
+    for (int j = 0; j < 4; ++j)
 #pragma unroll
-    for (int i = 0; i < 8; ++i) word[i] = 0u;
+        for (int i = 0; i < 8; ++i) {
+            const float4 v = c0[3 * j * kCellW + 3 * (i >> 1) + (i & 1) * kHalf];
+            const float c[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int b = 0; b < 32; ++b) {
-        const float u = nr2 > 0.0f ? __fdiv_rn(h[b], nr2) : 0.0f;
-        const int q = (int)__fadd_rn(__fmul_rn(u, 512.0f), 0.5f);
-        word[b >> 2] |= (uint32_t)min(q, 255) << (8 * (b & 3));
-    }
-    if (valid) {
-        uint4* out = reinterpret_cast<uint4*>(J.desc + (plane + (size_t)y * J.w + x) * kDesc + 32 * r);
-        out[0] = make_uint4(word[0], word[1], word[2], word[3]);
-        out[1] = make_uint4(word[4], word[5], word[6], word[7]);
+            for (int q = 0; q < 4; ++q) {
+                const float u = fminf(quotient(c[q], d1), 0.2f);
+                ss = __fadd_rn(ss, __fmul_rn(u, u));
+            }
+        }
+    const Divisor d2 = divisor_of(__fsqrt_rn(ss));
+    uint8_t* out = J.desc + (plane + (size_t)y * J.w + x) * kDesc;
+#pragma unroll 1
+    for (int j = 0; j < 4; ++j) {
+        uint32_t word[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float4 v = c0[3 * j * kCellW + 3 * (i >> 1) + (i & 1) * kHalf];
+            const float c[4] = {v.x, v.y, v.z, v.w};
+            uint32_t q8[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                // u 512 is exact, so one fused step rounds like the sum; adding
+                // 2^23 towards zero leaves the truncated integer in the low bits
+                const float u = quotient(fminf(quotient(c[q], d1), 0.2f), d2);
+                q8[q] = __float_as_uint(__fadd_rz(fminf(__fmaf_rn(u, 512.0f, 0.5f), 255.0f), 8388608.0f));
+            }
+            word[i] = __byte_perm(__byte_perm(q8[0], q8[1], 0x0040), __byte_perm(q8[2], q8[3], 0x0040), 0x5410);
+        }
+        // one 32-byte store per cell row: whole sectors
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(out + 32 * j), "r"(word[0]),
+                     "r"(word[1]), "r"(word[2]), "r"(word[3]), "r"(word[4]), "r"(word[5]), "r"(word[6]), "r"(word[7])
+                     : "memory");
     }
 }
 
@@ -410,16 +456,14 @@ __global__ void __launch_bounds__(128) k_sift_project(SiftJob J) {
 }
 
 struct SiftLayout {
-    size_t grey, mag, bin, desc, s1, s2, axes, proj, total;
+    size_t grey, desc, s1, s2, axes, proj, total;
 };
 
 SiftLayout sift_layout(int w, int h) {
     const size_t np = (size_t)w * h;
     SiftLayout L;
     L.grey = 0;
-    L.mag = L.grey + align256(4 * np);
-    L.bin = L.mag + align256(4 * np * sizeof(float));
-    L.desc = L.bin + align256(4 * np);
+    L.desc = L.grey + align256(4 * np);
     L.s1 = L.desc + align256(4 * np * kDesc);
     L.s2 = L.s1 + align256(kDesc * 8);
     L.axes = L.s2 + align256(kDesc * kDesc * 8);
@@ -456,8 +500,6 @@ extern "C" int sff_sift_features(const uint8_t* const* rgb_dev4, int32_t pitch_b
     J.w = width;
     J.h = height;
     J.grey = reinterpret_cast<uint8_t*>(ws + L.grey);
-    J.mag = reinterpret_cast<float*>(ws + L.mag);
-    J.bin = reinterpret_cast<uint8_t*>(ws + L.bin);
     J.desc = reinterpret_cast<uint8_t*>(ws + L.desc);
     J.s1 = reinterpret_cast<unsigned long long*>(ws + L.s1);
     J.s2 = reinterpret_cast<unsigned long long*>(ws + L.s2);
@@ -465,13 +507,13 @@ extern "C" int sff_sift_features(const uint8_t* const* rgb_dev4, int32_t pitch_b
     J.proj = reinterpret_cast<float*>(ws + L.proj);
     cudaStream_t st = (cudaStream_t)stream;
     const dim3 g((width + 127) / 128, height, 4);
-    const dim3 gd((width + kDescThreads / 4 - 1) / (kDescThreads / 4), height, 4);
     for (int s = 0; s < params->num_scales; ++s) {
         J.s = s;
         J.n = 1 << s;
         SFF_LAUNCH(k_sift_grey, g, 128, 0, st, J);
-        SFF_LAUNCH(k_sift_grad, g, 128, 0, st, J);
-        SFF_LAUNCH(k_sift_desc, gd, kDescThreads, 0, st, J);
+        // the n residues of a tile column (row) side by side: their pixels share sectors
+        const auto tiles = [&](int len, int tile) { return (unsigned)(J.n * ((len + J.n * tile - 1) / (J.n * tile))); };
+        SFF_LAUNCH(k_sift_desc, dim3(tiles(width, kTileW), tiles(height, kTileH), 4), kTileW * kTileH, 0, st, J);
         if (s == 0) {  // the principal axes of the full-resolution descriptors
             if (cudaMemsetAsync(J.s1, 0, L.axes - L.s1, st) != cudaSuccess) return SFF_ERR_CUDA;
             const size_t count = 4 * (size_t)width * height;

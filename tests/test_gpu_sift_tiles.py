@@ -1,0 +1,36 @@
+"""SIFT-PCA features at the edges of the descriptor tiles (32 x 16 pixels of
+one residue class mod the stride): sizes one below, at and one above a whole
+number of tiles at strides 1 and 8, and images smaller than a stride's tile.
+Bit-exact against the oracle, which follows the same operation order."""
+import os
+
+import numpy as np
+import pytest
+
+import scenegen
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("w,h", [(8, 8), (9, 15), (31, 16), (32, 17), (33, 33), (257, 129), (255, 127), (300, 50)])
+def test_phi_at_tile_edges(w, h):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import oracle
+    import paper_1710_10096_gb300 as sff
+    sff.build()
+    oracle.build()
+    oracle.set_threads(os.cpu_count() or 1)
+    images = scenegen.random_images(w, h, seed=w + 1000 * h, n=4)
+    images[1][:] = 77  # no gradient: all-zero descriptors
+    images[2][:, : w // 2] = images[2][:1, :1]  # flat beside noise
+    p = sff.default_params(num_scales=4)
+    dev = [torch.as_tensor(np.ascontiguousarray(im)).cuda() for im in images]
+    phis = [torch.full((4, h, w, 4), float("nan"), dtype=torch.float32, device="cuda") for _ in range(4)]
+    ws = torch.empty(sff.sift_workspace_bytes(w, h), dtype=torch.uint8, device="cuda")
+    sff.sift_features(dev, phis, ws, p)
+    torch.cuda.synchronize()
+    want, _, _ = oracle.sift_phi(images, num_scales=4)
+    for got, o in zip(phis, want):
+        assert np.array_equal(got.cpu().numpy(), o)
