@@ -280,6 +280,7 @@ void profile_mark(const char* name, cudaStream_t st, bool after, int launches = 
 int match_status_read(cudaStream_t st, unsigned* out, bool reset);
 int seeds_status_read(cudaStream_t st, unsigned* out, bool reset);
 int features_status_read(cudaStream_t st, unsigned* out, bool reset);
+int sift_status_read(cudaStream_t st, unsigned* out, bool reset);
 
 int check_size(int w, int h);
 int check_params(const sff_params* p);

@@ -30,15 +30,17 @@
 // k_sift_grey:    smoothed grey image of one scale (4 images, blockIdx.z).
 // k_sift_desc:    gradients, cell sums and quantised descriptors of a tile of
 //                 pixels, one thread per pixel.
-// k_sift_cov:     64 descriptors per step in shared memory, transposed;
-//                 every thread accumulates 64 of the 128 x 128 products with
-//                 dp4a, flushed into 64-bit sums.
+// k_sift_cov:     sums and sums of products of the descriptors on the tensor
+//                 cores, exact, into 64-bit integers.
 // k_sift_axes:    one cluster of four CTAs: mean, covariance, power
 //                 iterations, projection weights.
 // k_sift_project: phi of every pixel of one scale of the four images.
 #include <algorithm>
 
+#include <cuda_fp16.h>
+
 #include "sff_internal.cuh"
+#include "sff_tc.cuh"
 
 namespace sff {
 namespace {
@@ -49,9 +51,6 @@ constexpr int kDesc = 128;
 constexpr int kTileW = 32, kTileH = 16;
 constexpr int kSampW = kTileW + 11, kSampH = kTileH + 11;
 constexpr int kCellW = kTileW + 9, kCellH = kTileH + 9;
-constexpr int kCovPix = 64;       // descriptors per step of k_sift_cov
-constexpr int kCovThreads = 256;
-constexpr int kCovFlush = 16384;  // descriptors between flushes of the 32-bit partial sums
 constexpr int kPowerIters = 200;
 
 struct SiftJob {
@@ -60,7 +59,7 @@ struct SiftJob {
     uint8_t* grey;           // [4][H][W]
     uint8_t* desc;           // [4][H][W][128]
     unsigned long long* s1;  // [128] sums
-    unsigned long long* s2;  // [128][128] sums of products
+    unsigned long long* s2;  // [128][128] sums of products of (component - 128), entries j >= i
     double* axes;            // [3][128]
     float* proj;             // [3][128] single-precision axes, then [3] biases
     float* phi[4];           // [S][H][W][4] each
@@ -242,54 +241,197 @@ __global__ void __launch_bounds__(kTileW * kTileH, 3) k_sift_desc(SiftJob J) {
 }
 
 // Sums of the descriptors and of their pairwise products over the four
-// images' full-resolution descriptors.
-__global__ void __launch_bounds__(kCovThreads) k_sift_cov(SiftJob J, size_t count) {
-    __shared__ uint32_t tile[kDesc][kCovPix / 4];  // [component][4 descriptors]
-    const int t = threadIdx.x;
-    uint32_t acc[kDesc * kDesc / kCovThreads];
-    uint32_t s1 = 0;
+// images' full-resolution descriptors: one matrix product S2 = Q Q^T on the
+// tensor cores, Q = the 128 x count matrix of the descriptors less 128, in
+// fp16 (integers -128..127, exact).  A product is at most 2^14 in magnitude, so
+// the fp32 sums of kCovGroup = 1024 descriptors are exact in any order; then
+// they are added to 32-bit integers in registers and, before those can
+// overflow, to the 64-bit sums in memory.  Both operands are the same tile: a
+// descriptor's 8 consecutive components are 16 bytes of an MN-major core
+// matrix, so the conversion needs no transposition.  One CTA per SM; each step
+// converts kCovStep descriptors that were loaded two steps earlier, one thread
+// issues the MMAs, and the next steps fill other stages meanwhile.  Bound by the
+// descriptor reads.  1242 x 375 (1.86 M descriptors): 1419 us (dp4a over a
+// shared-memory transpose) -> 159 us.
+constexpr int kCovStep = 128;                   // descriptors per step (K)
+constexpr int kCovStages = 3;                   // steps in shared memory
+constexpr int kCovGroup = 1024;                 // descriptors per exact fp32 sum
+constexpr int kCovSteps = kCovGroup / kCovStep;
+constexpr int kCovMaxGroups = 120;              // groups per 32-bit sum: 120 * 2^24 < 2^31
+constexpr int kCovThreads = 512;
+constexpr int kCovCtas = 152;                   // one per SM
+constexpr int kCovStageBytes = kCovStep * kDesc * 2;
+constexpr int kCovKGroup = kDesc * 16;          // bytes between K groups of 8 descriptors
+constexpr int kCovSmemBytes = kCovStages * kCovStageBytes + 1024;  // + alignment slack
+// instruction descriptor, kind::f16: fp32 D (bits 4-5 = 1), fp16 A and B (bits
+// 7-12 = 0), both MN-major (bits 15, 16), N = M = 128
+constexpr uint32_t kCovIdesc =
+    (1u << 4) | (1u << 15) | (1u << 16) | ((uint32_t)(kDesc >> 3) << 17) | ((uint32_t)(kDesc >> 4) << 24);
+
+__device__ unsigned int g_sift_status;  // bit 0: a bounded wait of k_sift_cov gave up; bit 1: its drain did
+
+// 4 components as two fp16 pairs, each less 128 (1024 + b as a bit pattern,
+// then an exact subtraction).
+__device__ __forceinline__ uint2 centred_halves(uint32_t w) {
+    const __half2 off = __halves2half2(__ushort_as_half(0x6480), __ushort_as_half(0x6480));  // 1152
+    const uint32_t lo = __byte_perm(w, 0x64646464u, 0x4140), hi = __byte_perm(w, 0x64646464u, 0x4342);
+    const __half2 a = __hsub2(*reinterpret_cast<const __half2*>(&lo), off);
+    const __half2 b = __hsub2(*reinterpret_cast<const __half2*>(&hi), off);
+    return make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+}
+
+__global__ void __launch_bounds__(kCovThreads, 1) k_sift_cov(SiftJob J, size_t count) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ uint64_t bar[kCovStages];
+    __shared__ uint32_t tmem_slot;
+    __shared__ uint32_t s1[kDesc];
+    uint8_t* sm = smem_raw + ((1024 - (smem_addr(smem_raw) & 1023)) & 1023);
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    if (t == 0) {
+        for (int k = 0; k < kCovStages; ++k) mbar_init(&bar[k], 1);
+        mbar_fence_init();
+    }
+    if (t < kDesc) s1[t] = 0;
+    if (warp == 0) tmem_alloc(&tmem_slot, kDesc);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_slot;
+
+    const size_t steps_all = (count + kCovStep - 1) / kCovStep;
+    const int steps = (int)((steps_all - blockIdx.x + gridDim.x - 1) / gridDim.x);  // grid <= steps_all
+    // this thread's part of a step: descriptor 8 warp + lane % 8 (its K group
+    // is the warp's), components 16 c .. 16 c + 15 for c = lane / 8 and c + 4; a
+    // quarter warp then writes 128 contiguous bytes
+    const int kd = 8 * warp + (lane & 7), c0 = lane >> 3;
+    auto load = [&](int u, uint4 (&v)[2]) {
+        const size_t d = ((size_t)blockIdx.x + (size_t)u * gridDim.x) * kCovStep + kd;
+        const uint4* src = reinterpret_cast<const uint4*>(J.desc + d * kDesc);
+        const bool in = u < steps && d < count;
 #pragma unroll
-    for (int e = 0; e < kDesc * kDesc / kCovThreads; ++e) acc[e] = 0;
-    size_t since = 0;
-    auto flush = [&]() {
+        for (int r = 0; r < 2; ++r)  // past the end: 128 = a centred 0
+            v[r] = in ? __ldg(src + c0 + 4 * r) : make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
+        return in;
+    };
+    int acc[32];  // component i = 32 (warp % 4) + lane against components 32 (warp / 4) ..
 #pragma unroll
-        for (int e = 0; e < kDesc * kDesc / kCovThreads; ++e) {
-            if (acc[e]) atomicAdd(J.s2 + t + e * kCovThreads, (unsigned long long)acc[e]);
+    for (int e = 0; e < 32; ++e) acc[e] = 0;
+    uint32_t part[2][8];  // 16-bit sums of this thread's components: even, odd bytes of each word
+#pragma unroll
+    for (int e = 0; e < 16; ++e) part[e >> 3][e & 7] = 0;
+    auto flush = [&]() {  // the CTA's sums to memory
+        const int i = 32 * (warp & 3) + lane;
+#pragma unroll
+        for (int e = 0; e < 32; ++e) {
+            const int j = 32 * (warp >> 2) + e;
+            if (j >= i) atomicAdd(J.s2 + i * kDesc + j, (unsigned long long)(long long)acc[e]);
             acc[e] = 0;
         }
-        if (t < kDesc && s1) atomicAdd(J.s1 + t, (unsigned long long)s1);
-        s1 = 0;
+        __syncthreads();
+        if (t < kDesc) {
+            atomicAdd(J.s1 + t, (unsigned long long)s1[t]);
+            s1[t] = 0;
+        }
+        __syncthreads();
     };
-    for (size_t base = (size_t)blockIdx.x * kCovPix; base < count; base += (size_t)gridDim.x * kCovPix) {
-        __syncthreads();
-        // transpose 64 descriptors into [component][descriptor] bytes
-        for (int k = t; k < kCovPix * kDesc / 4; k += kCovThreads) {
-            const int p = k / (kDesc / 4), w4 = k % (kDesc / 4);
-            uint32_t word = 0;
-            if (base + p < count) word = reinterpret_cast<const uint32_t*>(J.desc + (base + p) * kDesc)[w4];
+
+    uint4 cur[2], nxt[2];
+    bool cur_in = load(0, cur), nxt_in = load(1, nxt);
+    bool ok = true, failed = false;
+    int issued = 0, groups = 0;
+    for (int u = 0; u < steps; ++u) {
+        const int s = u % kCovStages;
+        if (u >= kCovStages) ok = ok && mbar_wait(&bar[s], (unsigned)(u / kCovStages - 1) & 1u, kDefaultWaitNs);
+        uint8_t* stage = sm + s * kCovStageBytes + warp * kCovKGroup + (lane & 7) * 16;
 #pragma unroll
-            for (int b = 0; b < 4; ++b)
-                reinterpret_cast<uint8_t*>(&tile[w4 * 4 + b][p / 4])[p % 4] = (uint8_t)(word >> (8 * b));
+        for (int r = 0; r < 2; ++r) {
+            const uint32_t w[4] = {cur[r].x, cur[r].y, cur[r].z, cur[r].w};
+            uint2 h[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                h[e] = centred_halves(w[e]);
+                if (cur_in) {
+                    part[r][2 * e] += w[e] & 0x00ff00ffu;
+                    part[r][2 * e + 1] += (w[e] >> 8) & 0x00ff00ffu;
+                }
+            }
+            // component groups 2 c and 2 c + 1 of 8
+            uint4* dst = reinterpret_cast<uint4*>(stage + 256 * (c0 + 4 * r));
+            dst[0] = make_uint4(h[0].x, h[0].y, h[1].x, h[1].y);
+            dst[8] = make_uint4(h[2].x, h[2].y, h[3].x, h[3].y);
         }
-        __syncthreads();
 #pragma unroll
-        for (int e = 0; e < kDesc * kDesc / kCovThreads; ++e) {
-            const int idx = t + e * kCovThreads, i = idx / kDesc, j = idx % kDesc;
-            uint32_t a = acc[e];
-#pragma unroll
-            for (int p4 = 0; p4 < kCovPix / 4; ++p4) a = __dp4a(tile[i][p4], tile[j][p4], a);
-            acc[e] = a;
+        for (int r = 0; r < 2; ++r) cur[r] = nxt[r];
+        cur_in = nxt_in;
+        nxt_in = load(u + 2, nxt);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the stage visible to the tensor cores
+        tc_fence_before();
+        if (!__syncthreads_and(ok)) {
+            failed = true;
+            break;
         }
-        if (t < kDesc)
+        tc_fence_after();
+        if (t == 0) {
+            const uint32_t base = smem_addr(sm + s * kCovStageBytes);
 #pragma unroll
-            for (int p4 = 0; p4 < kCovPix / 4; ++p4) s1 = __dp4a(tile[t][p4], 0x01010101u, s1);
-        since += kCovPix;
-        if (since >= kCovFlush) {
-            flush();
-            since = 0;
+            for (int k = 0; k < kCovStep / 16; ++k) {
+                const uint64_t d = smem_desc(base + 2 * k * kCovKGroup, kCovKGroup, 128);
+                tc_mma(tmem, d, d, kCovIdesc, u % kCovSteps != 0 || k > 0);
+            }
+            tc_commit(&bar[s]);
+        }
+        issued = u + 1;
+        if (u % kCovSteps == kCovSteps - 1 || u == steps - 1) {
+            // the group's sums out of tensor memory before the next MMA, which
+            // follows the next barrier, starts them anew
+            ok = __all_sync(0xffffffffu, mbar_wait(&bar[s], (unsigned)(u / kCovStages) & 1u, kDefaultWaitNs));
+            if (ok) {
+                tc_fence_after();
+                uint32_t v[32];
+                tmem_ld32(tmem + ((uint32_t)(32 * (warp & 3)) << 16), v, 32 * (warp >> 2));
+                tmem_ld_wait(v);
+                tc_fence_before();
+#pragma unroll
+                for (int e = 0; e < 32; ++e) acc[e] += __float2int_rn(__uint_as_float(v[e]));
+            }
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    uint32_t* dst = s1 + 16 * (c0 + 4 * r) + 4 * (e >> 1) + (e & 1);
+                    atomicAdd(dst, part[r][e] & 0xffffu);
+                    atomicAdd(dst + 2, part[r][e] >> 16);
+                    part[r][e] = 0;
+                }
+            if (++groups == kCovMaxGroups) {
+                flush();
+                groups = 0;
+            }
         }
     }
-    flush();
+    if (!failed && !__syncthreads_and(ok)) failed = true;
+    if (failed) {
+        // status, and the MMAs in flight complete before the tensor memory is released
+        if (t == 0) {
+            atomicOr(&g_sift_status, 1u);
+            if (issued > 0 && !mbar_wait(&bar[(issued - 1) % kCovStages], (unsigned)((issued - 1) / kCovStages) & 1u,
+                                         kDrainFactor * kDefaultWaitNs))
+                atomicOr(&g_sift_status, 2u);
+        }
+    } else {
+        flush();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 0) tmem_dealloc(tmem, kDesc);
+}
+
+// Sum of the products of components i and j over the count descriptors, from
+// the sums of the centred ones: (a - 128)(b - 128) = a b - 128 (a + b) + 128^2.
+__device__ __forceinline__ double product_sum(const SiftJob& J, int i, int j, double count) {
+    const long long c = (long long)J.s2[i < j ? i * kDesc + j : j * kDesc + i];
+    return (double)(c + 128ll * (long long)(J.s1[i] + J.s1[j]) - 16384ll * (long long)count);
 }
 
 // The principal axes, by one cluster of kAxesCtas CTAs.  The FP64 pipe bounds
@@ -405,7 +547,7 @@ __global__ void __cluster_dims__(kAxesCtas, 1, 1) __launch_bounds__(kDesc) k_sif
     double cov[kChain], axr[2][kChain];
 #pragma unroll
     for (int k = 0; k < kChain; ++k)
-        cov[k] = __dsub_rn(__ddiv_rn((double)J.s2[row * kDesc + 4 * k + r], count),
+        cov[k] = __dsub_rn(__ddiv_rn(product_sum(J, row, 4 * k + r, count), count),
                            __dmul_rn(mean[row], mean[4 * k + r]));
     cluster_barrier();  // every CTA of the cluster runs before the first remote store
     power_axis<0>(cov, axr, ax, v, raw, upd);
@@ -473,6 +615,19 @@ SiftLayout sift_layout(int w, int h) {
 }
 
 }  // namespace
+
+// Reads (and with reset clears) the condition bits of the SIFT kernels, in
+// stream order; the caller synchronises the stream.
+int sift_status_read(cudaStream_t st, unsigned* out, bool reset) {
+    static const unsigned zero = 0;
+    if (cudaMemcpyFromSymbolAsync(out, g_sift_status, sizeof(unsigned), 0, cudaMemcpyDeviceToHost, st) != cudaSuccess)
+        return SFF_ERR_CUDA;
+    if (reset && cudaMemcpyToSymbolAsync(g_sift_status, &zero, sizeof(unsigned), 0, cudaMemcpyHostToDevice, st) !=
+                     cudaSuccess)
+        return SFF_ERR_CUDA;
+    return SFF_OK;
+}
+
 }  // namespace sff
 
 extern "C" size_t sff_sift_workspace_bytes(int32_t width, int32_t height) {
@@ -507,6 +662,9 @@ extern "C" int sff_sift_features(const uint8_t* const* rgb_dev4, int32_t pitch_b
     J.proj = reinterpret_cast<float*>(ws + L.proj);
     cudaStream_t st = (cudaStream_t)stream;
     const dim3 g((width + 127) / 128, height, 4);
+    // the attribute is per device: set it on the current one at every call
+    if (cudaFuncSetAttribute(k_sift_cov, cudaFuncAttributeMaxDynamicSharedMemorySize, kCovSmemBytes) != cudaSuccess)
+        return SFF_ERR_CUDA;
     for (int s = 0; s < params->num_scales; ++s) {
         J.s = s;
         J.n = 1 << s;
@@ -517,8 +675,8 @@ extern "C" int sff_sift_features(const uint8_t* const* rgb_dev4, int32_t pitch_b
         if (s == 0) {  // the principal axes of the full-resolution descriptors
             if (cudaMemsetAsync(J.s1, 0, L.axes - L.s1, st) != cudaSuccess) return SFF_ERR_CUDA;
             const size_t count = 4 * (size_t)width * height;
-            const int blocks = (int)std::min<size_t>((count + kCovPix - 1) / kCovPix, 152 * 4);
-            SFF_LAUNCH(k_sift_cov, dim3(blocks), kCovThreads, 0, st, J, count);
+            const int blocks = (int)std::min<size_t>((count + kCovStep - 1) / kCovStep, kCovCtas);
+            SFF_LAUNCH(k_sift_cov, dim3(blocks), kCovThreads, kCovSmemBytes, st, J, count);
             SFF_LAUNCH(k_sift_axes, dim3(kAxesCtas), kDesc, 0, st, J, (double)count);
         }
         SFF_LAUNCH(k_sift_project, g, 128, 0, st, J);

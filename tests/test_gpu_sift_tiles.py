@@ -34,3 +34,28 @@ def test_phi_at_tile_edges(w, h):
     want, _, _ = oracle.sift_phi(images, num_scales=4)
     for got, o in zip(phis, want):
         assert np.array_equal(got.cpu().numpy(), o)
+
+
+@pytest.mark.parametrize("w,h", [(1416, 904), (500, 37)])
+def test_axes_of_many_descriptors(w, h):
+    """The covariance's sums over more descriptors than one 32-bit partial
+    sum takes (1416 x 904), and over a count that is no multiple of a step."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import oracle
+    import paper_1710_10096_gb300 as sff
+    sff.build()
+    oracle.build()
+    oracle.set_threads(os.cpu_count() or 1)
+    images = scenegen.random_images(w, h, seed=w, n=4)
+    images[3] //= 8
+    p = sff.default_params(num_scales=1)
+    dev = [torch.as_tensor(np.ascontiguousarray(im)).cuda() for im in images]
+    phis = [torch.empty((1, h, w, 4), dtype=torch.float32, device="cuda") for _ in range(4)]
+    ws = torch.empty(sff.sift_workspace_bytes(w, h), dtype=torch.uint8, device="cuda")
+    sff.sift_features(dev, phis, ws, p)
+    assert sff.device_status() == sff.OK
+    want, _, _ = oracle.sift_phi(images, num_scales=1)
+    for got, o in zip(phis, want):
+        assert np.array_equal(got.cpu().numpy(), o)
