@@ -571,30 +571,62 @@ __global__ void __cluster_dims__(kAxesCtas, 1, 1) __launch_bounds__(kDesc) k_sif
     }
 }
 
-__global__ void __launch_bounds__(128) k_sift_project(SiftJob J) {
-    __shared__ float a[3 * kDesc + 3];
-    for (int k = threadIdx.x; k < 3 * kDesc + 3; k += blockDim.x) a[k] = J.proj[k];
+// phi of one scale, two pixels per thread, so that a weight is read from shared
+// memory once for both.  The descriptors come through shared memory by coalesced
+// asynchronous copies (a thread's own 128 bytes are four lines away from its
+// neighbour's; rows padded by 16 bytes, conflict-free).  A byte becomes a float as the low bits of 2^23 (one
+// byte permute), less 2^23: the conversion instruction runs at an eighth of
+// the FP32 rate.  Bound by the FP32 pipe (7 operations per component and
+// pixel; packed pairs issue half as often but pass at the same rate, and the
+// assembler contracts their products and sums).  1242 x 375, four images:
+// 105 us a scale (one pixel per thread, conversions) -> 84 us.
+constexpr int kProjThreads = 128;
+
+__global__ void __launch_bounds__(kProjThreads) k_sift_project(SiftJob J) {
+    __shared__ float4 a[kDesc];  // the three weights of a component
+    __shared__ uint4 row[2 * kProjThreads][kDesc / 16 + 1];
+    const int v = blockIdx.y;
+    const size_t np = (size_t)J.w * J.h;
+    const size_t first = (size_t)blockIdx.x * (2 * kProjThreads);
+    const uint4* desc = reinterpret_cast<const uint4*>(J.desc + ((size_t)v * np + first) * kDesc);
+    const int chunks = (int)min((size_t)(2 * kProjThreads), np - first) * (kDesc / 16);
+    for (int e = threadIdx.x; e < chunks; e += kProjThreads)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(
+                         (unsigned)__cvta_generic_to_shared(&row[e / (kDesc / 16)][e % (kDesc / 16)])),
+                     "l"(desc + e)
+                     : "memory");
+    for (int k = threadIdx.x; k < kDesc; k += kProjThreads)
+        a[k] = make_float4(J.proj[k], J.proj[kDesc + k], J.proj[2 * kDesc + k], 0.0f);
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y, v = blockIdx.z;
-    if (x >= J.w) return;
-    const size_t p = (size_t)y * J.w + x;
-    const uint4* q = reinterpret_cast<const uint4*>(J.desc + ((size_t)v * J.h * J.w + p) * kDesc);
-    float t[3] = {0.0f, 0.0f, 0.0f};
+    const size_t p0 = first + threadIdx.x, p1 = p0 + kProjThreads;
+    if (p0 >= np) return;
+    const uint4 *q0 = row[threadIdx.x], *q1 = row[p1 < np ? threadIdx.x + kProjThreads : threadIdx.x];
+    float t[2][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
+#pragma unroll 2
     for (int k16 = 0; k16 < kDesc / 16; ++k16) {  // 16 components per load, in index order
-        const uint4 w = q[k16];
-        const uint32_t words[4] = {w.x, w.y, w.z, w.w};
+        const uint4 w0 = q0[k16], w1 = q1[k16];
+        const uint32_t u[2][4] = {{w0.x, w0.y, w0.z, w0.w}, {w1.x, w1.y, w1.z, w1.w}};
 #pragma unroll
         for (int b = 0; b < 16; ++b) {
-            const float qv = (float)((words[b >> 2] >> (8 * (b & 3))) & 0xffu);
-            const int k = k16 * 16 + b;
+            const float4 w = a[k16 * 16 + b];
 #pragma unroll
-            for (int c = 0; c < 3; ++c) t[c] = __fadd_rn(t[c], __fmul_rn(a[c * kDesc + k], qv));
+            for (int i = 0; i < 2; ++i) {
+                const float q =
+                    __fsub_rn(__uint_as_float(__byte_perm(u[i][b >> 2], 0x4b000000u, 0x7650u + (b & 3))), 8388608.0f);
+                t[i][0] = __fadd_rn(t[i][0], __fmul_rn(w.x, q));
+                t[i][1] = __fadd_rn(t[i][1], __fmul_rn(w.y, q));
+                t[i][2] = __fadd_rn(t[i][2], __fmul_rn(w.z, q));
+            }
         }
     }
-    float r[3];
+    float4* phi = reinterpret_cast<float4*>(phi_of(J, v)) + (size_t)J.s * np;
+    const float b0 = J.proj[3 * kDesc], b1 = J.proj[3 * kDesc + 1], b2 = J.proj[3 * kDesc + 2];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) r[c] = __fsub_rn(t[c], a[3 * kDesc + c]);
-    reinterpret_cast<float4*>(phi_of(J, v))[(size_t)J.s * J.w * J.h + p] = make_float4(r[0], r[1], r[2], 0.0f);
+    for (int i = 0; i < 2; ++i)
+        if (i == 0 || p1 < np)
+            phi[i ? p1 : p0] =
+                make_float4(__fsub_rn(t[i][0], b0), __fsub_rn(t[i][1], b1), __fsub_rn(t[i][2], b2), 0.0f);
 }
 
 struct SiftLayout {
@@ -662,6 +694,7 @@ extern "C" int sff_sift_features(const uint8_t* const* rgb_dev4, int32_t pitch_b
     J.proj = reinterpret_cast<float*>(ws + L.proj);
     cudaStream_t st = (cudaStream_t)stream;
     const dim3 g((width + 127) / 128, height, 4);
+    const dim3 gp((unsigned)(((size_t)width * height + 2 * kProjThreads - 1) / (2 * kProjThreads)), 4);
     // the attribute is per device: set it on the current one at every call
     if (cudaFuncSetAttribute(k_sift_cov, cudaFuncAttributeMaxDynamicSharedMemorySize, kCovSmemBytes) != cudaSuccess)
         return SFF_ERR_CUDA;
@@ -679,7 +712,7 @@ extern "C" int sff_sift_features(const uint8_t* const* rgb_dev4, int32_t pitch_b
             SFF_LAUNCH(k_sift_cov, dim3(blocks), kCovThreads, kCovSmemBytes, st, J, count);
             SFF_LAUNCH(k_sift_axes, dim3(kAxesCtas), kDesc, 0, st, J, (double)count);
         }
-        SFF_LAUNCH(k_sift_project, g, 128, 0, st, J);
+        SFF_LAUNCH(k_sift_project, gp, kProjThreads, 0, st, J);
     }
     return launch_status();
 }
