@@ -59,3 +59,40 @@ def test_axes_of_many_descriptors(w, h):
     want, _, _ = oracle.sift_phi(images, num_scales=1)
     for got, o in zip(phis, want):
         assert np.array_equal(got.cpu().numpy(), o)
+
+
+def test_scratch_of_one_scale_gives_the_same_phi():
+    """The order of the scales does not depend on the results: scratch for one
+    scale's descriptors (what larger images get) and for all of them, on a side
+    stream and inside a captured graph."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1710_10096_gb300 as sff
+    sff.build()
+    w, h = 161, 83
+    p = sff.default_params()
+    dev = [torch.as_tensor(im).cuda() for im in scenegen.make_quad("planes", w, h, 5).images()]
+    full = sff.sift_workspace_bytes(w, h)
+    small = full - 3 * 4 * w * h * 128
+    outs = []
+    for nbytes in (full, small + 4096):
+        phis = [torch.full((4, h, w, 4), float("nan"), device="cuda") for _ in range(4)]
+        ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            sff.sift_features(dev, phis, ws, p, stream=s)
+            s.synchronize()
+            outs.append([t.clone() for t in phis])
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=s):
+                sff.sift_features(dev, phis, ws, p, stream=torch.cuda.current_stream())
+            for t in phis:
+                t.zero_()
+            g.replay()
+        s.synchronize()
+        outs.append([t.clone() for t in phis])
+    for o in outs[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(outs[0], o))
+    with pytest.raises(sff.SffError):
+        sff.sift_features(dev, phis, torch.empty(small - 4096, dtype=torch.uint8, device="cuda"), p)
