@@ -42,6 +42,7 @@
 #include <algorithm>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include <cuda.h>  // CUtensorMap and its encoder's signature (resolved at run time)
 
@@ -1728,32 +1729,141 @@ __global__ void __launch_bounds__(256) k_random_search(const __grid_constant__ F
 // itself.  The initialisation's nearest neighbours are still those of the WHT
 // features (Sec. 3.1 "Initialization"); its combinations are scored with
 // this cost.
+//
+// The phi of the four views at the scale being matched, each row in residue
+// classes of the column mod n (repacked by k_sift_pack; at n = 1 the caller's
+// arrays as they are): column x at (x mod n) m + x / n.  The 7 columns of a
+// window row are then 112 contiguous bytes, one or two lines; in the caller's
+// order they lie in up to 7.  (Planes of 8 and 4 bytes in classes mod 2 n, made for
+// one candidate per lane, take 4 lines a row here: 9.4 against 8.9 ms for both
+// fields of a 1242 x 375 quad.)
 struct SiftViews {
-    const float4 *ref, *tmp, *ste, *crs;  // phi of the scale, [y][x]
+    const float4* v[4];  // reference, temporal, stereo, cross
     int w, h, n, sigma;
+    int m;      // columns per residue class
+    int pitch;  // n m: elements per row
+};
+struct SiftPhi {
+    const float4* v[4];
+    float4* packed;  // 4 x [h][pitch]
 };
 
-__device__ __forceinline__ float sift_dist(float4 a, float4 b) {
-    const float dx = __fsub_rn(a.x, b.x), dy = __fsub_rn(a.y, b.y), dz = __fsub_rn(a.z, b.z);
-    return __fsqrt_rn(__fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz)));
+template <int N>
+__device__ __forceinline__ int sift_slot(int x, int m) {
+    return (x & (N - 1)) * m + x / N;
 }
 
-__device__ int sift_cost(const SiftViews& S, int px, int py, const Vec4& a) {
+template <int N>
+__global__ void k_sift_pack(SiftPhi P, SiftViews S) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y, k = blockIdx.z;
+    const int x = e % S.m * N + e / S.m;
+    if (e >= S.pitch || x >= S.w) return;
+    P.packed[((size_t)k * S.h + y) * S.pitch + e] = __ldg(P.v[k] + (size_t)y * S.w + x);
+}
+
+__device__ __forceinline__ float sift_dist2(float4 a, float4 b) {
+    const float dx = __fsub_rn(a.x, b.x), dy = __fsub_rn(a.y, b.y), dz = __fsub_rn(a.z, b.z);
+    return __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
+}
+
+// Square root of x in [2^-96, 2^100], correctly rounded: g = x y with y the
+// approximate reciprocal root, one step by the exact remainder x - g g
+// (Markstein 1990).  Equal to sqrt.rn for every float of the range (all
+// 1.6 billion compared on a GB300).  sqrt.rn passes 5 lanes per clock and SM, the
+// approximation 16, the four others 128.
+constexpr float kRootMin = 0x1p-96f, kRootSumMax = 0x1p48f;
+__device__ __forceinline__ float root_in_range(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    const float g = __fmul_rn(x, y);
+    return __fmaf_rn(__fmaf_rn(-g, g, x), __fmul_rn(0.5f, y), g);
+}
+
+// The sum of Eq. 1 for any values, one thread, by sqrt.rn (0 for 0).
+template <int N>
+__device__ float sift_cost_any(const SiftViews& S, int px, int py, const Vec4& a) {
+    auto get = [&](int k, int x, int y) {
+        return __ldg(S.v[k] + (size_t)clampi(y, 0, S.h - 1) * S.pitch + sift_slot<N>(clampi(x, 0, S.w - 1), S.m));
+    };
+    auto root = [](float d) { return d == 0.0f ? 0.0f : __fsqrt_rn(d); };
     float c = 0.0f;
-    for (int j = -3; j <= 3; ++j) {
-        const int y = py + j * S.n;
-        const size_t ry = (size_t)clampi(y, 0, S.h - 1) * S.w, ty = (size_t)clampi(y + a.v, 0, S.h - 1) * S.w;
-        for (int i = -3; i <= 3; ++i) {
-            const int x = px + i * S.n;
-            const float4 r = __ldg(S.ref + ry + clampi(x, 0, S.w - 1));
-            const float4 t = __ldg(S.tmp + ty + clampi(x + a.u, 0, S.w - 1));
-            const float4 st = __ldg(S.ste + ry + clampi(x - S.sigma * a.d0, 0, S.w - 1));
-            const float4 cr = __ldg(S.crs + ty + clampi(x + a.u - S.sigma * a.d1, 0, S.w - 1));
-            c = __fadd_rn(c, sift_dist(r, t));
-            c = __fadd_rn(c, sift_dist(r, st));
-            c = __fadd_rn(c, sift_dist(r, cr));
+#pragma unroll 1
+    for (int k = 0; k < 49; ++k) {
+        const int x = px + (k % 7 - 3) * N, y = py + (k / 7 - 3) * N;
+        const float4 f = get(0, x, y);
+        c = __fadd_rn(c, root(sift_dist2(f, get(1, x + a.u, y + a.v))));
+        c = __fadd_rn(c, root(sift_dist2(f, get(2, x - S.sigma * a.d0, y))));
+        c = __fadd_rn(c, root(sift_dist2(f, get(3, x + a.u - S.sigma * a.d1, y + a.v))));
+    }
+    return c;
+}
+
+// Eq. 1 of up to 8 candidates by one warp: 8 lanes per candidate, lane q taking
+// column q - 3 of the window (lane 7 repeats column 3), so that all 28 loads of a
+// lane are independent and in flight together: with one thread per candidate a
+// half-step took about 100 us at every scale, each candidate a chain of 49 load
+// latencies.  The 147 distances go to shared memory and one lane per candidate
+// adds them in the definition's order.  at(k, px, py, vec): candidate k < n, the
+// same for the 8 lanes; n is warp-uniform.  Lane k < n returns candidate k's cost
+// as the float's bit pattern.  A candidate with a squared distance below the fast
+// root's range (a zero among them), or a sum that may hold one above it (then it
+// is at least 2^50 or no number), is evaluated again by the general form.
+constexpr int kSiftStride = 148;  // 147 distances, rows of whole 16 bytes
+template <int N, class At>
+__device__ __forceinline__ int sift_costs(const SiftViews& S, float* buf, int lane, int n, At at) {
+    const int g = lane >> 3, q = lane & 7, col = (min(q, 6) - 3) * N;
+    unsigned slow = 0;
+    for (int k0 = 0; k0 < n; k0 += 4) {
+        float lo = 3.0e38f;
+        if (k0 + g < n) {
+            int px, py;
+            Vec4 a;
+            at(k0 + g, px, py, a);
+            const int x = px + col;
+            const int s0 = sift_slot<N>(clampi(x, 0, S.w - 1), S.m), s1 = sift_slot<N>(clampi(x + a.u, 0, S.w - 1), S.m),
+                      s2 = sift_slot<N>(clampi(x - S.sigma * a.d0, 0, S.w - 1), S.m),
+                      s3 = sift_slot<N>(clampi(x + a.u - S.sigma * a.d1, 0, S.w - 1), S.m);
+            float* d = buf + (k0 + g) * kSiftStride + 3 * q;
+#pragma unroll
+            for (int j = 0; j < 7; ++j) {
+                const int y = py + (j - 3) * N;
+                const size_t r = (size_t)clampi(y, 0, S.h - 1) * S.pitch,
+                             t = (size_t)clampi(y + a.v, 0, S.h - 1) * S.pitch;
+                const float4 f = __ldg(S.v[0] + r + s0);
+                const float d0 = sift_dist2(f, __ldg(S.v[1] + t + s1));
+                const float d1 = sift_dist2(f, __ldg(S.v[2] + r + s2));
+                const float d2 = sift_dist2(f, __ldg(S.v[3] + t + s3));
+                lo = fminf(lo, fminf(d0, fminf(d1, d2)));
+                if (q < 7) {
+                    d[21 * j] = root_in_range(d0);
+                    d[21 * j + 1] = root_in_range(d1);
+                    d[21 * j + 2] = root_in_range(d2);
+                }
+            }
+        }
+        const unsigned low = __ballot_sync(0xffffffffu, lo < kRootMin);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) slow |= (unsigned)(((low >> (8 * k)) & 0xffu) != 0) << (k0 + k);
+    }
+    __syncwarp();
+    float c = 0.0f;
+    if (lane < n) {
+        const float4* d = reinterpret_cast<const float4*>(buf + lane * kSiftStride);
+#pragma unroll 6
+        for (int k = 0; k < 36; ++k) {
+            const float4 v = d[k];
+            c = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(c, v.x), v.y), v.z), v.w);
+        }
+        const float4 v = d[36];
+        c = __fadd_rn(__fadd_rn(__fadd_rn(c, v.x), v.y), v.z);
+        if (((slow >> lane) & 1u) || !(c < kRootSumMax)) {
+            int px, py;
+            Vec4 a;
+            at(lane, px, py, a);
+            c = sift_cost_any<N>(S, px, py, a);
         }
     }
+    __syncwarp();
     return __float_as_int(c);
 }
 
@@ -1811,11 +1921,15 @@ __device__ int warp_row_topk(const RefFeat& r, const int4* rec, const int* rec_n
     return cnt;
 }
 
-// One warp per coarsest-grid query: all K_T x K_E x K_E combinations, each
-// scored by one lane; the first minimum in (temporal, stereo, cross) rank
+// One warp per coarsest-grid query: all K_T x K_E x K_E combinations, eight
+// at a time (sift_costs); the first minimum in (temporal, stereo, cross) rank
 // order wins, as in a sequential loop with a strict comparison.
-__global__ void k_sift_init(const __grid_constant__ Fields F, SiftViews S, int n, int knn_t, int knn_e, uint2* field,
+template <int N>
+__global__ void k_sift_init(const __grid_constant__ Fields F, SiftViews S, int knn_t, int knn_e, uint2* field,
                             int* cost) {
+    constexpr int n = N;
+    __shared__ __align__(16) float s_dist[8][8 * kSiftStride];
+    float* buf = s_dist[threadIdx.x >> 5];
     const Field& A = F.f[0];
     const Views& V = A.V;
     const int gw = A.gw;
@@ -1836,46 +1950,30 @@ __global__ void k_sift_init(const __grid_constant__ Fields F, SiftViews S, int n
         const int tx = (e.y % gw) * n, ty = (e.y / gw) * n;
         const int nx = warp_row_topk(r, A.rec + (size_t)A.gq * 3, A.rec_n + A.gq, n, gw, e.y / gw, tx, V.sigma, lane,
                                      knn_e, xd, xx);
-        // lane l scores combination (l / nx, l % nx)
-        unsigned long long key = ~0ull;
-        Vec4 cand = {tx - px, ty - py, 0, 0};
-        for (int l0 = 0; l0 < ns * nx; l0 += 32) {
-            const int l = l0 + lane;
-            if (l < ns * nx) {
-                int sxl = sx[0], cxl = xx[0];
+        // combination l: (l / nx, l % nx)
+        auto combination = [&](int l) {
+            int sxl = sx[0], cxl = xx[0];
 #pragma unroll
-                for (int t = 0; t < SFF_MAX_KNN; ++t) {
-                    if (t == l / nx) sxl = sx[t];
-                    if (t == l % nx) cxl = xx[t];
-                }
-                Vec4 u = {tx - px, ty - py, V.sigma * (px - sxl), V.sigma * (tx - cxl)};
-                u.u = (int16_t)u.u;
-                u.v = (int16_t)u.v;
-                u.d0 = (int16_t)u.d0;
-                u.d1 = (int16_t)u.d1;
-                const int c = sift_cost(S, px, py, u);
-                const unsigned long long kk = ((unsigned long long)(unsigned)c << 32) | (unsigned)l;
-                if (kk < key) {
-                    key = kk;
-                    cand = u;
-                }
+            for (int t = 0; t < SFF_MAX_KNN; ++t) {
+                if (t == l / nx) sxl = sx[t];
+                if (t == l % nx) cxl = xx[t];
             }
-        }
-        // the smallest (cost, combination) key of the warp and its lane
-        unsigned long long m = key;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long om = __shfl_xor_sync(0xffffffffu, m, o);
-            m = om < m ? om : m;
-        }
-        const int c = (int)(m >> 32);
-        const int owner = __ffs(__ballot_sync(0xffffffffu, key == m && m != ~0ull)) - 1;
-        if (owner >= 0 && c < best) {
-            best = c;
-            bv.u = __shfl_sync(0xffffffffu, cand.u, owner);
-            bv.v = __shfl_sync(0xffffffffu, cand.v, owner);
-            bv.d0 = __shfl_sync(0xffffffffu, cand.d0, owner);
-            bv.d1 = __shfl_sync(0xffffffffu, cand.d1, owner);
+            return Vec4{(int16_t)(tx - px), (int16_t)(ty - py), (int16_t)(V.sigma * (px - sxl)),
+                        (int16_t)(V.sigma * (tx - cxl))};
+        };
+        for (int l0 = 0; l0 < ns * nx; l0 += 8) {
+            const int m = min(8, ns * nx - l0);
+            const int c = sift_costs<N>(S, buf, lane, m, [&](int l, int& x, int& y, Vec4& a) {
+                x = px;
+                y = py;
+                a = combination(l0 + l);
+            });
+            // the first minimum of the batch
+            const unsigned lowest = __reduce_min_sync(0xffffffffu, lane < m ? (unsigned)c : 0xffffffffu);
+            if ((int)lowest < best) {
+                best = (int)lowest;
+                bv = combination(l0 + __ffs(__ballot_sync(0xffffffffu, lane < m && (unsigned)c == lowest)) - 1);
+            }
         }
     }
     if (lane == 0) {
@@ -1884,68 +1982,165 @@ __global__ void k_sift_init(const __grid_constant__ Fields F, SiftViews S, int n
     }
 }
 
-__global__ void k_sift_inherit(SiftViews S, int gw, int gh, uint2* field, int* cost) {
-    const int gx = blockIdx.x * blockDim.x + threadIdx.x, gy = blockIdx.y;
-    if (gx >= gw || gy >= gh) return;
-    const int x = gx * S.n, y = gy * S.n;
-    const size_t i = pix(S.w, x, y);
-    if (((gx | gy) & 1) == 0 && cost[i] != kEmpty) {
-        cost[i] = sift_cost(S, x, y, unpack_vec(field[i]));
+// Points of the coarser grid keep their vector, with the cost at this scale
+// (8 of them per warp); the other points of this scale's grid start empty.
+template <int N>
+__global__ void __launch_bounds__(128) k_sift_inherit(SiftViews S, int gw, int gh, uint2* field, int* cost) {
+    __shared__ __align__(16) float s_dist[4][8 * kSiftStride];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int gx0 = 2 * 8 * (blockIdx.x * 4 + warp), gy = 2 * blockIdx.y;
+    if (gx0 >= gw) return;  // warp-uniform
+    const int m = min(8, (gw - gx0 + 1) / 2);
+    const size_t i0 = pix(S.w, gx0 * N, gy * N);
+    // an empty point's vector is 0: its cost is evaluated and dropped
+    const int c = sift_costs<N>(S, s_dist[warp], lane, m, [&](int k, int& x, int& y, Vec4& a) {
+        x = (gx0 + 2 * k) * N;
+        y = gy * N;
+        a = unpack_vec(field[i0 + (size_t)2 * k * N]);
+    });
+    if (lane >= m) return;
+    const int gx = gx0 + 2 * lane;
+    const size_t i = i0 + (size_t)2 * lane * N;
+    if (cost[i] != kEmpty) {
+        cost[i] = c;
     } else {
-        cost[i] = kEmpty;
         field[i] = make_uint2(0u, 0u);
     }
+#pragma unroll
+    for (int k = 1; k < 4; ++k) {
+        if (gx + (k & 1) >= gw || gy + (k >> 1) >= gh) continue;
+        const size_t j = i + (k & 1) * N + (size_t)(k >> 1) * N * S.w;
+        cost[j] = kEmpty;
+        field[j] = make_uint2(0u, 0u);
+    }
 }
 
-// Half-step of one colour: the pixel's own vector against its horizontal,
-// then its vertical predecessor's (strictly lower cost wins).
-__global__ void k_sift_half(SiftViews S, int gw, int gh, int colour, int dx, int dy, uint2* field, int* cost) {
-    const int gx = blockIdx.x * blockDim.x + threadIdx.x, gy = blockIdx.y;
-    if (gx >= gw || gy >= gh || ((gx + gy) & 1) != colour) return;
-    const int x = gx * S.n, y = gy * S.n;
-    const size_t i = pix(S.w, x, y);
-    int bc = cost[i];
-    uint2 bw = field[i];
-    const int qx[2] = {x - dx * S.n, x}, qy[2] = {y, y - dy * S.n};
+// One half-step of one colour: the random search of the previous iteration
+// (colour 0), the two predecessors, then this iteration's search (colour 1); a
+// search reads only its own pixel, so the order is that of half-step, half-step,
+// search (see k_iteration).  A warp takes kSiftTileX x kSiftTileY grid pixels, 16
+// of the colour, on its own: no barrier joins it to the others.
+//
+// A cost is 147 distances, so only candidates that can win are scored: not a
+// vector equal to the pixel's own or to the other predecessor's, nor one that
+// the pixel has scored before (stamp_limits); two thirds of the predecessors
+// drop out.  What remains is listed in pixel order and scored 8 at a time
+// (sift_costs), so nearly every lane works.  Both fields of a 1242 x 375 quad:
+// 18.4 ms (one thread per pixel, half the lanes of a half-step idle, every
+// predecessor scored, sqrt.rn) -> 8.8 ms, issue at 55 %, L1 at 60 % (scale 0).
+constexpr int kSiftTileX = 8, kSiftTileY = 4;
+constexpr int kSiftSlots = kSiftTileX * kSiftTileY / 2;  // pixels of a colour
+constexpr int kSiftWarps = 4;                            // 2 x 2 tiles per CTA
+
+struct SiftStep {
+    int gw, gh, s, it, dx, dy, mirror, colour;
+    int propagate;  // 0: only the search before it
+    int before, after;  // iteration of the search before / after the propagation (-1: none)
+    uint2 key;
+    uint2* field;
+    int* cost;
+    uint8_t* stamp;  // [gh][gw]
+};
+
+template <int N>
+__global__ void __launch_bounds__(32 * kSiftWarps, 4) k_sift_step(SiftViews S, SiftStep T) {
+    struct Warp {
+        float dist[8 * kSiftStride];
+        uint2 vec[3][kSiftSlots];  // candidates: search, horizontal, vertical
+        int cost[3][kSiftSlots];
+        uint8_t list[3 * kSiftSlots];  // candidates to score: candidate << 4 | pixel
+    };
+    static_assert(kSiftSlots == 16 && kSiftTileX % 2 == 0, "list entries, colours");
+    __shared__ __align__(16) Warp s_warp[kSiftWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    Warp& W = s_warp[warp];
+    const int tx0 = (2 * blockIdx.x + (warp & 1)) * kSiftTileX, ty0 = (2 * blockIdx.y + (warp >> 1)) * kSiftTileY;
+    // grid pixel of slot k of this tile and colour
+    auto grid_x = [&](int k) {
+        return tx0 + 2 * (k % (kSiftTileX / 2)) + ((ty0 + k / (kSiftTileX / 2) + T.colour) & 1);
+    };
+    auto grid_y = [&](int k) { return ty0 + k / (kSiftTileX / 2); };
+    const int gx = grid_x(lane), gy = grid_y(lane);
+    const bool valid = lane < kSiftSlots && gx < T.gw && gy < T.gh;
+    const size_t i = pix(S.w, gx * N, gy * N);
+    bool need[3] = {false, false, false};
+    Vec4 cand[3];
+    // scores the candidates k < kn with need[k] set, listed in the order of k and
+    // of the pixels
+    auto score = [&](int kn) {
+        int total = 0;
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        if (qx[k] < 0 || qy[k] < 0 || qx[k] >= S.w || qy[k] >= S.h) continue;
-        const size_t j = pix(S.w, qx[k], qy[k]);
-        if (cost[j] == kEmpty) continue;
-        const uint2 w = field[j];
-        const int c = sift_cost(S, x, y, unpack_vec(w));
-        if (c < bc) {
-            bc = c;
-            bw = w;
+        for (int k = 0; k < 3; ++k) {
+            if (k >= kn) continue;
+            const unsigned ballot = __ballot_sync(0xffffffffu, need[k]);
+            if (need[k]) {
+                W.vec[k][lane] = pack_vec(cand[k]);
+                W.list[total + __popc(ballot & ((1u << lane) - 1u))] = (uint8_t)(k << 4 | lane);
+            }
+            total += __popc(ballot);
+        }
+        __syncwarp();
+        for (int e0 = 0; e0 < total; e0 += 8) {
+            const int n = min(8, total - e0);
+            const int c = sift_costs<N>(S, W.dist, lane, n, [&](int k, int& x, int& y, Vec4& a) {
+                const int e = W.list[e0 + k], p = e & 15;
+                x = grid_x(p) * N;
+                y = grid_y(p) * N;
+                a = unpack_vec(W.vec[e >> 4][p]);
+            });
+            if (lane < n) W.cost[W.list[e0 + lane] >> 4][W.list[e0 + lane] & 15] = c;
+        }
+        __syncwarp();
+    };
+    int c = kEmpty;
+    Vec4 cur = {0, 0, 0, 0};
+    if (valid) {
+        c = T.cost[i];
+        cur = unpack_vec(T.field[i]);
+        if (T.before >= 0 && c != kEmpty)
+            need[0] = rs_candidate(N, T.s, T.key, T.mirror, T.before, (uint32_t)i, cur, cand[0]);
+        if (T.propagate) {
+            const bool has_a = gx - T.dx >= 0 && gx - T.dx < T.gw, has_b = gy - T.dy >= 0 && gy - T.dy < T.gh;
+            const ptrdiff_t oa = -(ptrdiff_t)T.dx * N, ob = -(ptrdiff_t)T.dy * N * S.w;
+            const size_t si = (size_t)gy * T.gw + gx;
+            const int ca = has_a ? T.cost[i + oa] : kEmpty, cb = has_b ? T.cost[i + ob] : kEmpty;
+            if (ca != kEmpty) cand[1] = unpack_vec(T.field[i + oa]);
+            if (cb != kEmpty) cand[2] = unpack_vec(T.field[i + ob]);
+            const StampLimits lim = stamp_limits(T.it, T.colour);
+            const bool stale_a = T.it >= 2 && ca != kEmpty && (int)T.stamp[si - T.dx] <= lim.h;
+            const bool stale_b = T.it >= 2 && cb != kEmpty && (int)T.stamp[si - (ptrdiff_t)T.dy * T.gw] <= lim.v;
+            need[1] = ca != kEmpty && !stale_a && !(c != kEmpty && same_vec(cand[1], cur));
+            need[2] = cb != kEmpty && !stale_b && !(c != kEmpty && same_vec(cand[2], cur)) &&
+                      !(ca != kEmpty && same_vec(cand[1], cand[2]));
         }
     }
-    field[i] = bw;
-    cost[i] = bc;
-}
-
-__global__ void k_sift_search(SiftViews S, int gw, int gh, int s, int it, int mirror, uint2 key, uint2* field,
-                              int* cost) {
-    const int gx = blockIdx.x * blockDim.x + threadIdx.x, gy = blockIdx.y;
-    if (gx >= gw || gy >= gh) return;
-    const int x = gx * S.n, y = gy * S.n;
-    const size_t i = pix(S.w, x, y);
-    const int c0 = cost[i];
-    if (c0 == kEmpty) return;
-    const Vec4 a = unpack_vec(field[i]);
-    const uint4 r = philox4x32_10(make_uint4((uint32_t)i, (uint32_t)it, (uint32_t)(s + 4 * mirror), 0u), key);
-    Vec4 u = {a.u + rs_offset(r.x, S.n), a.v + rs_offset(r.y, S.n), a.d0 + rs_offset(r.z, S.n),
-              a.d1 + rs_offset(r.w, S.n)};
-    if (u.d0 < 0) u.d0 = 0;
-    if (u.d1 < 0) u.d1 = 0;
-    u.u = (int16_t)u.u;
-    u.v = (int16_t)u.v;
-    u.d0 = (int16_t)u.d0;
-    u.d1 = (int16_t)u.d1;
-    const int c = sift_cost(S, x, y, u);
-    if (c < c0) {
-        field[i] = pack_vec(u);
-        cost[i] = c;
+    score(3);
+    bool changed = false;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        if (need[k] && W.cost[k][lane] < c) {
+            c = W.cost[k][lane];
+            cur = cand[k];
+            changed = true;
+        }
+    if (T.after >= 0) {
+        need[0] = valid && c != kEmpty &&
+                  rs_candidate(N, T.s, T.key, T.mirror, T.after, (uint32_t)i, cur, cand[0]);
+        __syncwarp();
+        score(1);
+        if (need[0] && W.cost[0][lane] < c) {
+            c = W.cost[0][lane];
+            cur = cand[0];
+            changed = true;
+        }
     }
+    if (!valid) return;
+    if (changed) {
+        T.field[i] = pack_vec(cur);
+        T.cost[i] = c;
+    }
+    if (T.propagate && (changed || T.it == 0))
+        T.stamp[(size_t)gy * T.gw + gx] = (uint8_t)(changed ? 2 * T.it + 1 + T.colour : 0);
 }
 
 // Instantiated variants of the iteration kernel; any of them gives identical
@@ -2162,8 +2357,18 @@ FieldScratch field_scratch(int w, int h, const sff_params& p) {
 
 size_t field_ws_bytes(int w, int h, const sff_params& p) { return field_scratch(w, h, p).total; }
 
-// Workspace of sff_match_views / sff_match_quad: the scratch of two fields.
-size_t match_ws_bytes(int w, int h, const sff_params& p) { return 2 * field_ws_bytes(w, h, p); }
+// The repacked phi of sff_match_views_sift (k_sift_pack): 16 bytes per pixel of
+// four views, rows padded to whole residue classes.
+size_t sift_pack_bytes(int w, int h, const sff_params& p) {
+    const int n = 1 << (p.num_scales - 1);
+    return n > 1 ? align256((size_t)4 * h * ((w + n - 1) / n * n) * 16) : 0;
+}
+
+// Workspace of the matching calls: the scratch of two fields (sff_match_quad)
+// or of one and the repacked phi.
+size_t match_ws_bytes(int w, int h, const sff_params& p) {
+    return field_ws_bytes(w, h, p) + std::max(field_ws_bytes(w, h, p), sift_pack_bytes(w, h, p));
+}
 
 // Opts k_knn_tc into its dynamic shared memory, once per device.
 bool knn_smem_ready() {
@@ -2451,34 +2656,77 @@ int run_field_sift(const FieldSpec& fs, const float* const* phi, const sff_param
     int* cost = fs.cost;
     const size_t np = (size_t)w * h;
     SFF_LAUNCH(k_sift_clear, dim3((unsigned)((np + 255) / 256)), 256, 0, st, field, cost, np);
-    for (int s = S - 1; s >= 0; --s) {
-        const int n = 1 << s, gw = (w + n - 1) / n, gh = (h + n - 1) / n;
+    SiftStep T = {};
+    T.mirror = fs.mirror;
+    T.key = A.key;
+    T.field = field;
+    T.cost = cost;
+    T.stamp = reinterpret_cast<uint8_t*>(ws + sc.stamp);
+    // one scale at stride N
+    auto scale = [&](auto stride, int s) -> int {
+        constexpr int N = decltype(stride)::value;
+        const int gw = (w + N - 1) / N, gh = (h + N - 1) / N;
         const size_t off = (size_t)s * np;
-        SiftViews SV{reinterpret_cast<const float4*>(phi[0]) + off, reinterpret_cast<const float4*>(phi[1]) + off,
-                     reinterpret_cast<const float4*>(phi[2]) + off, reinterpret_cast<const float4*>(phi[3]) + off,
-                     w, h, n, fs.mirror ? -1 : 1};
-        const dim3 g((gw + 127) / 128, gh);
+        SiftViews SV{};
+        SiftPhi SP{};
+        SV.w = w;
+        SV.h = h;
+        SV.n = N;
+        SV.sigma = fs.mirror ? -1 : 1;
+        SV.m = (w + N - 1) / N;
+        SV.pitch = N * SV.m;
+        SP.packed = reinterpret_cast<float4*>(ws + sc.total);
+        for (int k = 0; k < 4; ++k) {
+            SP.v[k] = reinterpret_cast<const float4*>(phi[k]) + off;
+            SV.v[k] = N > 1 ? SP.packed + (size_t)k * h * SV.pitch : SP.v[k];
+        }
+        if (N > 1) SFF_LAUNCH(k_sift_pack<N>, dim3((SV.pitch + 255) / 256, h, 4), 256, 0, st, SP, SV);
         if (s == S - 1) {
             A.V = Views{plane_of(fs.ref, s, S, w, h), plane_of(fs.tmp, s, S, w, h), plane_of(fs.ste, s, S, w, h),
                         plane_of(fs.crs, s, S, w, h), w, h, fs.mirror ? -1 : 1};
             A.gw = gw;
             A.gh = gh;
             dim3 g0((tc_rows(A.gq) * 8 + 255) / 256, 4, 1);
-            SFF_LAUNCH(k_gather_grid, g0, 256, 0, st, F, n);
+            SFF_LAUNCH(k_gather_grid, g0, 256, 0, st, F, N);
             if (!knn_smem_ready()) return SFF_ERR_CUDA;
             dim3 g1((A.gq + kTcRows - 1) / kTcRows, 1, 1);
             SFF_LAUNCH(k_knn_tc, g1, kTcThreads, kTcSmemBytes, st, F);
-            SFF_LAUNCH(k_sift_init, dim3((A.gq + 7) / 8), 256, 0, st, F, SV, n, P.knn_temporal, P.knn_epipolar, field,
+            SFF_LAUNCH(k_sift_init<N>, dim3((A.gq + 7) / 8), 256, 0, st, F, SV, P.knn_temporal, P.knn_epipolar, field,
                        cost);
         } else {
-            SFF_LAUNCH(k_sift_inherit, g, 128, 0, st, SV, gw, gh, field, cost);
+            SFF_LAUNCH(k_sift_inherit<N>, dim3(((gw + 1) / 2 + 31) / 32, (gh + 1) / 2), 128, 0, st, SV, gw, gh, field,
+                       cost);
         }
+        T.gw = gw;
+        T.gh = gh;
+        T.s = s;
+        const dim3 g((gw + 2 * kSiftTileX - 1) / (2 * kSiftTileX), (gh + 2 * kSiftTileY - 1) / (2 * kSiftTileY));
         for (int it = 0; it < I; ++it) {
-            for (int colour = 0; colour < 2; ++colour)
-                SFF_LAUNCH(k_sift_half, g, 128, 0, st, SV, gw, gh, colour, kDirs[it % 4][0], kDirs[it % 4][1], field,
-                           cost);
-            SFF_LAUNCH(k_sift_search, g, 128, 0, st, SV, gw, gh, s, it, fs.mirror, A.key, field, cost);
+            T.it = it;
+            T.dx = kDirs[it % 4][0];
+            T.dy = kDirs[it % 4][1];
+            T.propagate = 1;
+            for (int colour = 0; colour < 2; ++colour) {
+                T.colour = colour;
+                T.before = colour ? -1 : it - 1;
+                T.after = colour ? it : -1;
+                SFF_LAUNCH(k_sift_step<N>, g, 32 * kSiftWarps, 0, st, SV, T);
+            }
         }
+        if (I > 0) {  // colour 0's search of the last iteration
+            T.colour = T.propagate = 0;
+            T.before = I - 1;
+            T.after = -1;
+            SFF_LAUNCH(k_sift_step<N>, g, 32 * kSiftWarps, 0, st, SV, T);
+        }
+        return SFF_OK;
+    };
+    for (int s = S - 1; s >= 0; --s) {
+        const int status = s == 0 ? scale(std::integral_constant<int, 1>{}, s)
+                           : s == 1 ? scale(std::integral_constant<int, 2>{}, s)
+                           : s == 2 ? scale(std::integral_constant<int, 4>{}, s)
+                                    : scale(std::integral_constant<int, 8>{}, s);
+        if (status) return status;
     }
     return launch_status();
 }

@@ -96,3 +96,48 @@ def test_scratch_of_one_scale_gives_the_same_phi():
         assert all(torch.equal(a, b) for a, b in zip(outs[0], o))
     with pytest.raises(sff.SffError):
         sff.sift_features(dev, phis, torch.empty(small - 4096, dtype=torch.uint8, device="cuda"), p)
+
+
+@pytest.mark.parametrize("w,h,S,knn_t,knn_e", [(8, 8, 4, 8, 8), (9, 11, 1, 3, 1), (67, 35, 4, 4, 2), (130, 33, 3, 8, 3),
+                                               (16, 40, 2, 1, 8)])
+def test_sift_fields_at_tile_edges(w, h, S, knn_t, knn_e):
+    """The matching with the SIFT cost where tiles, windows and candidate lists
+    are partial (images smaller than a window's reach, one to eight
+    combinations and more), on features with exact zeros among the distances
+    (flat areas shared by the views) and with values outside the fast root's
+    range: the fields and the costs' bit patterns equal the oracle's."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import oracle
+    import paper_1710_10096_gb300 as sff
+    sff.build()
+    oracle.build()
+    oracle.set_threads(os.cpu_count() or 1)
+    rng = np.random.default_rng(w * h + S)
+    images = scenegen.random_images(w, h, seed=w + h, n=4)
+    for im in images:
+        im[: h // 2, : w // 2] = 90
+    p = sff.default_params(num_scales=S, iterations=5, knn_temporal=knn_t, knn_epipolar=knn_e)
+    op = oracle.default_params(**p.as_dict())
+    dev = [torch.as_tensor(im).cuda() for im in images]
+    ws = torch.empty(sff.workspace_bytes(w, h, p), dtype=torch.uint8, device="cuda")
+    pyr = [torch.empty(sff.pyramid_bytes(w, h, p), dtype=torch.uint8, device="cuda") for _ in range(4)]
+    for im, py in zip(dev, pyr):
+        sff.features(im, py, ws, p)
+    phis = [(rng.standard_normal((S, h, w, 4)) * 40).astype(np.float32) for _ in range(4)]
+    for f in phis:
+        f[..., 3] = 0
+        f[:, : h // 2, : w // 2] = 1.5                      # exact zero distances
+        f[:, h // 2:, : w // 4, :3] *= np.float32(1e-18)     # squares below 2^-96
+        f[0, -1, -1, 0] = np.float32(3e17)                   # a square above 2^100
+    dphi = [torch.as_tensor(f).cuda() for f in phis]
+    for mirror, order in ((0, (0, 2, 1, 3)), (1, (3, 1, 2, 0))):
+        field = torch.empty((h, w, 4), dtype=torch.int16, device="cuda")
+        cost = torch.empty((h, w), dtype=torch.int32, device="cuda")
+        sff.match_views_sift(*[pyr[k] for k in order], *[dphi[k] for k in order], w, h, mirror, 77, field, cost, ws, p)
+        torch.cuda.synchronize()
+        feats = [oracle.features(im, op)[0] for im in images]
+        wf, wc = oracle.match_views_sift(*[feats[k] for k in order], *[phis[k] for k in order], w, h, mirror, 77, op)
+        assert np.array_equal(cost.cpu().numpy(), wc)
+        assert np.array_equal(field.cpu().numpy(), wf)
