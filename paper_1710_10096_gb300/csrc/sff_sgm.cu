@@ -19,26 +19,19 @@
 // k_sgm_census: grey and census of both images from a shared-memory tile.
 // k_sgm_cost:   the cost volume, one byte per pixel and disparity (a path
 //               step then reads D bytes instead of D census words).
-// k_sgm_paths:  one warp per path line of one direction (blockIdx.z), the
-//               lanes holding D / 32 consecutive disparities each; one step
-//               per pixel, the costs of the next 32 pixels of the line in
-//               flight into a shared-memory ring (cp.async): the
-//               neighbours' d +- 1 values by shuffles, the minimum over d
-//               by one redux; L_r to [dir][y][x][d].
-// k_sgm_wta:    one warp per pixel: the 8 directions summed per disparity,
-//               the (sum, d) minimum by a warp reduction.
+// k_sgm_paths:  the path lines of all directions; L_r to [dir][y][x][d].
+// k_sgm_wta:    the 8 directions summed per disparity, the (sum, d) minimum.
+#include <cstring>
+
 #include "sff_internal.cuh"
 
 namespace sff {
 namespace {
 
 constexpr int kDirs = 8;
-constexpr int kPathWarps = 4;  // warps (lines) per CTA of k_sgm_paths
-constexpr int kRing = 32;      // pixels whose costs a path warp has in flight (shared-memory ring)
-constexpr int kWtaWarps = 8;   // warps (pixels) per CTA of k_sgm_wta
+constexpr int kWtaWarps = 8;   // warps per CTA of k_sgm_wta
 constexpr int kCensusW = 9, kCensusH = 7;
 constexpr int kTileX = 32, kTileY = 8;
-constexpr int kInf = 1 << 20;
 constexpr unsigned kFull = 0xffffffffu;
 
 struct SgmJob {
@@ -80,115 +73,116 @@ __global__ void __launch_bounds__(kTileX * kTileY) k_sgm_census(SgmJob S) {
     (blockIdx.z ? S.census[1] : S.census[0])[(size_t)y * S.w + x] = bits;
 }
 
-template <int J>
-__device__ __forceinline__ void store_bytes(uint8_t* p, const int (&v)[J]) {
-    if constexpr (J == 1) {
-        *p = (uint8_t)v[0];
-    } else if constexpr (J == 2) {
-        *reinterpret_cast<uint16_t*>(p) = (uint16_t)(v[0] | (v[1] << 8));
-    } else if constexpr (J == 4) {
-        *reinterpret_cast<uint32_t*>(p) = (uint32_t)v[0] | ((uint32_t)v[1] << 8) | ((uint32_t)v[2] << 16) |
-                                          ((uint32_t)v[3] << 24);
-    } else {
-        static_assert(J == 8, "D = 32, 64, 128 or 256");
-        uint2 w;
-        w.x = (uint32_t)v[0] | ((uint32_t)v[1] << 8) | ((uint32_t)v[2] << 16) | ((uint32_t)v[3] << 24);
-        w.y = (uint32_t)v[4] | ((uint32_t)v[5] << 8) | ((uint32_t)v[6] << 16) | ((uint32_t)v[7] << 24);
-        *reinterpret_cast<uint2*>(p) = w;
+// K bytes in registers: one access of 16, 8, 4 or 2 bytes.
+template <int K>
+struct Bytes;
+template <>
+struct Bytes<16> { using Vec = uint4; };
+template <>
+struct Bytes<8> { using Vec = uint2; };
+template <>
+struct Bytes<4> { using Vec = uint32_t; };
+template <>
+struct Bytes<2> { using Vec = uint16_t; };
+
+// The costs of K consecutive disparities as 16-bit pairs: word j holds bytes j and
+// K/2 + j.
+__device__ __forceinline__ void unpack_pairs(const uint4& v, uint32_t (&c)[8]) {
+    // costs are below 128, so the permute's sign-replicating selectors (bit 3
+    // set) give the zero bytes
+    const uint32_t lo[2] = {v.x, v.y}, hi[2] = {v.z, v.w};
+#pragma unroll
+    for (uint32_t j = 0; j < 8; ++j) {
+        const uint32_t k = j & 3;
+        asm("prmt.b32 %0, %1, %2, %3;"
+            : "=r"(c[j])
+            : "r"(lo[j >> 2]), "r"(hi[j >> 2]), "r"(k | (8 + k) << 4 | (4 + k) << 8 | (12 + k) << 12));
     }
 }
-
-// J bytes as one machine word (kept packed while loads are in flight).
-template <int J>
-struct RawOf;
-template <>
-struct RawOf<1> { using T = uint8_t; };
-template <>
-struct RawOf<2> { using T = uint16_t; };
-template <>
-struct RawOf<4> { using T = uint32_t; };
-template <>
-struct RawOf<8> { using T = uint2; };
-
-template <int J>
-__device__ __forceinline__ typename RawOf<J>::T load_raw(const uint8_t* q) {
-    return *reinterpret_cast<const typename RawOf<J>::T*>(q);
+__device__ __forceinline__ void unpack_pairs(const uint2& v, uint32_t (&c)[4]) {
+#pragma unroll
+    for (uint32_t k = 0; k < 4; ++k)
+        asm("prmt.b32 %0, %1, %2, %3;"
+            : "=r"(c[k])
+            : "r"(v.x), "r"(v.y), "r"(k | (8 + k) << 4 | (4 + k) << 8 | (12 + k) << 12));
+}
+__device__ __forceinline__ void unpack_pairs(const uint32_t& v, uint32_t (&c)[2]) {
+    c[0] = v & 0x00ff00ffu;
+    c[1] = (v >> 8) & 0x00ff00ffu;
+}
+__device__ __forceinline__ void unpack_pairs(const uint16_t& v, uint32_t (&c)[1]) {
+    c[0] = __byte_perm((uint32_t)v, 0u, 0x4140);
 }
 
-template <int J>
-__device__ __forceinline__ void unpack(typename RawOf<J>::T t, int (&v)[J]) {
-    if constexpr (J == 8) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            v[j] = (t.x >> (8 * j)) & 0xff;
-            v[4 + j] = (t.y >> (8 * j)) & 0xff;
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < J; ++j) v[j] = ((uint32_t)t >> (8 * j)) & 0xff;
-    }
+// And back, every half below 256.
+__device__ __forceinline__ void pack_four(const uint32_t* c, uint32_t& lo, uint32_t& hi) {
+    const uint32_t a = __byte_perm(c[0], c[1], 0x6240), b = __byte_perm(c[2], c[3], 0x6240);
+    lo = __byte_perm(a, b, 0x5410);
+    hi = __byte_perm(a, b, 0x7632);
 }
-
-template <int J>
-__device__ __forceinline__ void load_bytes(const uint8_t* q, int (&v)[J]) {
-    if constexpr (J == 1) {
-        v[0] = q[0];
-    } else if constexpr (J == 2) {
-        const uint16_t t = *reinterpret_cast<const uint16_t*>(q);
-        v[0] = t & 0xff;
-        v[1] = t >> 8;
-    } else if constexpr (J == 4) {
-        const uint32_t t = *reinterpret_cast<const uint32_t*>(q);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) v[j] = (t >> (8 * j)) & 0xff;
-    } else {
-        const uint2 t = *reinterpret_cast<const uint2*>(q);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            v[j] = (t.x >> (8 * j)) & 0xff;
-            v[4 + j] = (t.y >> (8 * j)) & 0xff;
-        }
-    }
+__device__ __forceinline__ void pack_pairs(const uint32_t (&c)[8], uint4& v) {
+    pack_four(c, v.x, v.z);
+    pack_four(c + 4, v.y, v.w);
+}
+__device__ __forceinline__ void pack_pairs(const uint32_t (&c)[4], uint2& v) { pack_four(c, v.x, v.y); }
+__device__ __forceinline__ void pack_pairs(const uint32_t (&c)[2], uint32_t& v) { v = c[0] | c[1] << 8; }
+__device__ __forceinline__ void pack_pairs(const uint32_t (&c)[1], uint16_t& v) {
+    v = (uint16_t)__byte_perm(c[0], 0u, 0x4420);
 }
 
 // C(p, d) for every pixel.  One CTA per segment of kCostSeg pixels of a row:
 // the right image's census words the segment needs (x - D + 1 .. the
-// segment's end, positions clamped at 0) are staged in shared memory once;
-// each warp then takes pixels of the segment, J disparities per lane, the
-// J costs of a lane packed into J bytes of [y][x][d].
+// segment's end, positions clamped at 0) are staged in shared memory once; a
+// thread keeps its disparity, so a warp reads 32 consecutive words, and the
+// bytes are put together in shared memory for whole 16-byte stores.  Bound by
+// the popcounts.  1242 x 375, D = 128: 59 us (J consecutive disparities per
+// lane: the reads conflicted four ways) -> 36 us.
 constexpr int kCostSeg = 64;
 constexpr int kCostThreads = 256;
 
-template <int J>
+template <int D>
 __global__ void __launch_bounds__(kCostThreads) k_sgm_cost(SgmJob S) {
-    constexpr int D = 32 * J;
-    __shared__ uint64_t right[kCostSeg + D - 1];
-    const int y = blockIdx.y, x0 = blockIdx.x * kCostSeg;
-    const uint64_t* rrow = S.census[1] + (size_t)y * S.w;
+    __shared__ uint64_t right[kCostSeg + D - 1], left[kCostSeg];
+    __shared__ __align__(16) uint8_t out[kCostSeg * D];
+    const int y = blockIdx.y, x0 = blockIdx.x * kCostSeg, t = threadIdx.x;
+    const size_t row = (size_t)y * S.w;
     const int base = x0 - (D - 1);  // census position of right[0]
-    for (int i = threadIdx.x; i < kCostSeg + D - 1; i += kCostThreads)
-        right[i] = rrow[min(max(base + i, 0), S.w - 1)];
+    for (int i = t; i < kCostSeg + D - 1; i += kCostThreads)
+        right[i] = S.census[1][row + min(max(base + i, 0), S.w - 1)];
+    if (t < kCostSeg) left[t] = S.census[0][row + min(x0 + t, S.w - 1)];
     __syncthreads();
-    const int lane = threadIdx.x & 31;
-    for (int k = threadIdx.x >> 5; k < kCostSeg; k += kCostThreads / 32) {
-        const int x = x0 + k;
-        if (x >= S.w) break;  // uniform over the warp
-        const size_t p = (size_t)y * S.w + x;
-        const uint64_t c = S.census[0][p];
-        int v[J];
-#pragma unroll
-        for (int j = 0; j < J; ++j) v[j] = __popcll(c ^ right[max(x - (lane * J + j), 0) - base]);
-        store_bytes<J>(S.cost + p * D + lane * J, v);
-    }
+    // right[k + D - 1 - d] is position x0 + k - d (already clamped)
+    const int d = t % D;
+#pragma unroll 4
+    for (int k = t / D; k < kCostSeg; k += kCostThreads / D)
+        out[k * D + d] = (uint8_t)__popcll(left[k] ^ right[k + D - 1 - d]);
+    __syncthreads();
+    const int bytes = min(kCostSeg, S.w - x0) * D;
+    uint4* dst = reinterpret_cast<uint4*>(S.cost + (row + x0) * D);
+    for (int i = t; i < bytes / 16; i += kCostThreads) dst[i] = reinterpret_cast<const uint4*>(out)[i];
 }
 
-template <int J>
-__global__ void __launch_bounds__(kPathWarps * 32) k_sgm_paths(SgmJob S) {
-    const int dir = blockIdx.z;
+// The path costs of one direction.  G lanes take a line's D disparities, K = D / G
+// consecutive ones each, and a warp 32 / G neighbouring lines.  Two disparities
+// share a 32-bit word as 16-bit halves: word j of a lane holds d = b + j and b +
+// K/2 + j, so that the d - 1 and d + 1 neighbours of a word are the words beside it
+// and only the two outer ones need a shuffle and a permute.  Every value stays
+// below 2^16 and every difference taken is >= 0, so plain 32-bit adds and
+// subtracts act on both halves:
+//   L(p, d) = C + min(P, min(P(d - 1), P(d + 1)) + P1, m + P2) - m.
+// Starting from P = m = 0 gives L = C at a line's first pixel.  Beyond the
+// disparity range: 0x7fff.  The costs of the next pixels are in flight in registers.
+constexpr int kAheadNarrow = 16, kAheadWide = 8;  // 8 and 4: 197 us
+
+template <int D, int K>
+__device__ __forceinline__ void path_lines(const SgmJob& S, int dir, int block) {
+    constexpr int G = D / K, NP = K / 2, kAhead = K <= 4 ? kAheadNarrow : kAheadWide;
+    static_assert(G >= 2 && G <= 32, "lanes per line");
+    using Vec = typename Bytes<K>::Vec;
     const int rx = c_dir[dir][0], ry = c_dir[dir][1];
-    const int lane = threadIdx.x & 31;
-    const int line = blockIdx.x * kPathWarps + (threadIdx.x >> 5);
-    const int W = S.w, H = S.h, D = S.D;
+    const int lane = threadIdx.x & 31, gl = lane % G;
+    const int line = block * (32 / G) + lane / G;
+    const int W = S.w, H = S.h;
     // the line's first pixel: the pixels whose predecessor is outside the image
     int x, y, nlines;
     if (ry == 0) {
@@ -209,151 +203,139 @@ __global__ void __launch_bounds__(kPathWarps * 32) k_sgm_paths(SgmJob S) {
             y = ry > 0 ? 1 + (line - W) : H - 2 - (line - W);
         }
     }
-    if (line >= nlines) return;  // warp-uniform
-    uint8_t* out = S.paths + (size_t)dir * W * H * D + lane * J;
-    // steps until the line leaves the image
-    const int n = min(rx > 0 ? W - x : rx < 0 ? x + 1 : 1 << 30, ry > 0 ? H - y : ry < 0 ? y + 1 : 1 << 30);
-    const ptrdiff_t step = (ptrdiff_t)ry * W + rx;  // pixel index increment along the line
-    const size_t p0 = (size_t)y * W + x;
-    // The costs of the next kRing pixels of the line stream into a ring in
-    // shared memory with cp.async (one commit group per pixel, so a step
-    // waits only for its own pixel's group); the copy is spread over the
-    // lanes in 4-byte pieces.
-    extern __shared__ __align__(16) uint8_t ring_all[];
-    uint8_t* ring = ring_all + (size_t)(threadIdx.x >> 5) * kRing * D;
-    const uint8_t* line_cost = S.cost;
-    auto fetch = [&](int t) {  // pixel t of the line into its ring slot
-        if (t < n) {
-            const uint8_t* src = line_cost + (p0 + (ptrdiff_t)t * step) * D;
-            uint8_t* dst = ring + (t % kRing) * D;
-            for (int b = 4 * lane; b < D; b += 128) {
-                const unsigned sa = (unsigned)__cvta_generic_to_shared(dst + b);
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(src + b) : "memory");
+    // steps until the line leaves the image (0: no such line)
+    const int n = line >= nlines ? 0
+                                 : min(rx > 0 ? W - x : rx < 0 ? x + 1 : 1 << 30, ry > 0 ? H - y : ry < 0 ? y + 1 : 1 << 30);
+    const int most = (int)__reduce_max_sync(kFull, (unsigned)n);
+    const ptrdiff_t step = ((ptrdiff_t)ry * W + rx) * D;  // bytes from a pixel to the next
+    const size_t p0 = n ? ((size_t)y * W + x) * D + gl * K : 0;
+    const uint8_t* src = S.cost + p0;
+    uint8_t* dst = S.paths + (size_t)dir * W * H * D + p0;
+    Vec ahead[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+        ahead[u] = Vec{};
+        if (u < n) ahead[u] = *reinterpret_cast<const Vec*>(src + u * step);
+    }
+    src += kAhead * step;
+    const uint32_t p1x2 = (uint32_t)S.p1 * 0x00010001u, p2x2 = (uint32_t)S.p2 * 0x00010001u;
+    const bool first = gl == 0, last = gl == G - 1;
+    uint32_t prev[NP];
+#pragma unroll
+    for (int j = 0; j < NP; ++j) prev[j] = 0;
+    uint32_t m2 = 0;  // the minimum over d, in both halves
+    for (int t0 = 0; t0 < most; t0 += kAhead) {
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const int t = t0 + u;
+            uint32_t cost[NP];
+            unpack_pairs(ahead[u], cost);
+            if (t + kAhead < n) ahead[u] = *reinterpret_cast<const Vec*>(src);
+            src += step;
+            // the words below word 0 and above word NP - 1
+            const uint32_t lo = __shfl_up_sync(kFull, prev[NP - 1], 1, G), hi = __shfl_down_sync(kFull, prev[0], 1, G);
+            const uint32_t below = __byte_perm(first ? 0x7fff0000u : lo, prev[NP - 1], 0x5432);
+            const uint32_t above = __byte_perm(prev[0], last ? 0x00007fffu : hi, 0x5432);
+            const uint32_t mp2 = m2 + p2x2;
+            uint32_t cur[NP];
+#pragma unroll
+            for (int j = 0; j < NP; ++j) {
+                const uint32_t side = __vminu2(j > 0 ? prev[j - 1] : below, j < NP - 1 ? prev[j + 1] : above);
+                cur[j] = __vminu2(__viaddmin_u16x2(side, p1x2, mp2), prev[j]) + (cost[j] - m2);
             }
-        }
-        asm volatile("cp.async.commit_group;\n" ::: "memory");
-    };
-    for (int t = 0; t < kRing; ++t) fetch(t);
-    auto take = [&](int t) {  // pixel t's costs, this lane's J bytes
-        asm volatile("cp.async.wait_group %0;\n" ::"n"(kRing - 1) : "memory");
-        __syncwarp();
-        const typename RawOf<J>::T r = load_raw<J>(ring + (t % kRing) * D + lane * J);
-        __syncwarp();  // every lane has read the slot before it is refilled
-        fetch(t + kRing);
-        return r;
-    };
-    if constexpr (J == 1) {
-        int prev = 0, m = 0;
-        for (int t = 0; t < n; ++t) {
-            {
-                {
-                    const size_t p = p0 + (ptrdiff_t)t * step;
-                    int cur[1];
-                    unpack<1>(take(t), cur);
-                    if (t > 0) {
-                        const int lo = __shfl_up_sync(kFull, prev, 1), hi = __shfl_down_sync(kFull, prev, 1);
-                        const int pl = lane > 0 ? lo : kInf, pr = lane < 31 ? hi : kInf;
-                        cur[0] += min(min(prev, min(pl, pr) + S.p1), m + S.p2) - m;
-                    }
-                    store_bytes<1>(out + p * D, cur);
-                    m = __reduce_min_sync(kFull, cur[0]);
-                    prev = cur[0];
-                }
+            if (t < n) {
+                Vec v;
+                pack_pairs(cur, v);
+                *reinterpret_cast<Vec*>(dst) = v;
             }
-        }
-    } else {
-        // Two disparities per 32-bit word (16-bit halves; every value stays
-        // below 2^16 and every difference taken is >= 0, so plain 32-bit
-        // adds and subtracts act on both halves) and the recurrence on the
-        // DPX add-min instructions:
-        //   min(P, Lm + P1, Rp + P1, m + P2) = min(min(Lm + P1, m + P2),
-        //                                          min(Rp + P1, P)).
-        // Lm / Rp: the pair of each half's d - 1 / d + 1 values, from byte
-        // permutes of neighbouring pairs (the outer ones from the
-        // neighbouring lanes); beyond the disparity range 0x7fff.
-        constexpr int NP = J / 2;
-        const uint32_t p1x2 = (uint32_t)S.p1 * 0x00010001u;
-        uint32_t prev[NP];
-        uint32_t m = 0;
-        for (int t = 0; t < n; ++t) {
-            {
-                {
-                    const size_t p = p0 + (ptrdiff_t)t * step;
-                    const typename RawOf<J>::T raw = take(t);
-                    uint32_t c2[NP];  // costs as 16-bit pairs
-                    if constexpr (J == 2) {
-                        c2[0] = __byte_perm((uint32_t)raw, 0u, 0x4140);
-                    } else if constexpr (J == 4) {
-                        c2[0] = __byte_perm((uint32_t)raw, 0u, 0x4140);
-                        c2[1] = __byte_perm((uint32_t)raw, 0u, 0x4342);
-                    } else {
-                        c2[0] = __byte_perm(raw.x, 0u, 0x4140);
-                        c2[1] = __byte_perm(raw.x, 0u, 0x4342);
-                        c2[2] = __byte_perm(raw.y, 0u, 0x4140);
-                        c2[3] = __byte_perm(raw.y, 0u, 0x4342);
-                    }
-                    uint32_t cur[NP];
-                    if (t > 0) {
-                        const uint32_t lo = __shfl_up_sync(kFull, prev[NP - 1], 1);  // its high half: d = lane J - 1
-                        const uint32_t hi = __shfl_down_sync(kFull, prev[0], 1);     // its low half: d = lane J + J
-                        const uint32_t left = lane > 0 ? lo : 0x7fff0000u, right = lane < 31 ? hi : 0x00007fffu;
-                        const uint32_t mp2 = (m + (uint32_t)S.p2) * 0x00010001u, m2 = m * 0x00010001u;
+            dst += step;
+            uint32_t mm[NP];
 #pragma unroll
-                        for (int j = 0; j < NP; ++j) {
-                            const uint32_t lm = __byte_perm(j > 0 ? prev[j - 1] : left, prev[j], 0x5432);
-                            const uint32_t rp = __byte_perm(prev[j], j < NP - 1 ? prev[j + 1] : right, 0x5432);
-                            const uint32_t b = __vminu2(__viaddmin_u16x2(lm, p1x2, mp2),
-                                                             __viaddmin_u16x2(rp, p1x2, prev[j]));
-                            cur[j] = b + c2[j] - m2;
-                        }
-                    } else {
+            for (int j = 0; j < NP; ++j) prev[j] = mm[j] = cur[j];
 #pragma unroll
-                        for (int j = 0; j < NP; ++j) cur[j] = c2[j];
-                    }
-                    // back to bytes (every value < 256)
-                    if constexpr (J == 2) {
-                        *reinterpret_cast<uint16_t*>(out + p * D) = (uint16_t)__byte_perm(cur[0], 0u, 0x4420);
-                    } else if constexpr (J == 4) {
-                        *reinterpret_cast<uint32_t*>(out + p * D) = __byte_perm(cur[0], cur[1], 0x6420);
-                    } else {
-                        *reinterpret_cast<uint2*>(out + p * D) =
-                            make_uint2(__byte_perm(cur[0], cur[1], 0x6420), __byte_perm(cur[2], cur[3], 0x6420));
-                    }
-                    uint32_t mm = cur[0];
+            for (int w = NP / 2; w >= 1; w >>= 1)
 #pragma unroll
-                    for (int j = 1; j < NP; ++j) mm = __vminu2(mm, cur[j]);
-                    m = __reduce_min_sync(kFull, min(mm & 0xffffu, mm >> 16));
+                for (int j = 0; j < w; ++j) mm[j] = __vminu2(mm[j], mm[j + w]);
+            if constexpr (G == 32) {
+                m2 = __reduce_min_sync(kFull, min(mm[0] & 0xffffu, mm[0] >> 16)) * 0x00010001u;
+            } else {
+                m2 = __vminu2(mm[0], __byte_perm(mm[0], 0u, 0x1032));
 #pragma unroll
-                    for (int j = 0; j < NP; ++j) prev[j] = cur[j];
-                }
+                for (int o = 1; o < G; o <<= 1) m2 = __vminu2(m2, __shfl_xor_sync(kFull, m2, o));
             }
         }
     }
-    asm volatile("cp.async.wait_all;\n" ::: "memory");
 }
 
-template <int J>
+// Two splits of a line.  The horizontal lines are the longest chains of steps (W,
+// the others at most H) and few, so they get the shortest step: all lanes (16 at
+// D = 32) on one line and the minimum by one redux.  The others share a warp: the
+// fixed work of a step (addresses, loop, the minimum by shuffles) then serves
+// several lines.  One warp per CTA, the horizontal ones first.
+template <int D>
+struct Split {
+    static constexpr int kAcross = D >= 64 ? D / 32 : 2;  // disparities per lane, horizontal lines
+    static constexpr int kOther = D >= 128 ? 16 : 8;
+    __host__ __device__ static int blocks_across(int h) { return (h * (D / kAcross) + 31) / 32; }
+    __host__ __device__ static int blocks(int lines) { return (lines * (D / kOther) + 31) / 32; }
+};
+
+// All directions.  Bound by the ALU pipe (67 % while the SMs are busy) and
+// a tail of the horizontal lines (28 %).  1242 x 375, D = 128: 403 us (one line per
+// warp, d +- 1 by permutes per word, costs through a cp.async ring) -> 231 us (every
+// line on 8 lanes) -> 191 us.
+template <int D>
+__global__ void __launch_bounds__(32) k_sgm_paths(SgmJob S) {
+    using P = Split<D>;
+    const int across = P::blocks_across(S.h), b = (int)blockIdx.x;
+    if (b < 2 * across) {
+        path_lines<D, P::kAcross>(S, b & 1, b >> 1);
+    } else {
+        const int k = b - 2 * across, per = P::blocks(S.w + S.h - 1);
+        path_lines<D, P::kOther>(S, 2 + k / per, k % per);
+    }
+}
+
+// argmin over d of the sum of the 8 directions: K consecutive disparities per lane
+// and direction, summed as 16-bit pairs.  Bound by HBM.  1242 x 375, D = 128:
+// 96 us (one pixel per warp, 4 bytes a load) -> 72 us.
+template <int D>
 __global__ void __launch_bounds__(kWtaWarps * 32) k_sgm_wta(SgmJob S) {
-    const int lane = threadIdx.x & 31;
-    const size_t p = (size_t)blockIdx.x * kWtaWarps + (threadIdx.x >> 5);
+    constexpr int K = Split<D>::kOther, G = D / K, kWords = K / 4;
+    using Vec = typename Bytes<K>::Vec;
+    const int lane = threadIdx.x & 31, gl = lane % G;
     const size_t np = (size_t)S.w * S.h;
-    if (p >= np) return;  // warp-uniform
-    int sum[J];
+    const size_t p = ((size_t)blockIdx.x * kWtaWarps + (threadIdx.x >> 5)) * (32 / G) + lane / G;
+    const size_t o = min(p, np - 1) * D + gl * K;
+    Vec v[kDirs];
 #pragma unroll
-    for (int j = 0; j < J; ++j) sum[j] = 0;
+    for (int r = 0; r < kDirs; ++r) v[r] = __ldcs(reinterpret_cast<const Vec*>(S.paths + (size_t)r * np * D + o));
+    uint32_t even[kWords], odd[kWords];  // bytes 0 and 2, 1 and 3 of each word
+#pragma unroll
+    for (int j = 0; j < kWords; ++j) even[j] = odd[j] = 0;
 #pragma unroll
     for (int r = 0; r < kDirs; ++r) {
-        int v[J];
-        load_bytes<J>(S.paths + ((size_t)r * np + p) * S.D + lane * J, v);
+        uint32_t w[kWords];
+        memcpy(w, &v[r], sizeof w);
 #pragma unroll
-        for (int j = 0; j < J; ++j) sum[j] += v[j];
+        for (int j = 0; j < kWords; ++j) {
+            even[j] += w[j] & 0x00ff00ffu;
+            odd[j] += (w[j] >> 8) & 0x00ff00ffu;
+        }
     }
     // key = sum << 8 | d: the smallest key is the lowest sum, then the lowest d
-    unsigned key = 0xffffffffu;
+    uint32_t key = 0xffffffffu;
 #pragma unroll
-    for (int j = 0; j < J; ++j) key = min(key, ((unsigned)sum[j] << 8) | (unsigned)(lane * J + j));
-    key = __reduce_min_sync(kFull, key);
-    if (lane == 0) S.disp[p] = (int16_t)(key & 0xff);
+    for (int j = 0; j < kWords; ++j) {
+        const uint32_t d = gl * K + 4 * j;
+        key = min(key, (even[j] << 16) >> 8 | d);
+        key = min(key, (odd[j] << 16) >> 8 | (d + 1));
+        key = min(key, (even[j] >> 16) << 8 | (d + 2));
+        key = min(key, (odd[j] >> 16) << 8 | (d + 3));
+    }
+#pragma unroll
+    for (int o2 = 1; o2 < G; o2 <<= 1) key = min(key, __shfl_xor_sync(kFull, key, o2));
+    if (gl == 0 && p < np) S.disp[p] = (int16_t)(key & 0xff);
 }
 
 int check_sgm(const sff_sgm_params* P) {
@@ -378,17 +360,15 @@ SgmLayout sgm_layout(int w, int h, int D) {
     return L;
 }
 
-template <int J>
+template <int D>
 int launch_sgm(const SgmJob& S, cudaStream_t st) {
     const size_t np = (size_t)S.w * S.h;
-    SFF_LAUNCH(k_sgm_cost<J>, dim3((S.w + kCostSeg - 1) / kCostSeg, S.h), kCostThreads, 0, st, S);
+    SFF_LAUNCH(k_sgm_cost<D>, dim3((S.w + kCostSeg - 1) / kCostSeg, S.h), kCostThreads, 0, st, S);
+    using P = Split<D>;
     const int lines = S.w + S.h - 1;  // the diagonals have the most lines
-    const size_t ring = (size_t)kPathWarps * kRing * S.D;
-    if (ring > 48 * 1024 &&
-        cudaFuncSetAttribute(k_sgm_paths<J>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring) != cudaSuccess)
-        return SFF_ERR_CUDA;
-    SFF_LAUNCH(k_sgm_paths<J>, dim3((lines + kPathWarps - 1) / kPathWarps, 1, kDirs), kPathWarps * 32, ring, st, S);
-    SFF_LAUNCH(k_sgm_wta<J>, dim3((unsigned)((np + kWtaWarps - 1) / kWtaWarps)), kWtaWarps * 32, 0, st, S);
+    SFF_LAUNCH(k_sgm_paths<D>, dim3(2 * P::blocks_across(S.h) + (kDirs - 2) * P::blocks(lines)), 32, 0, st, S);
+    constexpr int kPix = kWtaWarps * 32 / (D / P::kOther);  // pixels per CTA
+    SFF_LAUNCH(k_sgm_wta<D>, dim3((unsigned)((np + kPix - 1) / kPix)), kWtaWarps * 32, 0, st, S);
     return SFF_OK;
 }
 
@@ -435,7 +415,7 @@ extern "C" int sff_sgm(const uint8_t* left_dev, const uint8_t* right_dev, int32_
     cudaStream_t st = (cudaStream_t)stream;
     SFF_LAUNCH(k_sgm_census, dim3((width + kTileX - 1) / kTileX, (height + kTileY - 1) / kTileY, 2),
                dim3(kTileX, kTileY), 0, st, S);
-    const int rc = S.D == 32 ? launch_sgm<1>(S, st) : S.D == 64 ? launch_sgm<2>(S, st)
-                   : S.D == 128 ? launch_sgm<4>(S, st) : launch_sgm<8>(S, st);
+    const int rc = S.D == 32 ? launch_sgm<32>(S, st) : S.D == 64 ? launch_sgm<64>(S, st)
+                   : S.D == 128 ? launch_sgm<128>(S, st) : launch_sgm<256>(S, st);
     return rc != SFF_OK ? rc : launch_status();
 }
