@@ -1644,50 +1644,231 @@ __global__ void __launch_bounds__(fused_threads<L, C, TX, TY>(), fused_min_block
 // replaced only on strictly lower cost), then the random search over every
 // non-empty grid pixel.  In sweep coordinates (a, b) a pixel depends on
 // (a - 1, b) and (a, b - 1) only, so the pixels of one anti-diagonal
-// a + b = t are independent: one CTA per field walks the gw + gh - 1
-// diagonals, a barrier between them.  The critical path is that many
-// dependent cost evaluations per iteration, so this order is an order of
-// magnitude slower per quad than the checkerboard; it exists to reproduce
-// the sequential scan exactly.
-constexpr int kSweepLanes = 2;
-constexpr int kSweepThreads = 1024;
+// a + b = t are independent: one CTA per field walks the diagonals, a barrier
+// between them.  The critical path is that many dependent cost evaluations per
+// iteration, so this order is an order of magnitude slower per quad than the
+// checkerboard; it exists to reproduce the sequential scan exactly.
+//
+// A warp takes a block of 32 / L consecutive rows, L lanes per row, row r one
+// column behind row r - 1, and walks along them on its own: a step's horizontal
+// predecessor is the group's last result, the vertical one the last result of the
+// group above (a shuffle), and the next pixel's state and reference record are
+// loaded a step ahead.  The block's last row goes to the next block's warp through
+// a ring in shared memory, so that no barrier joins the warps and each step waits
+// only for its own loads, not for the slowest of the whole diagonal.  Blocks go
+// round the warps; the last warp's rows reach warp 0's next block through the state
+// in memory (it must not wait for warp 0, which may wait for the warps between
+// them).  A warp thus waits for a column of the block above, or for a ring slot
+// that the block below has not read, and no circle of waits closes; both waits are
+// bounded.  With L = 8 each predecessor has its own four lanes.
+// 256 x 80, both fields: 28.8 ms (a barrier per diagonal, states from memory) ->
+// 15.2 ms.
+constexpr int kSweepWarps = 32, kSweepRing = 64, kSweepSignal = 16;
 
-__global__ void __launch_bounds__(kSweepThreads) k_sweep(const __grid_constant__ Fields F, int n, int dx, int dy) {
-    constexpr int L = kSweepLanes;
-    constexpr int kGroups = kSweepThreads / L;
+// A pixel's state in a ring slot: two 64-bit words, each read and written whole and
+// each carrying the column's tag, so that a reader needs no fence to tell a
+// complete state (a release per column would wait for the warp's stores to global
+// memory).  Tags count the columns that a ring has carried, from 1; a slot's tag
+// differs from the one before by kSweepRing, so 16 bits of it tell them apart.
+// Costs are below 2^24 (three distances of 48 squares of at most 255) or kEmpty.
+__device__ __forceinline__ ulonglong2 sweep_pack(int cost, uint2 v, int tag) {
+    const uint32_t c = cost == kEmpty ? 0xffffffu : (uint32_t)cost;
+    return make_ulonglong2((unsigned long long)v.x << 32 | ((c & 0xffffu) << 16) | (tag & 0xffff),
+                           (unsigned long long)v.y << 32 | ((c >> 16) << 16) | (tag & 0xffff));
+}
+__device__ __forceinline__ bool sweep_unpack(const volatile ulonglong2* slot, int tag, int& cost, uint2& v) {
+    const unsigned long long a = slot->x, b = slot->y;
+    const uint32_t c = ((uint32_t)a >> 16) | ((uint32_t)b & 0xffff0000u);
+    cost = c == 0xffffffu ? kEmpty : (int)c;
+    v = make_uint2((uint32_t)(a >> 32), (uint32_t)(b >> 32));
+    return (a & 0xffffu) == (tag & 0xffffu) && (b & 0xffffu) == (tag & 0xffffu);
+}
+
+// Calls ready() until it holds; false when the limit runs out.
+template <class Ready>
+__device__ __forceinline__ bool sweep_wait(Ready ready, unsigned long long limit_ns) {
+    if (ready()) return true;
+    const unsigned long long t0 = global_ns();
+    for (long long k = 0; k < kMaxPolls; ++k) {
+        if (ready()) return true;
+        if ((k & 63) == 63 && global_ns() - t0 > limit_ns) return false;
+    }
+    return false;
+}
+__device__ __forceinline__ bool sweep_passed(const int* counter, int need) {
+    int v;
+    asm volatile("ld.acquire.cta.shared.s32 %0, [%1];" : "=r"(v) : "r"(smem_addr(counter)) : "memory");
+    return v > need;
+}
+__device__ __forceinline__ void sweep_signal(int* counter, int value) {
+    asm volatile("st.release.cta.shared.s32 [%0], %1;" ::"r"(smem_addr(counter)), "r"(value) : "memory");
+}
+
+template <int L>
+__global__ void __launch_bounds__(32 * kSweepWarps) k_sweep(const __grid_constant__ Fields F, int n, int dx, int dy) {
+    constexpr int P = L == 8 ? 4 : L;  // lanes that share a record
+    constexpr int kRows = 32 / L;      // rows per block
+    __shared__ ulonglong2 s_ring[kSweepWarps][kSweepRing];  // last rows of the blocks, by column
+    __shared__ int s_made, s_read[kSweepWarps];  // columns written by the last warp, read from a warp's ring
     const Field& A = pick(F);
     const Views& V = A.V;
-    const int q = threadIdx.x & (L - 1);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const int q = lane & (P - 1), g = lane / L;
     const unsigned gmask = group_mask<L>();
-    const int grp = threadIdx.x / L;
-    const int gw = A.gw, gh = A.gh;
-    for (int t = 0; t < gw + gh - 1; ++t) {
-        const int b0 = max(0, t - (gw - 1)), b1 = min(gh - 1, t);
-        for (int b = b0 + grp; b <= b1; b += kGroups) {
-            const int a = t - b;
-            const int gx = dx > 0 ? a : gw - 1 - a, gy = dy > 0 ? b : gh - 1 - b;
-            const int x = gx * n, y = gy * n;
-            const size_t si = (size_t)gy * gw + gx;
-            const bool has_a = gx - dx >= 0 && gx - dx < gw, has_b = gy - dy >= 0 && gy - dy < gh;
-            // plain loads: the predecessors were written by this CTA on the
-            // previous diagonal
-            int c = A.cost[si];
-            Vec4 cur = unpack_vec(A.field[si]);
-            const int ca = has_a ? A.cost[si - dx] : kEmpty;
-            const int cb = has_b ? A.cost[si - (size_t)(dy * gw)] : kEmpty;
-            const uint2 wa = has_a ? A.field[si - dx] : make_uint2(0u, 0u);
-            const uint2 wb = has_b ? A.field[si - (size_t)(dy * gw)] : make_uint2(0u, 0u);
-            Slice<L> r;
-            load_slice<L>(V.ref, pix(V.w, x, y), q, r);
-            if (update_pixel<L>(V, r, q, gmask, n, 0, A.key, A.mirror, x, y, 0u, -1, -1, unpack_vec(wa), ca,
-                                unpack_vec(wb), cb, cur, c) &&
-                q == 0) {
-                A.field[si] = pack_vec(cur);
-                A.cost[si] = c;
+    const int gw = A.gw, gh = A.gh, blocks = (gh + kRows - 1) / kRows;
+    const unsigned long long wait_ns = g_wait_limit_ns ? g_wait_limit_ns : kDefaultWaitNs;
+    for (int k = lane; k < kSweepRing; k += 32) s_ring[warp][k] = make_ulonglong2(0ull, 0ull);
+    if (lane == 0) s_read[warp] = 0;
+    if (threadIdx.x == 0) s_made = 0;
+    __syncthreads();
+    int made = 0, read = 0;  // last seen of s_made / this warp's s_read
+    bool live = true;
+    for (int blk = warp, round = 0; blk < blocks && live; blk += warps, ++round) {
+        const int from = (warp + warps - 1) % warps;         // the warp of the block above
+        const int base = round * gw;                          // columns this warp's ring has carried before
+        const int base_from = (blk - 1) / warps * gw;         // ... and the ring of the block above
+        const int b = blk * kRows + g;  // this group's row in sweep order
+        const bool mine = b < gh;
+        const int gy = mine ? (dy > 0 ? b : gh - 1 - b) : 0, y = gy * n;
+        const size_t row = (size_t)gy * gw;
+        auto col = [&](int a) { return dx > 0 ? a : gw - 1 - a; };
+        // the next pixel: its state and reference record (the record's norm is
+        // computed when its turn comes: here it would wait for the load)
+        int c1 = kEmpty;
+        uint2 w1 = make_uint2(0u, 0u);
+        Slice<P> r1;
+        auto fetch = [&](int a) {
+            if (!mine || a < 0 || a >= gw) return;
+            c1 = A.cost[row + col(a)];
+            w1 = A.field[row + col(a)];
+            const size_t i = pix(V.w, col(a) * n, y);
+#pragma unroll
+            for (int k = 0; k < Slice<P>::kChunks; ++k)
+                r1.c[k] = q + k * P < 3 ? chunk_of(V.ref, i, q + k * P) : make_int4(0, 0, 0, 0);
+        };
+        // this lane's chunk of the other views' records (L = 8)
+        const unsigned stride = V.ref.rs * (unsigned)sizeof(int4);
+        const char* pt = reinterpret_cast<const char*>(V.tmp.f + min(q, 2) * V.tmp.cs);
+        const char* ps = reinterpret_cast<const char*>(V.ste.f + min(q, 2) * V.ste.cs);
+        const char* pc = reinterpret_cast<const char*>(V.crs.f + min(q, 2) * V.crs.cs);
+        fetch(0);
+        int c = kEmpty;  // the group's last pixel: its horizontal predecessor
+        uint2 wc = make_uint2(0u, 0u);
+        for (int t = 0; t < gw + kRows - 1; ++t) {
+            const int a = t - g;
+            const bool act = mine && a >= 0 && a < gw;
+            const int ca = c;
+            const uint2 wa = wc;
+            // the vertical predecessor: the group above at this column
+            int cb = __shfl_up_sync(0xffffffffu, c, L);
+            uint2 wb = make_uint2(__shfl_up_sync(0xffffffffu, wc.x, L), __shfl_up_sync(0xffffffffu, wc.y, L));
+            if (blk > 0 && t < gw) {  // row 0 of the block: from the block above
+                if (warp > 0) {
+                    if (g == 0)
+                        live = sweep_wait([&]() { return sweep_unpack(&s_ring[from][(base_from + t) % kSweepRing], base_from + t + 1, cb, wb); },
+                                          wait_ns);
+                    if (!__all_sync(0xffffffffu, live)) {
+                        live = false;
+                        break;
+                    }
+                    if (lane == 0 && (t % kSweepSignal == kSweepSignal - 1 || t == gw - 1))
+                        sweep_signal(&s_read[from], base_from + t + 1);
+                } else {
+                    if (made <= base_from + t) {
+                        if (lane == 0) live = sweep_wait([&]() { return sweep_passed(&s_made, base_from + t); }, wait_ns);
+                        live = __shfl_sync(0xffffffffu, (int)live, 0);
+                        if (!live) break;
+                        made = __shfl_sync(0xffffffffu, *(volatile int*)&s_made, 0);
+                        __syncwarp();
+                    }
+                    if (g == 0) {
+                        const size_t up = row - (ptrdiff_t)dy * gw + col(t);
+                        cb = A.cost[up];
+                        wb = A.field[up];
+                    }
+                }
+            } else if (g == 0) {
+                cb = kEmpty;
+            }
+            if (act) {
+                const int gx = col(a), x = gx * n;
+                c = c1;
+                const uint2 w0 = w1;
+                Slice<P> r = r1;
+                fetch(a + 1);
+                r.nrm = 0;
+#pragma unroll
+                for (int k = 0; k < Slice<P>::kChunks; ++k) r.nrm = dot4(r.c[k], r.c[k], r.nrm);
+                bool changed = false;
+                if constexpr (L == 8) {
+                    // as update_pixel, lanes 0-3 scoring the horizontal
+                    // predecessor's vector, lanes 4-7 the vertical one's
+                    auto same = [](uint2 p, uint2 q) { return p.x == q.x && p.y == q.y; };
+                    wc = w0;
+                    const bool own = c != kEmpty;
+                    const bool do_a = ca != kEmpty && !(own && same(wa, w0));
+                    const bool do_b = cb != kEmpty && !(own && same(wb, w0)) && !(ca != kEmpty && same(wb, wa));
+                    if (do_a || do_b) {
+                        const bool vertical = lane & 4;
+                        // the three views' chunks in flight together; lane 3 of
+                        // four repeats chunk 2 and adds nothing
+                        const Vec4 v = unpack_vec(vertical ? wb : wa);
+                        const int tx = clampi(x + v.u, 0, V.w - 1), ty = clampi(y + v.v, 0, V.h - 1);
+                        const int sx = clampi(x - V.sigma * v.d0, 0, V.w - 1);
+                        const int cx = clampi(x + v.u - V.sigma * v.d1, 0, V.w - 1);
+                        const unsigned rt = (unsigned)ty * V.w, rs = (unsigned)y * V.w;
+                        const int4 vt = __ldg(reinterpret_cast<const int4*>(pt + (size_t)(rt + tx) * stride)),
+                                   vs = __ldg(reinterpret_cast<const int4*>(ps + (size_t)(rs + sx) * stride)),
+                                   vc = __ldg(reinterpret_cast<const int4*>(pc + (size_t)(rt + cx) * stride));
+                        const int dot = dot4(r.c[0], vt, dot4(r.c[0], vs, dot4(r.c[0], vc, 0)));
+                        const int nrm = dot4(vt, vt, dot4(vs, vs, dot4(vc, vc, 3 * r.nrm)));
+                        const int sum = group_sum<4>(q < 3 ? nrm - 2 * dot : 0, gmask),
+                                  other = __shfl_xor_sync(gmask, sum, 4);
+                        const int na = vertical ? other : sum, nv = vertical ? sum : other;
+                        if (do_a && na < c) {
+                            c = na;
+                            wc = wa;
+                            changed = true;
+                        }
+                        if (do_b && nv < c) {
+                            c = nv;
+                            wc = wb;
+                            changed = true;
+                        }
+                    }
+                } else {
+                    Vec4 cur = unpack_vec(w0);
+                    changed = update_pixel<P>(V, r, q, gmask, n, 0, A.key, A.mirror, x, y, 0u, -1, -1, unpack_vec(wa), ca,
+                                              unpack_vec(wb), cb, cur, c);
+                    wc = pack_vec(cur);
+                }
+                if (changed && (lane & (L - 1)) == 0) {
+                    A.field[row + gx] = wc;
+                    A.cost[row + gx] = c;
+                }
+            }
+            const int al = t - (kRows - 1);  // the last row's column
+            if (al < 0 || blk + 1 >= blocks) continue;
+            if (warp + 1 < warps) {
+                if (base + al - kSweepRing >= read) {  // the slot's last column may not have been read
+                    if (lane == 0)
+                        live = sweep_wait([&]() { return sweep_passed(&s_read[warp], base + al - kSweepRing); }, wait_ns);
+                    live = __shfl_sync(0xffffffffu, (int)live, 0);
+                    if (!live) break;
+                    read = __shfl_sync(0xffffffffu, *(volatile int*)&s_read[warp], 0);
+                }
+                if (lane == 32 - L) {
+                    const ulonglong2 w = sweep_pack(c, wc, base + al + 1);
+                    volatile ulonglong2* slot = &s_ring[warp][(base + al) % kSweepRing];
+                    slot->x = w.x;
+                    slot->y = w.y;
+                }
+            } else if (lane == 32 - L && (al % kSweepSignal == kSweepSignal - 1 || al == gw - 1)) {
+                sweep_signal(&s_made, base + al + 1);
             }
         }
-        __syncthreads();
     }
+    if (!live && lane == 0) note_timeout();
 }
 
 // The random search of iteration `it` over every non-empty grid pixel, in
@@ -2501,7 +2682,13 @@ int run_fields(const FieldSpec* spec, int nf, const sff_params& P, const sff_tun
             }
             dim3 gr((mgw + 63) / 64, mgh, nf);
             for (int it = 0; it < I; ++it) {
-                SFF_LAUNCH(k_sweep, dim3(1, 1, nf), kSweepThreads, 0, st, F, n, kDirs[it % 4][0], kDirs[it % 4][1]);
+                // the most lanes per row that leave every block a warp
+                const int lanes = mgh <= 4 * kSweepWarps ? 8 : mgh <= 8 * kSweepWarps ? 4 : 2;
+                const int threads = 32 * std::min(kSweepWarps, (mgh * lanes + 31) / 32);
+                const dim3 gs(1, 1, nf);
+                if (lanes == 8) SFF_LAUNCH(k_sweep<8>, gs, threads, 0, st, F, n, kDirs[it % 4][0], kDirs[it % 4][1]);
+                else if (lanes == 4) SFF_LAUNCH(k_sweep<4>, gs, threads, 0, st, F, n, kDirs[it % 4][0], kDirs[it % 4][1]);
+                else SFF_LAUNCH(k_sweep<2>, gs, threads, 0, st, F, n, kDirs[it % 4][0], kDirs[it % 4][1]);
                 SFF_LAUNCH(k_random_search, gr, 256, 0, st, F, n, s, it);
             }
             prev = cur;
