@@ -98,8 +98,11 @@ typedef struct sff_params {
  *              fit 1024; min_ctas 0.
  * Scale 0 takes (lanes_per_pixel, slots, tile_x, tile_y, min_ctas).  Scale
  * s >= 1 takes coarse[s - 1] = {lanes, slots, tile_x, tile_y, min_ctas}; all zero means
- * derived from the grid size: (1, 4, 16, 8, 0) below 200 grid pixels per SM
- * over all fields of the launch, else (1, 0, 32, 16, 0).
+ * derived from the grid pixels per SM over all fields of the launch: (1, 4, 16, 8,
+ * 0) below 200, (1, 0, 32, 8, 7) from 1280 to 1792, else (1, 0, 32, 8, 0).
+ * A tuning equal to sff_default_tuning's leaves every choice of the iterations to
+ * the library, scale 0 and the schedules (pair_fields, alternate_order, pdl, fuse)
+ * included: derived from the grid sizes in the same way.
  * sff_tuning_supported() checks a setting. */
 typedef struct sff_tuning {
     int32_t lanes_per_pixel; /* threads that share one pixel's feature loads */

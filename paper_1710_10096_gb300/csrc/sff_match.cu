@@ -2485,25 +2485,70 @@ bool tuning_valid(const sff_tuning& t) {
     return true;
 }
 
-// Variant of the iteration kernel at one scale.  Scale 0 takes the tuned
-// variant, a coarser scale its tuning entry when one is given.  Otherwise it
-// is chosen by the number of grid pixels per SM over all fields: a coarse
-// scale is latency-bound (few grid pixels per SM, each a chain of dependent
-// feature loads).  Measured per launch on the 1242x375 driving quad (both
-// fields): at scale 1 (1536 pixels per SM) and scale 2 (385) one lane per
-// pixel on 32 x 16 tiles was fastest of all 38 variants (23.2, 12.9 us), at
-// scale 3 (96) the latency form with a slot per candidate on 16 x 8 tiles
-// (8.9 us against 13.3).  Every variant gives the same result.
-constexpr int kSmCount = 152;
-constexpr long kPixPerSmSlots = 200;
+// How one scale's iterations run.
+struct ScalePlan {
+    const IterVariant* v;
+    bool pdl, fuse, alternate, pair;
+};
 
-const IterVariant* variant_for_scale(const sff_tuning& t, int s, const int* gw, const int* gh, int nf) {
-    if (s == 0) return find_variant(t.lanes_per_pixel, t.slots, t.tile_x, t.tile_y, t.min_ctas);
-    const int32_t* c = t.coarse[s - 1];
-    if ((c[0] | c[1] | c[2] | c[3] | c[4]) != 0) return find_variant(c[0], c[1], c[2], c[3], c[4]);
-    long px = 0;
-    for (int k = 0; k < nf; ++k) px += (long)gw[k] * gh[k];
-    return px / kSmCount < kPixPerSmSlots ? find_variant(1, 4, 16, 8, 0) : find_variant(1, 0, 32, 16, 0);
+// The variant derived from the grid pixels per SM over all fields of a launch.
+// Measured with every setting below on whole stages (default parameters,
+// 160 x 60 to 1917 x 1083 and the 32-quad batch; us with the other choice / with
+// this one):
+//   - below 200 (a coarse scale, latency-bound): the latency form with a slot per
+//     candidate on 16 x 8 tiles (1242 x 375 scale 3, 97 a SM: 13.3 / 8.9 per
+//     iteration; at 269 a SM it loses to the throughput form, 512 x 160: 542 / 508);
+//   - from 1280 to 1792: 32 x 8 tiles compiled for 7 resident CTAs, which then fit
+//     one wave (1242 x 375 scale 1: 1395 / 1370 the stage);
+//   - else 32 x 8 tiles (32 x 16 before: 1242 x 375 scale 0 1630 / 1434, 1917 x
+//     1083 7207 / 6361 the stage, the batch 26.6 / 22.8 ms).
+// Every variant gives the same result.
+constexpr int kSmCount = 152;
+constexpr long kPixPerSmSlots = 200, kPixPerSmWaveLo = 1280, kPixPerSmWaveHi = 1792;
+
+const IterVariant* derived_variant(long px) {
+    const long per = px / kSmCount;
+    if (per < kPixPerSmSlots) return find_variant(1, 4, 16, 8, 0);
+    return find_variant(1, 0, 32, 8, per >= kPixPerSmWaveLo && per < kPixPerSmWaveHi ? 7 : 0);
+}
+
+bool default_tuning(const sff_tuning& t) {
+    sff_tuning d;
+    sff_default_tuning(&d);
+    return memcmp(&t, &d, sizeof t) == 0;
+}
+
+// Scale s over px grid pixels of the launch's fields.  The default tuning leaves
+// everything to the library; with any other, scale 0 takes the tuned variant, a
+// coarser scale its entry when one is given, and the schedule is the tuning's.
+// The library's schedule: the scales below the slot limit fused into one
+// cooperative launch (256 x 80 415 / 396, 512 x 160 508 / 491 us the stage), the
+// others as dependent launches (1242 x 375 1732 / 1630; the launches' gaps); a
+// quad's two fields side by side and, where the four images' records of the grid
+// exceed half of L2, every other launch backwards (together 1395 / 1349 and, 1917 x
+// 1083, 6324 / 5901).
+constexpr double kAlternateBytes = 64e6;
+
+ScalePlan plan_scale(const sff_tuning& t, bool derive, int s, long px) {
+    ScalePlan p;
+    if (derive) {
+        p.v = derived_variant(px);
+        p.fuse = s > 0 && p.v->slots > 0;
+        if (s == 0 && p.v->slots > 0) p.v = find_variant(1, 0, 32, 8, 0);  // 256 x 80: 597 / 524 us
+        p.pdl = !p.fuse;
+        p.alternate = !p.fuse && 2.0 * kFeat * (double)px > kAlternateBytes;
+        p.pair = true;
+        return p;
+    }
+    const int32_t* c = s > 0 ? t.coarse[s - 1] : nullptr;
+    p.v = s == 0 ? find_variant(t.lanes_per_pixel, t.slots, t.tile_x, t.tile_y, t.min_ctas)
+          : (c[0] | c[1] | c[2] | c[3] | c[4]) != 0 ? find_variant(c[0], c[1], c[2], c[3], c[4])
+                                                    : derived_variant(px);
+    p.pdl = (t.pdl >> s) & 1;
+    p.fuse = (t.fuse >> s) & 1;
+    p.alternate = (t.alternate_order >> s) & 1;
+    p.pair = t.pair_fields != 0;
+    return p;
 }
 
 int coarse_gq(int w, int h, const sff_params& p) {
@@ -2571,6 +2616,7 @@ bool knn_smem_ready() {
 int run_fields(const FieldSpec* spec, int nf, const sff_params& P, const sff_tuning& T, cudaStream_t st,
                bool sequential, const cudaEvent_t* scale_ready, const ForkHook* fork_hook) {
     if (!tuning_valid(T) || nf < 1 || nf > kMaxFields) return SFF_ERR_ARG;
+    const bool derive = default_tuning(T);
     const int S = P.num_scales, I = P.iterations;
     static const int kDirs[4][2] = {{1, 1}, {-1, -1}, {1, -1}, {-1, 1}};
     static Fields F;  // host staging of the kernel parameter (copied at each launch)
@@ -2723,15 +2769,18 @@ int run_fields(const FieldSpec* spec, int nf, const sff_params& P, const sff_tun
                 ggw = std::max(ggw, gw[k]);
                 ggh = std::max(ggh, gh[k]);
             }
-            const IterVariant* sv = variant_for_scale(T, s, gw + f0, gh + f0, f1 - f0);
+            long px = 0;
+            for (int k = f0; k < f1; ++k) px += (long)gw[k] * gh[k];
+            const ScalePlan plan = plan_scale(T, derive, s, px);
+            const IterVariant* sv = plan.v;
             // pairs: every field f0 + 2j, f0 + 2j + 1 one quad's two fields
-            bool pair = T.pair_fields != 0 && ((f1 - f0) & 1) == 0;
+            bool pair = plan.pair && ((f1 - f0) & 1) == 0;
             for (int k = f0; pair && k < f1; k += 2)
                 pair = spec[k + 1].width == spec[k].width && spec[k + 1].height == spec[k].height &&
                        spec[k + 1].ref == spec[k].crs;
             const unsigned tiles_x = (ggw + sv->tx - 1) / sv->tx;
             dim3 gi(pair ? 2 * tiles_x : tiles_x, (ggh + sv->ty - 1) / sv->ty, pair ? (f1 - f0) / 2 : f1 - f0);
-            const bool fuse = ((T.fuse >> s) & 1) != 0 && I > 0;
+            const bool fuse = plan.fuse && I > 0;
             if (I > 0 && ::sff::profiling()) ::sff::profile_mark(kIterNames[s], st, false);
             if (fuse) {
                 // one cooperative launch for all iterations (a variant with a
@@ -2779,7 +2828,7 @@ int run_fields(const FieldSpec* spec, int nf, const sff_params& P, const sff_tun
                     F.f[k].cost_out = Bc[in ^ 1][k];
                 }
                 IterStep H{n,      s,  kDirs[it % 4][0], kDirs[it % 4][1], it, it == I - 1, f0, pair ? 1 : 0,
-                           ((T.alternate_order >> s) & 1) ? (it & 1) : 0, inherit && it == 0 ? 1 : 0};
+                           plan.alternate ? (it & 1) : 0, inherit && it == 0 ? 1 : 0};
                 if (tv) {
                     // TMA-staged reference records (scale 0)
                     cudaLaunchConfig_t cfg = {};
@@ -2791,9 +2840,9 @@ int run_fields(const FieldSpec* spec, int nf, const sff_params& P, const sff_tun
                     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
                     attr[0].val.programmaticStreamSerializationAllowed = 1;
                     cfg.attrs = attr;
-                    cfg.numAttrs = ((T.pdl >> s) & 1) ? 1 : 0;
+                    cfg.numAttrs = plan.pdl ? 1 : 0;
                     if (cudaLaunchKernelEx(&cfg, tv->k, F, H, RM) != cudaSuccess) return SFF_ERR_CUDA;
-                } else if ((T.pdl >> s) & 1) {
+                } else if (plan.pdl) {
                     // scheduled while the previous iteration's last CTAs run;
                     // its CTAs wait in griddepcontrol.wait until it is done
                     cudaLaunchConfig_t cfg = {};
