@@ -2523,19 +2523,20 @@ bool default_tuning(const sff_tuning& t) {
 // coarser scale its entry when one is given, and the schedule is the tuning's.
 // The library's schedule: the scales below the slot limit fused into one
 // cooperative launch (256 x 80 415 / 396, 512 x 160 508 / 491 us the stage), the
-// others as dependent launches (1242 x 375 1732 / 1630; the launches' gaps); a
-// quad's two fields side by side and, where the four images' records of the grid
+// others as dependent launches (1242 x 375 1732 / 1630; the launches' gaps), but not
+// in a captured graph, whose gaps are short and where they hold up the features'
+// stream (the batch 20.9 without, 23.4 ms with them); a quad's two fields side by side and, where the four images' records of the grid
 // exceed half of L2, every other launch backwards (together 1395 / 1349 and, 1917 x
 // 1083, 6324 / 5901).
 constexpr double kAlternateBytes = 64e6;
 
-ScalePlan plan_scale(const sff_tuning& t, bool derive, int s, long px) {
+ScalePlan plan_scale(const sff_tuning& t, bool derive, bool capturing, int s, long px) {
     ScalePlan p;
     if (derive) {
         p.v = derived_variant(px);
         p.fuse = s > 0 && p.v->slots > 0;
         if (s == 0 && p.v->slots > 0) p.v = find_variant(1, 0, 32, 8, 0);  // 256 x 80: 597 / 524 us
-        p.pdl = !p.fuse;
+        p.pdl = !p.fuse && !capturing;
         p.alternate = !p.fuse && 2.0 * kFeat * (double)px > kAlternateBytes;
         p.pair = true;
         return p;
@@ -2617,6 +2618,8 @@ int run_fields(const FieldSpec* spec, int nf, const sff_params& P, const sff_tun
                bool sequential, const cudaEvent_t* scale_ready, const ForkHook* fork_hook) {
     if (!tuning_valid(T) || nf < 1 || nf > kMaxFields) return SFF_ERR_ARG;
     const bool derive = default_tuning(T);
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    const bool capturing = cudaStreamIsCapturing(st, &capture) == cudaSuccess && capture != cudaStreamCaptureStatusNone;
     const int S = P.num_scales, I = P.iterations;
     static const int kDirs[4][2] = {{1, 1}, {-1, -1}, {1, -1}, {-1, 1}};
     static Fields F;  // host staging of the kernel parameter (copied at each launch)
@@ -2771,7 +2774,7 @@ int run_fields(const FieldSpec* spec, int nf, const sff_params& P, const sff_tun
             }
             long px = 0;
             for (int k = f0; k < f1; ++k) px += (long)gw[k] * gh[k];
-            const ScalePlan plan = plan_scale(T, derive, s, px);
+            const ScalePlan plan = plan_scale(T, derive, capturing, s, px);
             const IterVariant* sv = plan.v;
             // pairs: every field f0 + 2j, f0 + 2j + 1 one quad's two fields
             bool pair = plan.pair && ((f1 - f0) & 1) == 0;
