@@ -624,7 +624,8 @@ int sff_device_status(void* stream, int32_t reset);
 /* Failure injection for tests of the device-side error path (no counterpart
  * in the paper).  step >= 0: in every later launch of the temporal K-NN
  * kernel the thread that issues the tensor-core MMAs stops before the MMAs of
- * that step (tile visit; 2 per candidate tile) and issues nothing further, so
+ * that step (visit of 128 candidates; each is visited twice, two visits at a
+ * time) and issues nothing further, so
  * the waits on that step's results run out; nothing issued is left in
  * flight.  step = -1: off.  wait_limit_us > 0 sets the time limit of every
  * bounded device wait (drains: ten times it); 0 restores the default of 1 s.

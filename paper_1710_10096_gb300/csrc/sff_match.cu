@@ -103,31 +103,34 @@ __device__ __forceinline__ const Field& pick(const Fields& F) { return F.f[block
 // distance whatever the order of its sums.  K = 54 is padded to 64.
 //
 // Operands sit in global memory already in the tcgen05 "no swizzle,
-// K-major" shared-memory layout, 128 rows per 16 KB tile: core matrix
+// K-major" shared-memory layout, 128 query or 256 candidate rows per tile: core matrix
 // (row group m, K group k) of 8 rows x 8 bf16 at byte
-//     k * kTcKGroupStride + m * 128 + (row % 8) * 16 + (col % 8) * 2,
+//     k * 16 * rows + m * 128 + (row % 8) * 16 + (col % 8) * 2,
 // so one bulk copy moves a tile.
-constexpr int kTcRows = 128;                        // candidates per tile (M) = queries per CTA (N)
+constexpr int kTcRows = 128;                        // queries per CTA (M)
+constexpr int kTcCand = 256;                        // candidates per tile (N)
 constexpr int kTcK = 64;                            // augmented row length (bf16)
-constexpr int kTcTileBytes = kTcRows * kTcK * 2;    // 16 KB
-constexpr int kTcKGroupStride = kTcRows * 16;       // bytes between K groups of 8 columns
-constexpr int kTcStages = 6;                        // candidate tiles in shared memory
-constexpr int kTcAcc = 4;                           // fp32 accumulators in tensor memory
+constexpr int kTcQueryBytes = kTcRows * kTcK * 2;   // 16 KB
+constexpr int kTcTileBytes = kTcCand * kTcK * 2;    // 32 KB
+constexpr int kTcQueryGroup = kTcRows * 16;         // bytes between K groups of 8 columns
+constexpr int kTcTileGroup = kTcCand * 16;
+constexpr int kTcStages = 4;                        // candidate tiles in shared memory
+constexpr int kTcAcc = 2;                           // fp32 accumulators in tensor memory
 constexpr int kTcScanWarps = 16;                    // warps reading the accumulators
-constexpr int kTcScanCols = kTcRows * 4 / kTcScanWarps;  // query columns per scanning warp (32)
+constexpr int kTcScanCols = 32;                     // columns per tensor-memory load (two per warp and tile)
 constexpr int kTcMmaWarp = kTcScanWarps;            // issues the MMAs
 constexpr int kTcTmaWarp = kTcScanWarps + 1;        // issues the bulk copies
 constexpr int kTcThreads = (kTcScanWarps + 2) * 32;
-static_assert(kTcScanCols == 32, "one 32-column TMEM load per warp and step");
-constexpr int kTcCols = kTcAcc * kTcRows;           // TMEM columns (all 512)
+static_assert(kTcScanWarps == 16 && 8 * kTcScanCols == kTcCand, "4 lane groups x 4 column quarters");
+constexpr int kTcCols = kTcAcc * kTcCand;           // TMEM columns (all 512)
 // instruction descriptor, kind::f16: fp32 D (bits 4-5 = 1), bf16 A (7-9 = 1)
 // and B (10-12 = 1), both K-major, N >> 3 at bit 17, M >> 4 at bit 24
-constexpr uint32_t kTcIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTcRows >> 3) << 17) |
+constexpr uint32_t kTcIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTcCand >> 3) << 17) |
                               ((uint32_t)(kTcRows >> 4) << 24);
 // shared memory: queries | candidate stages | scratch (bucket minima, then
 // the per-lane-group candidate buffers) | limits | counts | barriers
 constexpr int kTcOffQ = 0;
-constexpr int kTcOffA = kTcOffQ + kTcTileBytes;
+constexpr int kTcOffA = kTcOffQ + kTcQueryBytes;
 constexpr int kTcOffScratch = kTcOffA + kTcStages * kTcTileBytes;
 constexpr int kTcMinStride = kTcRows + 1;                         // padded row: conflict-free both ways
 constexpr int kTcScratchBytes = kTcRows * kTcMinStride * 4;      // [query][bucket] minima
@@ -141,6 +144,7 @@ constexpr unsigned kInfBits = 0x7f800000u;   // +inf
 constexpr int kMaxFiniteBits = 0x7f7fffff;   // largest finite float
 
 __host__ __device__ __forceinline__ int tc_rows(int gq) { return (gq + kTcRows - 1) / kTcRows * kTcRows; }
+__host__ __device__ __forceinline__ int tc_cand_rows(int gq) { return (gq + kTcCand - 1) / kTcCand * kTcCand; }
 
 // Writes the augmented bf16 rows of the reference (role 0: queries) and
 // temporal (role 1: candidates) coarsest-grid points; rows past gq are zero.
@@ -149,7 +153,7 @@ __host__ __device__ __forceinline__ int tc_rows(int gq) { return (gq + kTcRows -
 __global__ void k_gather_grid(const __grid_constant__ Fields F, int n) {
     const Field& A = pick(F);
     const int role = blockIdx.y;
-    const int rows = tc_rows(A.gq);
+    const int rows = role ? tc_cand_rows(A.gq) : tc_rows(A.gq);
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (role >= 2) {
         // roles 2, 3: compact int8 records of the stereo and cross images
@@ -192,9 +196,9 @@ __global__ void k_gather_grid(const __grid_constant__ Fields F, int n) {
         const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
         w[k] = *reinterpret_cast<const uint32_t*>(&h);
     }
-    uint8_t* base = A.tk + (size_t)role * rows * (kTcK * 2);
-    const size_t off = (size_t)(r / kTcRows) * kTcTileBytes + (size_t)kg * kTcKGroupStride + ((r % kTcRows) >> 3) * 128 +
-                       (r & 7) * 16;
+    uint8_t* base = A.tk + (role ? (size_t)tc_rows(A.gq) * (kTcK * 2) : 0);
+    const int tile = role ? kTcCand : kTcRows;
+    const size_t off = (size_t)(r / tile) * tile * (kTcK * 2) + (size_t)kg * tile * 16 + ((r % tile) >> 3) * 128 + (r & 7) * 16;
     *reinterpret_cast<uint4*>(base + off) = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
@@ -215,71 +219,27 @@ __device__ __forceinline__ void note_timeout() {
     atomicOr(&g_match_status, kStatusTimeout);
 }
 
-// Reduces a buffer of `cnt` (<= kTcCap) candidates of one (lane group,
-// query) to its 8 best in (distance, index) order, at the front in order;
-// returns the limit they imply: the float bits just below the 8th distance
-// (a candidate that comes later has a larger index, so it needs a strictly
-// smaller distance).  The whole warp calls it.
-__device__ __forceinline__ int tc_compact(int2* buf, int cnt, int lane) {
-    const int2 x = lane < cnt ? buf[lane] : make_int2(0x7fffffff, 0x7fffffff);
-    int rank = 0;
-#pragma unroll
-    for (int m = 0; m < kTcCap; ++m) {
-        const int od = __shfl_sync(0xffffffffu, x.x, m), oi = __shfl_sync(0xffffffffu, x.y, m);
-        rank += m < cnt && (od < x.x || (od == x.x && oi < x.y));
-    }
-    __syncwarp();
-    if (lane < cnt && rank < 8) buf[rank] = x;
-    const unsigned at7 = __ballot_sync(0xffffffffu, lane < cnt && rank == 7);
-    const int d7 = __shfl_sync(0xffffffffu, x.x, at7 ? __ffs(at7) - 1 : 0);
-    __syncwarp();
-    return at7 ? __float_as_int((float)d7) - 1 : 0x7fffffff;
-}
-
-// Appends the lanes of `enter` (lane order = increasing candidate index) to
-// a full-enough buffer, compacting it to its 8 best whenever it fills;
-// every compaction lowers the limit, which drops the lanes no longer
-// within it.  Rare: only when a column brings more candidates than the
-// buffer holds (ties at the bound).
-__device__ __noinline__ void tc_append_slow(unsigned enter, int mine, int idx, int cnt, int2* buf, int* cntp, int* limp,
-                                            int lane) {
-    const unsigned lt = (1u << lane) - 1u;
-    while (enter) {
-        const int room = kTcCap - cnt;
-        const bool mine_in = (enter >> lane) & 1u;
-        const int rank = __popc(enter & lt);
-        if (mine_in && rank < room) buf[cnt + rank] = make_int2((int)__int_as_float(mine), idx);
-        const int took = min(room, __popc(enter));
-        enter = __ballot_sync(0xffffffffu, mine_in && rank >= room);
-        cnt += took;
-        __syncwarp();
-        if (cnt == kTcCap) {
-            const int nl = tc_compact(buf, cnt, lane);
-            cnt = 8;
-            const int l = min(*limp, nl);
-            __syncwarp();
-            if (lane == 0) *limp = l;
-            enter &= __ballot_sync(0xffffffffu, mine <= l);
+// Buffered candidates of one lane (its query, its 32 columns of each tile): entry
+// e at buf[e ^ (query mod kTcCap)], so that lanes appending at once use different
+// banks.  Reduces the cnt (> 8) entries to the 8 best in (distance, index) order
+// and returns the limit they imply: the float bits just below the 8th distance (a
+// candidate that comes later has a larger index, so it needs a strictly smaller
+// distance).  Rare: only when candidates tie or crowd at the bound.
+__device__ __noinline__ int tc_compact(int2* buf, int swizzle, int cnt) {
+    int worst = 0;
+    for (;; --cnt) {
+        worst = 0;
+        int2 w = buf[swizzle];
+        for (int e = 1; e < cnt; ++e) {
+            const int2 x = buf[e ^ swizzle];
+            if (x.x > w.x || (x.x == w.x && x.y > w.y)) {
+                w = x;
+                worst = e;
+            }
         }
+        if (cnt == 8) return __float_as_int((float)w.x) - 1;
+        buf[worst ^ swizzle] = buf[(cnt - 1) ^ swizzle];
     }
-    __syncwarp();
-    if (lane == 0) *cntp = cnt;
-    __syncwarp();
-}
-
-// v[j] for a warp-uniform j in 0..31: a tree of selects on the bits of j
-// (31 selects; a register array cannot be indexed at run time).
-__device__ __forceinline__ uint32_t select32(const uint32_t (&v)[32], int j) {
-    uint32_t a[16];
-#pragma unroll
-    for (int k = 0; k < 16; ++k) a[k] = (j & 1) ? v[2 * k + 1] : v[2 * k];
-#pragma unroll
-    for (int w = 8; w >= 1; w >>= 1) {
-        const bool hi = (j & (32 / (2 * w))) != 0;
-#pragma unroll
-        for (int k = 0; k < w; ++k) a[k] = hi ? a[2 * k + 1] : a[2 * k];
-    }
-    return a[0];
 }
 
 // Bounded wait on an accumulator for a whole warp (lane 0 polls); false
@@ -287,6 +247,7 @@ __device__ __forceinline__ uint32_t select32(const uint32_t (&v)[32], int j) {
 // already failed.
 __device__ __forceinline__ bool scan_wait(uint64_t* bar, unsigned parity, volatile int* fail, int lane,
                                           unsigned long long wait_ns) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
     bool ok = true;
     if (lane == 0) ok = mbar_wait(bar, parity, wait_ns) && *fail == 0;
     const bool failed = __shfl_sync(0xffffffffu, (int)ok, 0) == 0;
@@ -297,35 +258,43 @@ __device__ __forceinline__ bool scan_wait(uint64_t* bar, unsigned parity, volati
     return !failed;
 }
 
-// Reads the warp's 32 candidates x 32 queries of accumulator b and releases it.
-__device__ __forceinline__ void scan_load(uint32_t trow, int b, uint32_t (&v)[32], uint64_t* bar_free, int lane) {
-    tc_fence_after();
-    tmem_ld32(trow + (uint32_t)(b * kTcRows), v, 0);
+// Reads 32 queries x 32 candidates of an accumulator from column tcol on; with
+// `last` the warp has read its part and releases the accumulator.
+__device__ __forceinline__ void scan_load(uint32_t tcol, uint32_t (&v)[32], bool last, uint64_t* bar_free, int lane) {
+    tmem_ld32(tcol, v, 0);
     tmem_ld_wait(v);
+    if (!last) return;
     tc_fence_before();
     __syncwarp();
-    if (lane == 0) mbar_arrive(&bar_free[b]);
+    if (lane == 0) mbar_arrive(bar_free);
 }
 
 // Temporal K-NN of the kTcRows queries of one CTA over every candidate of
 // the field, exact in (distance, candidate index) order.
 //
 // Warp 17 streams candidate tiles into kTcStages shared-memory stages with
-// bulk copies; warp 16 issues, per tile, four M128 N128 K16 MMAs into one of
-// kTcAcc TMEM accumulators (rows = candidates, columns = queries) and
+// bulk copies; warp 16 issues, per tile, four M128 N256 K16 MMAs into one of
+// kTcAcc TMEM accumulators (rows = queries, columns = candidates) and
 // commits them to the accumulator's and the stage's barriers.  Warps 0-15
-// read an accumulator (warp w: lanes 32 (w % 4).., query columns
-// 32 (w / 4)..), release it and scan it while the MMAs of the next tiles
+// read an accumulator (warp w: lanes 32 (w % 4).., candidate columns
+// 64 (w / 4)..), release it and scan it while the MMAs of the next tile
 // run.  Every tile is visited twice:
-//   pass 1: each lane keeps, per query, the minimum over its candidates
-//           ("bucket" = candidate index mod 128); the 8th smallest of the
-//           128 bucket minima is reached by 8 distinct candidates, so it
-//           bounds the query's 8th-nearest distance from above -- exactly
-//           it, unless two of the 8 nearest share a bucket;
-//   pass 2: candidates within the bound are appended to a buffer per lane
-//           group and query (compacted to its 8 best if it fills, which
-//           lowers the limit); the four buffers of a query are merged at
-//           the end.
+//   pass 1: each lane keeps 32 minima ("buckets"), each over two of its
+//           columns of its tiles (four lanes a query, 128 buckets); the 8th
+//           smallest of the 128 bucket minima is reached by 8
+//           distinct candidates, so it bounds the query's 8th-nearest
+//           distance from above -- exactly it, unless two of the 8 nearest
+//           share a bucket;
+//   pass 2: candidates within the bound are appended to the lane's buffer
+//           (compacted to its 8 best when it may fill, which lowers the
+//           limit); the four buffers of a query are merged at the end.
+// A lane is one query, so its limit and count are registers and 32 columns are
+// dismissed by their minimum and one vote; with queries in the columns every
+// element took a limit read and a mask bit, and every hit a tree of selects
+// (1242 x 375: 123 -> 68 us, 1917 x 1083: 1222 -> 925, 256 x 80: 53 -> 18).  256
+// candidates a step instead of 128: the thread that issues the MMAs took about 840
+// clocks a step, whatever its size (-> 51, 577 and 21 us; each visit's MMAs take
+// 512 clocks).
 // Every wait is bounded; a timeout raises the CTA's failure flag, after
 // which the warps skip their work but still reach every barrier, and the
 // copy and MMA threads let their work in flight land before the tensor
@@ -354,11 +323,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_knn_tc(const __grid_constant_
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned long long wait_ns = g_wait_limit_ns ? g_wait_limit_ns : kDefaultWaitNs;
     const unsigned long long drain_ns = kDrainFactor * wait_ns;
-    const int nt = (gq + kTcRows - 1) / kTcRows;  // candidate tiles
+    const int nt = (gq + kTcCand - 1) / kTcCand;  // candidate tiles
     const int steps = 2 * nt;                      // two passes
-    const int rows = nt * kTcRows;
     const uint8_t* gQ = A.tk + (size_t)q0 * (kTcK * 2);
-    const uint8_t* gC = A.tk + (size_t)rows * (kTcK * 2);
+    const uint8_t* gC = A.tk + (size_t)tc_rows(gq) * (kTcK * 2);
 
     if (threadIdx.x == 0) {
         mbar_init(bar_q, 1);
@@ -383,8 +351,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_knn_tc(const __grid_constant_
         // ---- bulk copies (one thread): the queries once, then the
         // candidate tiles of both passes through the stages
         if (lane == 0) {
-            mbar_expect_tx(bar_q, kTcTileBytes);
-            bulk_copy_g2s(sQ, gQ, kTcTileBytes, bar_q);
+            mbar_expect_tx(bar_q, kTcQueryBytes);
+            bulk_copy_g2s(sQ, gQ, kTcQueryBytes, bar_q);
             int issued = 0;
             bool ok = true;
             for (; issued < steps; ++issued) {
@@ -415,7 +383,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_knn_tc(const __grid_constant_
         // ---- MMAs (one thread)
         if (lane == 0) {
             int committed = 0;
-            const int withhold = g_withhold_step;
+            const int withhold = g_withhold_step < 0 ? -1 : g_withhold_step / (kTcCand / 128);  // in 128-candidate visits
             bool ok = mbar_wait(bar_q, 0, wait_ns);
             const uint32_t qaddr = smem_addr(sQ);
             for (int u = 0; ok && u < steps; ++u) {
@@ -432,8 +400,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_knn_tc(const __grid_constant_
                 const uint32_t aaddr = smem_addr(sA + s * kTcTileBytes);
 #pragma unroll
                 for (int kk = 0; kk < kTcK / 16; ++kk)
-                    tc_mma(tmem + (uint32_t)(b * kTcRows), smem_desc(aaddr + kk * 2 * kTcKGroupStride, kTcKGroupStride, 128),
-                           smem_desc(qaddr + kk * 2 * kTcKGroupStride, kTcKGroupStride, 128), kTcIdesc, kk > 0);
+                    tc_mma(tmem + (uint32_t)(b * kTcCand), smem_desc(qaddr + kk * 2 * kTcQueryGroup, kTcQueryGroup, 128),
+                           smem_desc(aaddr + kk * 2 * kTcTileGroup, kTcTileGroup, 128), kTcIdesc, kk > 0);
                 tc_commit(&bar_mma[b]);
                 tc_commit(&bar_empty[s]);
                 committed = u + 1;
@@ -452,33 +420,46 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_knn_tc(const __grid_constant_
         }
         __syncwarp();
     } else {
-        // ---- scanners: warp w reads TMEM lanes 32 (w % 4).. (its candidates)
-        // and query columns 32 (w / 4)..
-        const int g = warp & 3, h = warp >> 2;
-        const uint32_t trow = tmem + ((uint32_t)(32 * g) << 16) + (uint32_t)(kTcScanCols * h);
-        const int qc = kTcScanCols * h;  // first query column of the warp
-        int* mylim = lim + g * kTcRows + qc;
-        int* mycnt = count + g * kTcRows + qc;
-        int2* bufs = reinterpret_cast<int2*>(scratch);  // [4][kTcRows][kTcCap] in pass 2
-        int2* mybuf = bufs + ((size_t)g * kTcRows + qc) * kTcCap;
+        // ---- scanners: warp w reads TMEM lanes 32 (w % 4).. (its queries, one per
+        // lane) and candidate columns 64 (w / 4)..
+        const int part = warp >> 2, first = 2 * kTcScanCols * part;
+        const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)first;
+        const int mine = 32 * (warp & 3) + lane;  // this lane's query; four lanes (parts) per query
+        int2* bufs = reinterpret_cast<int2*>(scratch);  // [4 parts][kTcRows][kTcCap] in pass 2
+        const int rem = gq - (nt - 1) * kTcCand - first;  // columns of the last tile that are candidates
+        // the last tile's padding columns never are
+        auto mask_tail = [&](uint32_t (&v)[32], int c) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+                if (c + j >= rem) v[j] = kInfBits;
+        };
         bool live = true;
         {
             // pass 1: bucket minima
             uint32_t mins[32];
 #pragma unroll
             for (int j = 0; j < 32; ++j) mins[j] = kInfBits;
-            for (int u = 0; u < nt && live; ++u) {
-                if (!(live = scan_wait(&bar_mma[u % kTcAcc], (unsigned)(u / kTcAcc) & 1u, fail, lane, wait_ns)))
-                    break;
-                uint32_t v[32];
-                scan_load(trow, u % kTcAcc, v, bar_free, lane);
-                if (u * kTcRows + 32 * g + lane < gq) {  // not a padding row of the last tile
+            for (int u = 0; u < nt; ++u) {
+                const int b = u % kTcAcc;
+                if (!(live = scan_wait(&bar_mma[b], (unsigned)(u / kTcAcc) & 1u, fail, lane, wait_ns))) break;
+                tc_fence_after();
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) mins[j] = min(mins[j], v[j]);  // unsigned: a -0 never lowers a bound
+                for (int c = 0; c < 2 * kTcScanCols; c += kTcScanCols) {
+                    uint32_t v[32];
+                    scan_load(trow + (uint32_t)(b * kTcCand + c), v, c > 0, &bar_free[b], lane);
+                    if (u == nt - 1) mask_tail(v, c);
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) {
+                        // the second 32 columns backwards: candidates a fixed
+                        // offset apart (vertical neighbours in a grid 32 wide are
+                        // often both near) then share no bucket
+                        uint32_t& m = mins[c > 0 ? 31 - j : j];
+                        m = min(m, v[j]);  // unsigned: a -0 never lowers a bound
+                    }
                 }
             }
 #pragma unroll
-            for (int j = 0; j < 32; ++j) scratch[(qc + j) * kTcMinStride + 32 * g + lane] = (int)mins[j];
+            for (int j = 0; j < 32; ++j) scratch[mine * kTcMinStride + 32 * part + j] = (int)mins[j];
         }
         asm volatile("bar.sync 1, %0;" ::"r"(kTcScanWarps * 32) : "memory");
         {
@@ -520,68 +501,88 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_knn_tc(const __grid_constant_
             lim[part * kTcRows + q] = (int)min(a[7], (uint32_t)kMaxFiniteBits);
         }
         asm volatile("bar.sync 1, %0;" ::"r"(kTcScanWarps * 32) : "memory");
-        for (int e = threadIdx.x; e < 4 * kTcRows * kTcCap; e += kTcScanWarps * 32)
-            bufs[e] = make_int2(0x7fffffff, 0x7fffffff);
-        for (int e = threadIdx.x; e < 4 * kTcRows; e += kTcScanWarps * 32) count[e] = 0;
-        asm volatile("bar.sync 1, %0;" ::"r"(kTcScanWarps * 32) : "memory");
-        // pass 2: every candidate within its query's limit goes to the
-        // buffer of (lane group, query), in increasing index order
-        const unsigned lt = (1u << lane) - 1u;
-        for (int u = nt; u < steps && live; ++u) {
-            if (!(live = scan_wait(&bar_mma[u % kTcAcc], (unsigned)(u / kTcAcc) & 1u, fail, lane, wait_ns))) break;
-            uint32_t v[32];
-            scan_load(trow, u % kTcAcc, v, bar_free, lane);
-            const int idx = (u - nt) * kTcRows + 32 * g + lane;
-            unsigned m = 0;  // columns where this lane's candidate is within the limit
-            if (idx < gq) {  // not a padding row of the last tile
+        // pass 2: every candidate within its query's limit goes to the lane's
+        // buffer, in increasing index order
+        {
+            int2* buf = bufs + ((size_t)part * kTcRows + mine) * kTcCap;
+            const int swizzle = mine % kTcCap;
+            int limit = q0 + mine < gq ? lim[part * kTcRows + mine] : -1, cnt = 0;
+            for (int u = nt; u < steps && live; ++u) {
+                const int b = u % kTcAcc;
+                if (!(live = scan_wait(&bar_mma[b], (unsigned)(u / kTcAcc) & 1u, fail, lane, wait_ns))) break;
+                tc_fence_after();
+#pragma unroll 1
+                for (int c = 0; c < 2 * kTcScanCols; c += kTcScanCols) {
+                    uint32_t v[32];
+                    scan_load(trow + (uint32_t)(b * kTcCand + c), v, c > 0, &bar_free[b], lane);
+                    if (u == steps - 1) mask_tail(v, c);
+                    // dismissed by the minimum of all 32 and one vote, else by that of 8
+                    int low[4];
 #pragma unroll
-                for (int j = 0; j < 32; j += 4) {
-                    const int4 l4 = *reinterpret_cast<const int4*>(mylim + j);
-                    m |= (unsigned)((int)v[j] <= l4.x) << j | (unsigned)((int)v[j + 1] <= l4.y) << (j + 1) |
-                         (unsigned)((int)v[j + 2] <= l4.z) << (j + 2) | (unsigned)((int)v[j + 3] <= l4.w) << (j + 3);
+                    for (int k = 0; k < 4; ++k) {
+                        low[k] = (int)v[8 * k];
+#pragma unroll
+                        for (int j = 1; j < 8; ++j) low[k] = min(low[k], (int)v[8 * k + j]);
+                    }
+                    const int lowest = min(min(low[0], low[1]), min(low[2], low[3]));
+                    if (!__any_sync(0xffffffffu, lowest <= limit)) continue;
+                    const int idx = (u - nt) * kTcCand + first + c;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        if (!__any_sync(0xffffffffu, low[k] <= limit)) continue;
+                        if (cnt > 8) {  // room for 8 more
+                            limit = min(limit, tc_compact(buf, swizzle, cnt));
+                            cnt = 8;
+                        }
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            const int d = (int)v[8 * k + j];
+                            if (d <= limit) buf[cnt++ ^ swizzle] = make_int2((int)__int_as_float(d), idx + 8 * k + j);
+                        }
+                    }
                 }
             }
-            unsigned cols = __reduce_or_sync(0xffffffffu, m);
-            while (cols) {
-                const int j = __ffs(cols) - 1;
-                cols &= cols - 1;
-                const int mine = (int)select32(v, j);
-                const unsigned ent = __ballot_sync(0xffffffffu, (m >> j) & 1u);
-                const int c = mycnt[j];
-                if (c + __popc(ent) <= kTcCap) {
-                    if ((m >> j) & 1u) mybuf[j * kTcCap + c + __popc(ent & lt)] = make_int2((int)__int_as_float(mine), idx);
-                    if (lane == 0) mycnt[j] = c + __popc(ent);
-                } else {
-                    tc_append_slow(ent, mine, idx, c, mybuf + j * kTcCap, mycnt + j, mylim + j, lane);
+            if (cnt > 8) {
+                tc_compact(buf, swizzle, cnt);
+                cnt = 8;
+            }
+            count[part * kTcRows + mine] = cnt;
+        }
+        // ---- merge the four buffers (at most 8 each, in any order) of each query:
+        // thread (query, column group) ranks its own entries among all of them
+        asm volatile("bar.sync 1, %0;" ::"r"(kTcScanWarps * 32) : "memory");
+        {
+            const int q = threadIdx.x & (kTcRows - 1), swizzle = q % kTcCap;
+            int2* out = A.best8 + (size_t)(q0 + q) * 8;
+            // after a failed wait the lists are empty: the queries start empty
+            // instead of reading stale candidate indices
+            const bool done = *fail == 0;
+            unsigned long long key[8];
+            int rank[8], total = 0;
+            const int n = done ? count[part * kTcRows + q] : 0;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int2 x = e < n ? bufs[((size_t)part * kTcRows + q) * kTcCap + (e ^ swizzle)] : make_int2(0, 0);
+                key[e] = (unsigned long long)(unsigned)x.x << 32 | (unsigned)x.y;
+                rank[e] = 0;
+            }
+            for (int p = 0; p < 4; ++p) {
+                const int m = done ? count[p * kTcRows + q] : 0;
+                total += m;
+                for (int e = 0; e < m; ++e) {
+                    const int2 x = bufs[((size_t)p * kTcRows + q) * kTcCap + (e ^ swizzle)];
+                    const unsigned long long k = (unsigned long long)(unsigned)x.x << 32 | (unsigned)x.y;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) rank[i] += k < key[i];
                 }
             }
-            __syncwarp();
-        }
-        // each buffer holding more than 8 candidates down to its 8 best
-        for (int j = 0; j < kTcScanCols; ++j) {
-            const int c = mycnt[j];
-            if (c > 8) tc_compact(mybuf + j * kTcCap, c, lane);
-        }
-        // ---- merge the four lane-group buffers (8 best each, in any order)
-        // of each query (warp w: kTcRows / kTcScanWarps queries)
-        asm volatile("bar.sync 1, %0;" ::"r"(kTcScanWarps * 32) : "memory");
-        for (int qq = 0; qq < kTcRows / kTcScanWarps; ++qq) {
-            const int q = warp * (kTcRows / kTcScanWarps) + qq;
-            if (q0 + q >= gq) break;
-            if (!live) {
-                // after a failed wait the lists are empty: the queries start
-                // empty instead of reading stale candidate indices
-                if (lane < 8) A.best8[(size_t)(q0 + q) * 8 + lane] = make_int2(0x7fffffff, 0x7fffffff);
-                continue;
-            }
-            const int2 e = bufs[((size_t)(lane >> 3) * kTcRows + q) * kTcCap + (lane & 7)];
-            int rank = 0;
+            if (q0 + q < gq) {
 #pragma unroll
-            for (int o = 0; o < 32; ++o) {
-                const int od = __shfl_sync(0xffffffffu, e.x, o), oi = __shfl_sync(0xffffffffu, e.y, o);
-                rank += (od < e.x) || (od == e.x && (oi < e.y || (oi == e.y && o < lane)));
+                for (int e = 0; e < 8; ++e)
+                    if (e < n && rank[e] < 8) out[rank[e]] = make_int2((int)(key[e] >> 32), (int)(unsigned)key[e]);
+                if (part == 0)
+                    for (int e = total; e < 8; ++e) out[e] = make_int2(0x7fffffff, 0x7fffffff);
             }
-            if (rank < 8) A.best8[(size_t)(q0 + q) * 8 + rank] = e;
         }
     }
     tc_fence_before();
@@ -2518,25 +2519,32 @@ bool default_tuning(const sff_tuning& t) {
     return memcmp(&t, &d, sizeof t) == 0;
 }
 
-// Scale s over px grid pixels of the launch's fields.  The default tuning leaves
-// everything to the library; with any other, scale 0 takes the tuned variant, a
-// coarser scale its entry when one is given, and the schedule is the tuning's.
-// The library's schedule: the scales below the slot limit fused into one
-// cooperative launch (256 x 80 415 / 396, 512 x 160 508 / 491 us the stage), the
-// others as dependent launches (1242 x 375 1732 / 1630; the launches' gaps), but not
-// in a captured graph, whose gaps are short and where they hold up the features'
-// stream (the batch 20.9 without, 23.4 ms with them); a quad's two fields side by side and, where the four images' records of the grid
-// exceed half of L2, every other launch backwards (together 1395 / 1349 and, 1917 x
-// 1083, 6324 / 5901).
+// Scale s over px grid pixels of the launch's fields, px0 at scale 0.  The default
+// tuning leaves everything to the library; with any other, scale 0 takes the tuned
+// variant, a coarser scale its entry when one is given, and the schedule is the
+// tuning's.  The library's schedule (us the stage, other choice / this one):
+//   - in small stages the scales below the slot limit are fused into one
+//     cooperative launch each (512 x 160 478 / 461, 640 x 192 590 / 569; 900 x 300
+//     906 / 898); in larger ones the features still run beside them, whose CTAs
+//     the grid barriers wait for (1024 x 436 1324 / 1260, 1242 x 375 1399 / 1300);
+//   - the others are dependent launches, which hide the launches' gaps (1242 x 375
+//     1732 / 1630 before the other changes), but not scales 2 and 3 of the
+//     largest stages, where the waiting CTAs take the features' place (1917 x 1083
+//     5446 / 5311), nor in a captured graph, whose gaps are short (the batch 23.4 /
+//     20.9 ms);
+//   - a quad's two fields side by side and, where the four images' records of the
+//     grid exceed half of L2, every other launch backwards (together 1395 / 1349
+//     and, 1917 x 1083, 6324 / 5901).
 constexpr double kAlternateBytes = 64e6;
+constexpr long kFuseStagePixPerSm = 4096, kDependentStagePixPerSm = 16384;
 
-ScalePlan plan_scale(const sff_tuning& t, bool derive, bool capturing, int s, long px) {
+ScalePlan plan_scale(const sff_tuning& t, bool derive, bool capturing, int s, long px, long px0) {
     ScalePlan p;
     if (derive) {
         p.v = derived_variant(px);
-        p.fuse = s > 0 && p.v->slots > 0;
+        p.fuse = s > 0 && p.v->slots > 0 && px0 / kSmCount < kFuseStagePixPerSm;
         if (s == 0 && p.v->slots > 0) p.v = find_variant(1, 0, 32, 8, 0);  // 256 x 80: 597 / 524 us
-        p.pdl = !p.fuse && !capturing;
+        p.pdl = !p.fuse && !capturing && (s < 2 || px0 / kSmCount < kDependentStagePixPerSm);
         p.alternate = !p.fuse && 2.0 * kFeat * (double)px > kAlternateBytes;
         p.pair = true;
         return p;
@@ -2570,7 +2578,7 @@ FieldScratch field_scratch(int w, int h, const sff_params& p) {
     FieldScratch f;
     f.best8 = 0;
     f.tk = f.best8 + align256((size_t)gq * 8 * sizeof(int2));
-    f.rec = f.tk + align256((size_t)2 * tc_rows(gq) * kTcK * 2);
+    f.rec = f.tk + align256(((size_t)tc_rows(gq) + tc_cand_rows(gq)) * kTcK * 2);
     f.rec_n = f.rec + align256((size_t)2 * gq * kFeat);
     f.field = f.rec_n + align256((size_t)2 * gq * sizeof(int));
     f.cost = f.field + align256((size_t)w * h * 8);
@@ -2705,7 +2713,7 @@ int run_fields(const FieldSpec* spec, int nf, const sff_params& P, const sff_tun
             mgq = std::max(mgq, F.f[k].gq);
         }
         if (s == S - 1) {
-            dim3 g0((tc_rows(mgq) * 8 + 255) / 256, 4, nf);
+            dim3 g0((tc_cand_rows(mgq) * 8 + 255) / 256, 4, nf);
             SFF_LAUNCH(k_gather_grid, g0, 256, 0, st, F, n);
             if (!knn_smem_ready()) return SFF_ERR_CUDA;
             if (fork_hook) {
@@ -2772,9 +2780,12 @@ int run_fields(const FieldSpec* spec, int nf, const sff_params& P, const sff_tun
                 ggw = std::max(ggw, gw[k]);
                 ggh = std::max(ggh, gh[k]);
             }
-            long px = 0;
-            for (int k = f0; k < f1; ++k) px += (long)gw[k] * gh[k];
-            const ScalePlan plan = plan_scale(T, derive, capturing, s, px);
+            long px = 0, px0 = 0;
+            for (int k = f0; k < f1; ++k) {
+                px += (long)gw[k] * gh[k];
+                px0 += (long)spec[k].width * spec[k].height;
+            }
+            const ScalePlan plan = plan_scale(T, derive, capturing, s, px, px0);
             const IterVariant* sv = plan.v;
             // pairs: every field f0 + 2j, f0 + 2j + 1 one quad's two fields
             bool pair = plan.pair && ((f1 - f0) & 1) == 0;
@@ -2925,7 +2936,7 @@ int run_field_sift(const FieldSpec& fs, const float* const* phi, const sff_param
                         plane_of(fs.crs, s, S, w, h), w, h, fs.mirror ? -1 : 1};
             A.gw = gw;
             A.gh = gh;
-            dim3 g0((tc_rows(A.gq) * 8 + 255) / 256, 4, 1);
+            dim3 g0((tc_cand_rows(A.gq) * 8 + 255) / 256, 4, 1);
             SFF_LAUNCH(k_gather_grid, g0, 256, 0, st, F, N);
             if (!knn_smem_ready()) return SFF_ERR_CUDA;
             dim3 g1((A.gq + kTcRows - 1) / kTcRows, 1, 1);
