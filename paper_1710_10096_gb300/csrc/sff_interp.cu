@@ -50,6 +50,7 @@ namespace {
 
 constexpr int kBlock = 3;            // sparsification block of Sec. 3.2
 constexpr int kModelWarps = 2;       // warps (seeds) per CTA of k_interp_models
+constexpr int kSeedsPerWarp = 2;     // seeds whose sums share a warp's instructions (16 lanes each)
 constexpr int kMaxK = 1024;          // largest k_geo / k_motion
 constexpr int kRegKeys = 16;         // candidate keys per lane held in registers during selection
 
@@ -152,13 +153,13 @@ __device__ __forceinline__ void ring_cell(int r, int k, int& ox, int& oy) {
 
 __device__ __forceinline__ int ring_cells(int r) { return r == 0 ? 1 : 8 * r; }
 
-// Sums v[0 .. N) over the warp by recursive halving: on return lane l holds
-// in v[0] the total of value l >> (5 - log2 N).
-template <int N>
+// Sums v[0 .. N) over groups of W lanes by recursive halving: on return lane l of
+// a group holds in v[0 .. N / W) the totals of values l N / W ...
+template <int N, int W>
 __device__ __forceinline__ void reduce_scatter(double (&v)[N], int lane) {
-    static_assert(N >= 1 && N <= 32 && (N & (N - 1)) == 0, "power of two up to 32");
+    static_assert(W <= 32 && (W & (W - 1)) == 0 && N % W == 0, "whole halves");
 #pragma unroll
-    for (int h = N / 2, o = 16; h >= 1; h >>= 1, o >>= 1) {
+    for (int o = W / 2, h = N / 2; o >= 1; o >>= 1, h >>= 1) {
         const bool up = lane & o;
 #pragma unroll
         for (int i = 0; i < h; ++i) {
@@ -167,9 +168,6 @@ __device__ __forceinline__ void reduce_scatter(double (&v)[N], int lane) {
             v[i] = keep + __shfl_xor_sync(kFull, send, o);
         }
     }
-    constexpr int kLog = N >= 32 ? 5 : N >= 16 ? 4 : N >= 8 ? 3 : N >= 4 ? 2 : N >= 2 ? 1 : 0;
-#pragma unroll
-    for (int o = 16 >> kLog; o >= 1; o >>= 1) v[0] += __shfl_xor_sync(kFull, v[0], o);
 }
 
 struct Candidates {
@@ -402,26 +400,18 @@ __device__ __forceinline__ void solve4(const double (&u)[10], double (&b)[4]) {
     }
 }
 
-// Shared memory of one warp of k_interp_models: candidate positions and map
-// words (J.slots each), the two neighbour lists (k_geo, k_motion slots of
-// 16 bits), 32 ints of scratch.
+// Shared memory of one warp of k_interp_models: candidate positions and map words
+// (J.slots each), the neighbour lists of its seeds (k_geo, k_motion position and
+// word pairs each), 32 ints of scratch.
 __host__ __device__ __forceinline__ size_t warp_smem_bytes(int slots, int kg, int km) {
-    return (size_t)slots * 8 + (((size_t)(kg + km) * 2 + 15) & ~(size_t)15) + 128;
+    return (size_t)slots * 8 + (size_t)kSeedsPerWarp * (kg + km) * 8 + 128;
 }
 
-__global__ void __launch_bounds__(kModelWarps * 32) k_interp_models(InterpJob J) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int si = blockIdx.x * kModelWarps + wid;
-    const int n = seed_count(J);
-    if (si >= n) return;  // warp-uniform
+// The two neighbourhoods of seed si into la[kg] and lm[km]; false when the
+// candidates do not fit the slots.
+__device__ __forceinline__ bool select_neighbours(const InterpJob& J, int si, int n, uint32_t* pos, int* word, int* scratch,
+                                                  uint2* la, uint2* lm, int& na, int& nm, int lane) {
     const int kg = J.p.k_geo, km = J.p.k_motion;
-    unsigned char* mine = smem_raw + (size_t)wid * warp_smem_bytes(J.slots, kg, km);
-    uint32_t* pos = reinterpret_cast<uint32_t*>(mine);
-    int* word = reinterpret_cast<int*>(mine + (size_t)J.slots * 4);
-    uint16_t* la = reinterpret_cast<uint16_t*>(mine + (size_t)J.slots * 8);
-    uint16_t* lm = la + kg;
-    int* scratch = reinterpret_cast<int*>(mine + warp_smem_bytes(J.slots, kg, km) - 128);
     const sff_seed s = J.seeds[si];
     const int bx = s.x / kBlock, by = s.y / kBlock;
     const int rmax = max(J.gbw, J.gbh);
@@ -534,10 +524,7 @@ __global__ void __launch_bounds__(kModelWarps * 32) k_interp_models(InterpJob J)
     int q = 0;
     for (; q <= rmax && (fa < kg || fm < km); ++q) scan(q);
     __syncwarp();
-    if (fill > J.slots) {
-        if (lane == 0) atomicOr(J.status, kErrOverflow);
-        return;
-    }
+    if (fill > J.slots) return false;
     if (fa >= kg && fm >= km) {
         const Candidates C1{pos, word, fill};
         int cnt[4];
@@ -550,15 +537,12 @@ __global__ void __launch_bounds__(kModelWarps * 32) k_interp_models(InterpJob J)
         __syncwarp();
     }
     const Candidates C{pos, word, fill};
-    if (C.m > J.slots) {
-        if (lane == 0) atomicOr(J.status, kErrOverflow);
-        return;
-    }
+    if (C.m > J.slots) return false;
     Threshold TA, TM;
     select_both(C, kg, km, fa, fm, min(bound_a, far_a), min(bound_m, far_m), n, scratch, lane, TA, TM);
 
-    // the members of both neighbourhoods, compacted into lists of slots
-    int na = 0, nm = 0;
+    // the members of both neighbourhoods, compacted into lists
+    na = nm = 0;
     for (int base = 0; base < C.m; base += 32) {
         const int j = base + lane;
         bool in_a = false, in_m = false;
@@ -571,28 +555,66 @@ __global__ void __launch_bounds__(kModelWarps * 32) k_interp_models(InterpJob J)
         }
         const unsigned ba = __ballot_sync(kFull, in_a), bm = __ballot_sync(kFull, in_m);
         const int qa = na + __popc(ba & lt), qm = nm + __popc(bm & lt);
-        if (in_a && qa < kg) la[qa] = (uint16_t)j;
-        if (in_m && qm < km) lm[qm] = (uint16_t)j;
+        if (in_a && qa < kg) la[qa] = make_uint2(C.pos[j], (uint32_t)C.word[j]);
+        if (in_m && qm < km) lm[qm] = make_uint2(C.pos[j], (uint32_t)C.word[j]);
         na += __popc(ba);
         nm += __popc(bm);
     }
     __syncwarp();
-    if (na > kg || nm > km) {  // unreachable: at most k members are selected
-        if (lane == 0) atomicOr(J.status, kErrOverflow);
-        return;
+    return na <= kg && nm <= km;  // at most k members are selected
+}
+
+// One warp per two seeds: the whole warp selects each seed's neighbourhoods in
+// turn, then the sums of both run side by side, 16 lanes per seed.  An FP64
+// instruction holds its sub-partition's pipe for 64 clocks whatever its active
+// lanes, so what counts is the number of warp instructions: with 32 lanes per seed
+// the 80 motion neighbours took three rounds (2.5 needed) and the two reductions 47
+// additions; 174 instead of 221 FP64 instructions per seed.  1242 x 375, default
+// neighbourhoods: 778 -> 714 us (with the disparity fill's seeds 989 -> 879); four
+// seeds per warp 887: their lists leave 12 warps per SM.
+__global__ void __launch_bounds__(kModelWarps * 32, 8) k_interp_models(InterpJob J) {
+    constexpr int SP = kSeedsPerWarp, W = 32 / SP;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int s0 = (blockIdx.x * kModelWarps + wid) * SP;
+    const int n = seed_count(J);
+    if (s0 >= n) return;  // warp-uniform
+    const int kg = J.p.k_geo, km = J.p.k_motion;
+    unsigned char* mine = smem_raw + (size_t)wid * warp_smem_bytes(J.slots, kg, km);
+    uint32_t* pos = reinterpret_cast<uint32_t*>(mine);
+    int* word = reinterpret_cast<int*>(mine + (size_t)J.slots * 4);
+    uint2* lists = reinterpret_cast<uint2*>(mine + (size_t)J.slots * 8);
+    int* scratch = reinterpret_cast<int*>(lists + SP * (kg + km));
+    const int sub = lane / W, l = lane % W, si = s0 + sub;  // this lane's seed
+    int na = 0, nm = 0;
+#pragma unroll 1
+    for (int k = 0; k < SP; ++k) {
+        if (s0 + k >= n) break;
+        int a, m;
+        uint2* la = lists + k * (kg + km);
+        if (!select_neighbours(J, s0 + k, n, pos, word, scratch, la, la + kg, a, m, lane)) {
+            if (lane == 0) atomicOr(J.status, kErrOverflow);
+            a = m = 0;  // the field is all zeros
+        }
+        if (sub == k) {
+            na = a;
+            nm = m;
+        }
+        __syncwarp();
     }
+    const uint2 *la = lists + sub * (kg + km), *lm = la + kg;
 
     // plane sums and the motion centroid: M00 M01 M02 M11 M12 M22 b0 b1 b2,
     // then W, W x0 (3)
     double g[16];
 #pragma unroll
     for (int k = 0; k < 16; ++k) g[k] = 0.0;
-    for (int t = lane; t < na; t += 32) {
-        const int j = la[t];
+    for (int t = l; t < na; t += W) {
+        const uint2 c = la[t];
         int dx, dy;
-        const unsigned d2 = cand_d2(C.pos[j], dx, dy);
+        const unsigned d2 = cand_d2(c.x, dx, dy);
         const double wt = weight_of(J, d2);
-        const double d = J.pts[(size_t)word_index(C.word[j]) * kPointDoubles + 6];
+        const double d = J.pts[(size_t)word_index((int)c.y) * kPointDoubles + 6];
         const double r0 = dx, r1 = dy;
         const double w0 = wt * r0, w1 = wt * r1;
         g[0] += w0 * r0;
@@ -605,25 +627,25 @@ __global__ void __launch_bounds__(kModelWarps * 32) k_interp_models(InterpJob J)
         g[7] += w1 * d;
         g[8] += wt * d;
     }
-    for (int t = lane; t < nm; t += 32) {
-        const int j = lm[t];
+    for (int t = l; t < nm; t += W) {
+        const uint2 c = lm[t];
         int dx, dy;
-        const unsigned d2 = cand_d2(C.pos[j], dx, dy);
+        const unsigned d2 = cand_d2(c.x, dx, dy);
         const double wt = weight_of(J, d2);
-        const double* X = J.pts + (size_t)word_index(C.word[j]) * kPointDoubles;
+        const double* X = J.pts + (size_t)word_index((int)c.y) * kPointDoubles;
         g[9] += wt;
         g[10] += wt * X[0];
         g[11] += wt * X[1];
         g[12] += wt * X[2];
     }
-    reduce_scatter(g, lane);  // value v on lanes 2v, 2v + 1
+    __syncwarp();
+    reduce_scatter<16, W>(g, lane);
+    auto value = [&](int k) { return __shfl_sync(kFull, g[0], sub * W + k); };  // on lane k of the group
     double cen[3] = {0.0, 0.0, 0.0};
     {
-        const double W = __shfl_sync(kFull, g[0], 18);
-        const double c0 = __shfl_sync(kFull, g[0], 20), c1 = __shfl_sync(kFull, g[0], 22),
-                     c2 = __shfl_sync(kFull, g[0], 24);
+        const double ws = value(9), c0 = value(10), c1 = value(11), c2 = value(12);
         if (nm > 0) {
-            const double iw = 1.0 / W;
+            const double iw = 1.0 / ws;
             cen[0] = c0 * iw;
             cen[1] = c1 * iw;
             cen[2] = c2 * iw;
@@ -631,15 +653,16 @@ __global__ void __launch_bounds__(kModelWarps * 32) k_interp_models(InterpJob J)
     }
     // centred motion sums: N (upper triangle of [r 1][r 1]^T, 10) and
     // R[j][a] = sum w r_a x1_j (12), r = x0 - c
-    double a[32];
+    constexpr int kSums = 32;
+    double a[kSums];
 #pragma unroll
-    for (int k = 0; k < 32; ++k) a[k] = 0.0;
-    for (int t = lane; t < nm; t += 32) {
-        const int j = lm[t];
+    for (int k = 0; k < kSums; ++k) a[k] = 0.0;
+    for (int t = l; t < nm; t += W) {
+        const uint2 c = lm[t];
         int dx, dy;
-        const unsigned d2 = cand_d2(C.pos[j], dx, dy);
+        const unsigned d2 = cand_d2(c.x, dx, dy);
         const double wt = weight_of(J, d2);
-        const double* X = J.pts + (size_t)word_index(C.word[j]) * kPointDoubles;
+        const double* X = J.pts + (size_t)word_index((int)c.y) * kPointDoubles;
         const double r[4] = {X[0] - cen[0], X[1] - cen[1], X[2] - cen[2], 1.0};
         const double wr[4] = {wt * r[0], wt * r[1], wt * r[2], wt};
         int e = 0;
@@ -652,14 +675,18 @@ __global__ void __launch_bounds__(kModelWarps * 32) k_interp_models(InterpJob J)
 #pragma unroll
             for (int p = 0; p < 4; ++p) a[10 + jj * 4 + p] += wr[p] * X[3 + jj];
     }
-    reduce_scatter(a, lane);  // value v on lane v
+    __syncwarp();
+    reduce_scatter<kSums, W>(a, lane);
 
     // the sums go to k_interp_solve: plane sums first, then N and R
+    if (si >= n) return;
     double* sums = J.sums + (size_t)si * kSumDoubles;
-    if (!(lane & 1) && lane < 18) sums[lane >> 1] = g[0];
-    if (lane < 22) sums[9 + lane] = a[0];
-    if (lane < 3) J.models[(size_t)si * kModelDoubles + 15 + lane] = lane == 0 ? cen[0] : lane == 1 ? cen[1] : cen[2];
-    if (lane == 0) J.motion[si] = nm;
+    if (l < 9) sums[l] = g[0];
+#pragma unroll
+    for (int i = 0; i < kSums / W; ++i)
+        if (l * (kSums / W) + i < 22) sums[9 + l * (kSums / W) + i] = a[i];
+    if (l < 3) J.models[(size_t)si * kModelDoubles + 15 + l] = l == 0 ? cen[0] : l == 1 ? cen[1] : cen[2];
+    if (l == 0) J.motion[si] = nm;
 }
 
 // The least-squares systems of every seed, one thread per system: the
@@ -942,7 +969,8 @@ extern "C" int sff_interpolate(const sff_seed* seeds_dev, const int32_t* count_d
         if (smem > 48 * 1024 &&
             cudaFuncSetAttribute(k_interp_models, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
             return SFF_ERR_CUDA;
-        SFF_LAUNCH(k_interp_models, dim3((capacity + kModelWarps - 1) / kModelWarps), kModelWarps * 32, smem, st, J);
+        constexpr int kPer = kModelWarps * kSeedsPerWarp;
+        SFF_LAUNCH(k_interp_models, dim3((capacity + kPer - 1) / kPer), kModelWarps * 32, smem, st, J);
         SFF_LAUNCH(k_interp_solve, dim3((capacity + 31) / 32), 128, 0, st, J);
     }
     int2* col = reinterpret_cast<int2*>(ws + L.nearest);
