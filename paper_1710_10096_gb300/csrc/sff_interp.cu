@@ -354,11 +354,14 @@ __device__ __forceinline__ bool selected(unsigned d2, int idx, unsigned D, int I
     return d2 < D || (d2 == D && idx <= I);
 }
 
-// Cholesky solve of one 4x4 system per lane (upper triangle u[10] row by
-// row, right-hand side b[4], solution into b); divisions by the diagonal
-// are multiplications by its reciprocal.
-__device__ __forceinline__ void solve4(const double (&u)[10], double (&b)[4]) {
+// Cholesky factorisation of one 4x4 matrix per lane (upper triangle u[10] row by
+// row), and the solution of one right-hand side into b[4]; divisions by the
+// diagonal are multiplications by its reciprocal.
+struct Factor4 {
     double L[4][4], inv[4];
+};
+__device__ __forceinline__ void factor4(const double (&u)[10], Factor4& F) {
+    auto& L = F.L;
     L[0][0] = u[0];
     L[1][0] = u[1];
     L[2][0] = u[2];
@@ -375,28 +378,30 @@ __device__ __forceinline__ void solve4(const double (&u)[10], double (&b)[4]) {
 #pragma unroll
         for (int k = 0; k < j; ++k) s -= L[j][k] * L[j][k];
         const double ljj = sqrt(s > 0.0 ? s : 1e-300);
-        inv[j] = 1.0 / ljj;
+        F.inv[j] = 1.0 / ljj;
 #pragma unroll
         for (int i = j + 1; i < 4; ++i) {
             double t = L[i][j];
 #pragma unroll
             for (int k = 0; k < j; ++k) t -= L[i][k] * L[j][k];
-            L[i][j] = t * inv[j];
+            L[i][j] = t * F.inv[j];
         }
     }
+}
+__device__ __forceinline__ void solve4(const Factor4& F, double (&b)[4]) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         double t = b[i];
 #pragma unroll
-        for (int k = 0; k < i; ++k) t -= L[i][k] * b[k];
-        b[i] = t * inv[i];
+        for (int k = 0; k < i; ++k) t -= F.L[i][k] * b[k];
+        b[i] = t * F.inv[i];
     }
 #pragma unroll
     for (int i = 3; i >= 0; --i) {
         double t = b[i];
 #pragma unroll
-        for (int k = i + 1; k < 4; ++k) t -= L[k][i] * b[k];
-        b[i] = t * inv[i];
+        for (int k = i + 1; k < 4; ++k) t -= F.L[k][i] * b[k];
+        b[i] = t * F.inv[i];
     }
 }
 
@@ -689,17 +694,20 @@ __global__ void __launch_bounds__(kModelWarps * 32, 8) k_interp_models(InterpJob
     if (l == 0) J.motion[si] = nm;
 }
 
-// The least-squares systems of every seed, one thread per system: the
-// plane (a 3x3 system, padded to 4x4 with an identity row, which leaves its
-// solution unchanged) and the three rows of [A | t] (4x4 each, one matrix).
+// The least-squares systems of every seed: the motion system (blockIdx.y 0, one
+// thread factors its 4x4 matrix once and solves the three rows of [A | t]) and the
+// plane (blockIdx.y 1; a 3x3 system, padded to 4x4 with an identity row, which
+// leaves its solution unchanged).  Bound by the FP64 pipe, so by warp
+// instructions: with the four systems on four neighbouring lanes the matrix was
+// factored three times and a warp held 8 seeds; 1242 x 375: 70 -> 26 us.
 __global__ void k_interp_solve(InterpJob J) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int si = t >> 2, row = t & 3;
+    const int si = blockIdx.x * blockDim.x + threadIdx.x;
     if (si >= seed_count(J)) return;
     const double* S = J.sums + (size_t)si * kSumDoubles;
     double* out = J.models + (size_t)si * kModelDoubles;
     double u[10], b[4];
-    if (row == 3) {
+    Factor4 F;
+    if (blockIdx.y == 1) {
         // M00 M01 M02 M11 M12 M22 into the padded upper triangle, b0 b1 b2
         u[0] = S[0];
         u[1] = S[1];
@@ -718,7 +726,8 @@ __global__ void k_interp_solve(InterpJob J) {
         b[1] = S[7];
         b[2] = S[8];
         b[3] = 0.0;
-        solve4(u, b);
+        factor4(u, F);
+        solve4(F, b);
         out[0] = b[0];
         out[1] = b[1];
         out[2] = b[2];
@@ -726,23 +735,25 @@ __global__ void k_interp_solve(InterpJob J) {
     }
     if (J.motion[si] == 0) {
 #pragma unroll
-        for (int p = 0; p < 4; ++p) out[3 + 4 * row + p] = 0.0;
+        for (int p = 0; p < 12; ++p) out[3 + p] = 0.0;
         return;
     }
 #pragma unroll
     for (int k = 0; k < 10; ++k) u[k] = S[9 + k];
-#pragma unroll
-    for (int p = 0; p < 4; ++p) b[p] = S[19 + 4 * row + p];
     const double lam = 1e-9 * (u[0] + u[4] + u[7] + u[9]) / 4 + 1e-300;
     u[0] += lam;
     u[4] += lam;
     u[7] += lam;
+    factor4(u, F);
 #pragma unroll
-    for (int p = 0; p < 3; ++p)
-        if (p == row) b[p] += lam;  // towards A = I
-    solve4(u, b);
+    for (int row = 0; row < 3; ++row) {
 #pragma unroll
-    for (int p = 0; p < 4; ++p) out[3 + 4 * row + p] = b[p];
+        for (int p = 0; p < 4; ++p) b[p] = S[19 + 4 * row + p];
+        b[row] += lam;  // towards A = I
+        solve4(F, b);
+#pragma unroll
+        for (int p = 0; p < 4; ++p) out[3 + 4 * row + p] = b[p];
+    }
 }
 
 // Closest seed of every pixel, exactly, in two separable passes: the
@@ -971,7 +982,7 @@ extern "C" int sff_interpolate(const sff_seed* seeds_dev, const int32_t* count_d
             return SFF_ERR_CUDA;
         constexpr int kPer = kModelWarps * kSeedsPerWarp;
         SFF_LAUNCH(k_interp_models, dim3((capacity + kPer - 1) / kPer), kModelWarps * 32, smem, st, J);
-        SFF_LAUNCH(k_interp_solve, dim3((capacity + 31) / 32), 128, 0, st, J);
+        SFF_LAUNCH(k_interp_solve, dim3((capacity + 63) / 64, 2), 64, 0, st, J);
     }
     int2* col = reinterpret_cast<int2*>(ws + L.nearest);
     SFF_LAUNCH(k_interp_columns, dim3((width + 31) / 32), dim3(32, kColSegments), 0, st, J, col);
