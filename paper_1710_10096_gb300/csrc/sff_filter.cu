@@ -133,6 +133,7 @@ __global__ void __launch_bounds__(kLocalThreads) k_cc_local(const __grid_constan
     __shared__ int lp[kTile * kTile];
     __shared__ uint2 lf[kTile * kTile];
     __shared__ uint8_t lk[kTile * kTile];
+    dependent_start();
     const FilterJob& Q = J.q[blockIdx.z];
     const int w = Q.w, h = Q.h;
     const int x0 = blockIdx.x * kTile, y0 = blockIdx.y * kTile;
@@ -190,6 +191,7 @@ __global__ void __launch_bounds__(kLocalThreads) k_cc_local(const __grid_constan
 // horizontal border (all columns).  The unions are the same whatever their
 // order, and so is every root (the minimum raster index).
 __global__ void k_cc_border(const __grid_constant__ FilterJobs J, int tau_r) {
+    dependent_start();
     const FilterJob& Q = J.q[blockIdx.z];
     const int w = Q.w, h = Q.h;
     const int nv = (w - 1) / kTile, nh = (h - 1) / kTile;  // borders with a pixel on both sides
@@ -214,6 +216,7 @@ __global__ void k_cc_border(const __grid_constant__ FilterJobs J, int tau_r) {
 // one atomic per distinct root per warp, and the "a rejected neighbour
 // could join" flag.
 __global__ void k_cc_stats(const __grid_constant__ FilterJobs J, int tau_r) {
+    dependent_start();
     const FilterJob& Q = J.q[blockIdx.z];
     const int w = Q.w, h = Q.h;
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
@@ -279,9 +282,9 @@ int run_filter(const FilterJob* jobs, int n, const sff_params& P, cudaStream_t s
         const long long p = (long long)((jobs[k].w - 1) / kTile) * jobs[k].h + (long long)((jobs[k].h - 1) / kTile) * jobs[k].w;
         pairs = pairs > p ? pairs : p;
     }
-    SFF_LAUNCH(k_cc_local, gt, kLocalThreads, 0, st, J, P.tau_r, P.tau_c);
-    if (pairs > 0) SFF_LAUNCH(k_cc_border, dim3((unsigned)((pairs + 127) / 128), 1, n), b2, 0, st, J, P.tau_r);
-    SFF_LAUNCH(k_cc_stats, g2, b2, 0, st, J, P.tau_r);
+    SFF_LAUNCH_DEPENDENT(k_cc_local, gt, kLocalThreads, 0, st, J, P.tau_r, P.tau_c);
+    if (pairs > 0) SFF_LAUNCH_DEPENDENT(k_cc_border, dim3((unsigned)((pairs + 127) / 128), 1, n), b2, 0, st, J, P.tau_r);
+    SFF_LAUNCH_DEPENDENT(k_cc_stats, g2, b2, 0, st, J, P.tau_r);
     if (remove) SFF_LAUNCH(k_cc_remove, g2, b2, 0, st, J, P.region_min);
     return launch_status();
 }

@@ -151,6 +151,7 @@ __host__ __device__ __forceinline__ int tc_cand_rows(int gq) { return (gq + kTcC
 // One thread per 8-column group of a row.  Roles 2 and 3 copy the stereo
 // and cross images' grid records into compact rows.
 __global__ void k_gather_grid(const __grid_constant__ Fields F, int n) {
+    dependent_start();
     const Field& A = pick(F);
     const int role = blockIdx.y;
     const int rows = role ? tc_cand_rows(A.gq) : tc_rows(A.gq);
@@ -304,7 +305,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_knn_tc(const __grid_constant_
     const Field& A = pick(F);
     const int gq = A.gq;
     const int q0 = blockIdx.x * kTcRows;
-    if (q0 >= gq) return;  // CTA-uniform, before any barrier or allocation
+    if (q0 >= gq) {  // CTA-uniform, before any barrier or allocation
+        dependent_start();
+        return;
+    }
     uint8_t* sm = smem_raw + ((1024 - (smem_addr(smem_raw) & 1023)) & 1023);
     uint8_t* sQ = sm + kTcOffQ;
     uint8_t* sA = sm + kTcOffA;
@@ -346,6 +350,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_knn_tc(const __grid_constant_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    dependent_start();  // the barriers and the tensor memory are set up beside the previous kernel
 
     if (warp == kTcTmaWarp) {
         // ---- bulk copies (one thread): the queries once, then the
@@ -629,6 +634,7 @@ __device__ __forceinline__ void warp_row_nearest(const RefFeat& r, const int4* r
 }
 
 __global__ void k_init_select(const __grid_constant__ Fields F, int n, int knn) {
+    dependent_start();
     const Field& A = pick(F);
     const Views& V = A.V;
     // the grid-barrier counters of every scale's fused iterations (one each)
@@ -2714,16 +2720,16 @@ int run_fields(const FieldSpec* spec, int nf, const sff_params& P, const sff_tun
         }
         if (s == S - 1) {
             dim3 g0((tc_cand_rows(mgq) * 8 + 255) / 256, 4, nf);
-            SFF_LAUNCH(k_gather_grid, g0, 256, 0, st, F, n);
+            SFF_LAUNCH_DEPENDENT(k_gather_grid, g0, 256, 0, st, F, n);
             if (!knn_smem_ready()) return SFF_ERR_CUDA;
             if (fork_hook) {
                 const int status = fork_hook->fn(fork_hook->ctx, st);
                 if (status) return status;
             }
             dim3 g1((mgq + kTcRows - 1) / kTcRows, 1, nf);
-            SFF_LAUNCH(k_knn_tc, g1, kTcThreads, kTcSmemBytes, st, F);
+            SFF_LAUNCH_DEPENDENT(k_knn_tc, g1, kTcThreads, kTcSmemBytes, st, F);
             dim3 g2((mgq + 7) / 8, 1, nf);
-            SFF_LAUNCH(k_init_select, g2, 256, 0, st, F, n, P.knn_temporal);
+            SFF_LAUNCH_DEPENDENT(k_init_select, g2, 256, 0, st, F, n, P.knn_temporal);
         } else {
             // the features of this scale may still be in flight on another stream
             if (scale_ready && cudaStreamWaitEvent(st, scale_ready[s], 0) != cudaSuccess) return SFF_ERR_CUDA;

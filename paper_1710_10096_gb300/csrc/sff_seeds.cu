@@ -45,6 +45,7 @@ __device__ unsigned int g_seed_status;
 // One thread per block: raster index of its best kept pixel or -1; one count
 // of found seeds per CTA.
 __global__ void __launch_bounds__(kChunk) k_block_best(const __grid_constant__ SeedJobs J) {
+    dependent_start();
     const SeedJob& Q = J.q[blockIdx.z];
     const int w = Q.w, h = Q.h, bw = (w + 2) / 3, nb = bw * ((h + 2) / 3);
     if ((int)blockIdx.x * kChunk >= nb) return;  // whole CTA beyond this quad's blocks
@@ -115,6 +116,7 @@ __global__ void __launch_bounds__(kChunk) k_write_seeds(const __grid_constant__ 
     __shared__ int warp_base[kChunk / 32];
     __shared__ int warp_prior[kChunk / 32];
     __shared__ int chunk_base;
+    dependent_start();
     const SeedJob& Q = J.q[blockIdx.z];
     const int w = Q.w, nb = ((Q.w + 2) / 3) * ((Q.h + 2) / 3);
     const int nchunks = (nb + kChunk - 1) / kChunk;
@@ -203,8 +205,8 @@ int run_seeds(const SeedJob* jobs, int n, cudaStream_t st) {
         const int nb = ((jobs[k].w + 2) / 3) * ((jobs[k].h + 2) / 3);
         mchunks = mchunks > (nb + kChunk - 1) / kChunk ? mchunks : (nb + kChunk - 1) / kChunk;
     }
-    SFF_LAUNCH(k_block_best, dim3(mchunks, 1, n), kChunk, 0, st, J);
-    SFF_LAUNCH(k_write_seeds, dim3(mchunks, 1, n), kChunk, 0, st, J);
+    SFF_LAUNCH_DEPENDENT(k_block_best, dim3(mchunks, 1, n), kChunk, 0, st, J);
+    SFF_LAUNCH_DEPENDENT(k_write_seeds, dim3(mchunks, 1, n), kChunk, 0, st, J);
     return launch_status();
 }
 
