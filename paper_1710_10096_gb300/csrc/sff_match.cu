@@ -1656,8 +1656,8 @@ __global__ void __launch_bounds__(fused_threads<L, C, TX, TY>(), fused_min_block
 // iteration, so this order is an order of magnitude slower per quad than the
 // checkerboard; it exists to reproduce the sequential scan exactly.
 //
-// A warp takes a block of 32 / L consecutive rows, L lanes per row, row r one
-// column behind row r - 1, and walks along them on its own: a step's horizontal
+// A warp takes a block of four consecutive rows, 8 lanes per row, row r one column
+// behind row r - 1, and walks along them on its own: a step's horizontal
 // predecessor is the group's last result, the vertical one the last result of the
 // group above (a shuffle), and the next pixel's state and reference record are
 // loaded a step ahead.  The block's last row goes to the next block's warp through
@@ -1667,9 +1667,11 @@ __global__ void __launch_bounds__(fused_threads<L, C, TX, TY>(), fused_min_block
 // in memory (it must not wait for warp 0, which may wait for the warps between
 // them).  A warp thus waits for a column of the block above, or for a ring slot
 // that the block below has not read, and no circle of waits closes; both waits are
-// bounded.  With L = 8 each predecessor has its own four lanes.
-// 256 x 80, both fields: 28.8 ms (a barrier per diagonal, states from memory) ->
-// 15.2 ms.
+// bounded.  Each predecessor of a row has its own four lanes.
+// Both fields, 256 x 80: 28.8 ms (a barrier per diagonal, states from memory) ->
+// 15.2 ms; 1242 x 375: 240 -> 196 ms; 300 x 1000: 156 -> 126 ms (238 and 204 with 4 or
+// 2 lanes per row where that leaves every block a warp of its own: a step then
+// takes more than twice as long).
 constexpr int kSweepWarps = 32, kSweepRing = 64, kSweepSignal = 16;
 
 // A pixel's state in a ring slot: two 64-bit words, each read and written whole and
@@ -1711,17 +1713,16 @@ __device__ __forceinline__ void sweep_signal(int* counter, int value) {
     asm volatile("st.release.cta.shared.s32 [%0], %1;" ::"r"(smem_addr(counter)), "r"(value) : "memory");
 }
 
-template <int L>
 __global__ void __launch_bounds__(32 * kSweepWarps) k_sweep(const __grid_constant__ Fields F, int n, int dx, int dy) {
-    constexpr int P = L == 8 ? 4 : L;  // lanes that share a record
-    constexpr int kRows = 32 / L;      // rows per block
+    constexpr int L = 8;           // lanes per row: four per predecessor
+    constexpr int kRows = 32 / L;  // rows per block
     __shared__ ulonglong2 s_ring[kSweepWarps][kSweepRing];  // last rows of the blocks, by column
     __shared__ int s_made, s_read[kSweepWarps];  // columns written by the last warp, read from a warp's ring
     const Field& A = pick(F);
     const Views& V = A.V;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
-    const int q = lane & (P - 1), g = lane / L;
-    const unsigned gmask = group_mask<L>();
+    const int q = lane & 3, g = lane / L;
+    const unsigned gmask = 0xffu << (lane & ~(L - 1));
     const int gw = A.gw, gh = A.gh, blocks = (gh + kRows - 1) / kRows;
     const unsigned long long wait_ns = g_wait_limit_ns ? g_wait_limit_ns : kDefaultWaitNs;
     for (int k = lane; k < kSweepRing; k += 32) s_ring[warp][k] = make_ulonglong2(0ull, 0ull);
@@ -1743,17 +1744,15 @@ __global__ void __launch_bounds__(32 * kSweepWarps) k_sweep(const __grid_constan
         // computed when its turn comes: here it would wait for the load)
         int c1 = kEmpty;
         uint2 w1 = make_uint2(0u, 0u);
-        Slice<P> r1;
+        int4 r1 = make_int4(0, 0, 0, 0);  // this lane's chunk
         auto fetch = [&](int a) {
             if (!mine || a < 0 || a >= gw) return;
             c1 = A.cost[row + col(a)];
             w1 = A.field[row + col(a)];
-            const size_t i = pix(V.w, col(a) * n, y);
-#pragma unroll
-            for (int k = 0; k < Slice<P>::kChunks; ++k)
-                r1.c[k] = q + k * P < 3 ? chunk_of(V.ref, i, q + k * P) : make_int4(0, 0, 0, 0);
+            r1 = chunk_of(V.ref, pix(V.w, col(a) * n, y), min(q, 2));
         };
-        // this lane's chunk of the other views' records (L = 8)
+        // this lane's chunk of the other views' records; lane 3 of four repeats
+        // chunk 2 and adds nothing
         const unsigned stride = V.ref.rs * (unsigned)sizeof(int4);
         const char* pt = reinterpret_cast<const char*>(V.tmp.f + min(q, 2) * V.tmp.cs);
         const char* ps = reinterpret_cast<const char*>(V.ste.f + min(q, 2) * V.ste.cs);
@@ -1801,53 +1800,41 @@ __global__ void __launch_bounds__(32 * kSweepWarps) k_sweep(const __grid_constan
                 const int gx = col(a), x = gx * n;
                 c = c1;
                 const uint2 w0 = w1;
-                Slice<P> r = r1;
+                const int4 r = r1;
                 fetch(a + 1);
-                r.nrm = 0;
-#pragma unroll
-                for (int k = 0; k < Slice<P>::kChunks; ++k) r.nrm = dot4(r.c[k], r.c[k], r.nrm);
                 bool changed = false;
-                if constexpr (L == 8) {
-                    // as update_pixel, lanes 0-3 scoring the horizontal
-                    // predecessor's vector, lanes 4-7 the vertical one's
-                    auto same = [](uint2 p, uint2 q) { return p.x == q.x && p.y == q.y; };
-                    wc = w0;
-                    const bool own = c != kEmpty;
-                    const bool do_a = ca != kEmpty && !(own && same(wa, w0));
-                    const bool do_b = cb != kEmpty && !(own && same(wb, w0)) && !(ca != kEmpty && same(wb, wa));
-                    if (do_a || do_b) {
-                        const bool vertical = lane & 4;
-                        // the three views' chunks in flight together; lane 3 of
-                        // four repeats chunk 2 and adds nothing
-                        const Vec4 v = unpack_vec(vertical ? wb : wa);
-                        const int tx = clampi(x + v.u, 0, V.w - 1), ty = clampi(y + v.v, 0, V.h - 1);
-                        const int sx = clampi(x - V.sigma * v.d0, 0, V.w - 1);
-                        const int cx = clampi(x + v.u - V.sigma * v.d1, 0, V.w - 1);
-                        const unsigned rt = (unsigned)ty * V.w, rs = (unsigned)y * V.w;
-                        const int4 vt = __ldg(reinterpret_cast<const int4*>(pt + (size_t)(rt + tx) * stride)),
-                                   vs = __ldg(reinterpret_cast<const int4*>(ps + (size_t)(rs + sx) * stride)),
-                                   vc = __ldg(reinterpret_cast<const int4*>(pc + (size_t)(rt + cx) * stride));
-                        const int dot = dot4(r.c[0], vt, dot4(r.c[0], vs, dot4(r.c[0], vc, 0)));
-                        const int nrm = dot4(vt, vt, dot4(vs, vs, dot4(vc, vc, 3 * r.nrm)));
-                        const int sum = group_sum<4>(q < 3 ? nrm - 2 * dot : 0, gmask),
-                                  other = __shfl_xor_sync(gmask, sum, 4);
-                        const int na = vertical ? other : sum, nv = vertical ? sum : other;
-                        if (do_a && na < c) {
-                            c = na;
-                            wc = wa;
-                            changed = true;
-                        }
-                        if (do_b && nv < c) {
-                            c = nv;
-                            wc = wb;
-                            changed = true;
-                        }
+                // as update_pixel, lanes 0-3 scoring the horizontal predecessor's
+                // vector, lanes 4-7 the vertical one's
+                auto same = [](uint2 p, uint2 q) { return p.x == q.x && p.y == q.y; };
+                wc = w0;
+                const bool own = c != kEmpty;
+                const bool do_a = ca != kEmpty && !(own && same(wa, w0));
+                const bool do_b = cb != kEmpty && !(own && same(wb, w0)) && !(ca != kEmpty && same(wb, wa));
+                if (do_a || do_b) {
+                    const bool vertical = lane & 4;
+                    const Vec4 v = unpack_vec(vertical ? wb : wa);
+                    const int tx = clampi(x + v.u, 0, V.w - 1), ty = clampi(y + v.v, 0, V.h - 1);
+                    const int sx = clampi(x - V.sigma * v.d0, 0, V.w - 1);
+                    const int cx = clampi(x + v.u - V.sigma * v.d1, 0, V.w - 1);
+                    const unsigned rt = (unsigned)ty * V.w, rs = (unsigned)y * V.w;
+                    // the three views' chunks in flight together
+                    const int4 vt = __ldg(reinterpret_cast<const int4*>(pt + (size_t)(rt + tx) * stride)),
+                               vs = __ldg(reinterpret_cast<const int4*>(ps + (size_t)(rs + sx) * stride)),
+                               vc = __ldg(reinterpret_cast<const int4*>(pc + (size_t)(rt + cx) * stride));
+                    const int dot = dot4(r, vt, dot4(r, vs, dot4(r, vc, 0)));
+                    const int nrm = dot4(vt, vt, dot4(vs, vs, dot4(vc, vc, 3 * dot4(r, r, 0))));
+                    const int sum = group_sum<4>(q < 3 ? nrm - 2 * dot : 0, gmask), other = __shfl_xor_sync(gmask, sum, 4);
+                    const int na = vertical ? other : sum, nv = vertical ? sum : other;
+                    if (do_a && na < c) {
+                        c = na;
+                        wc = wa;
+                        changed = true;
                     }
-                } else {
-                    Vec4 cur = unpack_vec(w0);
-                    changed = update_pixel<P>(V, r, q, gmask, n, 0, A.key, A.mirror, x, y, 0u, -1, -1, unpack_vec(wa), ca,
-                                              unpack_vec(wb), cb, cur, c);
-                    wc = pack_vec(cur);
+                    if (do_b && nv < c) {
+                        c = nv;
+                        wc = wb;
+                        changed = true;
+                    }
                 }
                 if (changed && (lane & (L - 1)) == 0) {
                     A.field[row + gx] = wc;
@@ -2745,13 +2732,8 @@ int run_fields(const FieldSpec* spec, int nf, const sff_params& P, const sff_tun
             }
             dim3 gr((mgw + 63) / 64, mgh, nf);
             for (int it = 0; it < I; ++it) {
-                // the most lanes per row that leave every block a warp
-                const int lanes = mgh <= 4 * kSweepWarps ? 8 : mgh <= 8 * kSweepWarps ? 4 : 2;
-                const int threads = 32 * std::min(kSweepWarps, (mgh * lanes + 31) / 32);
-                const dim3 gs(1, 1, nf);
-                if (lanes == 8) SFF_LAUNCH(k_sweep<8>, gs, threads, 0, st, F, n, kDirs[it % 4][0], kDirs[it % 4][1]);
-                else if (lanes == 4) SFF_LAUNCH(k_sweep<4>, gs, threads, 0, st, F, n, kDirs[it % 4][0], kDirs[it % 4][1]);
-                else SFF_LAUNCH(k_sweep<2>, gs, threads, 0, st, F, n, kDirs[it % 4][0], kDirs[it % 4][1]);
+                const int threads = 32 * std::min(kSweepWarps, (mgh + 3) / 4);
+                SFF_LAUNCH(k_sweep, dim3(1, 1, nf), threads, 0, st, F, n, kDirs[it % 4][0], kDirs[it % 4][1]);
                 SFF_LAUNCH(k_random_search, gr, 256, 0, st, F, n, s, it);
             }
             prev = cur;
