@@ -52,7 +52,8 @@ constexpr int kBlock = 3;            // sparsification block of Sec. 3.2
 constexpr int kModelWarps = 2;       // warps (seeds) per CTA of k_interp_models
 constexpr int kSeedsPerWarp = 2;     // seeds whose sums share a warp's instructions (16 lanes each)
 constexpr int kMaxK = 1024;          // largest k_geo / k_motion
-constexpr int kRegKeys = 16;         // candidate keys per lane held in registers during selection
+constexpr int kRegKeys = 16;         // candidate keys per lane held in registers during selection (half are, up to 256)
+constexpr int kTighten = 4;          // the ring bound is within 1/16 of the k-th distance so far
 
 // Candidate slots per seed: the rings up to the bound of the k-th nearest
 // hold about 4/pi times k seeds plus a margin of whole rings; 6 k + 256
@@ -187,13 +188,6 @@ struct Threshold {
     int I;
 };
 
-// Warp sum of an int.
-__device__ __forceinline__ int warp_sum_i(int c) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(kFull, c, o);
-    return c;
-}
-
 // The index threshold among the candidates tied at distance D: the need-th
 // smallest index of the set's members with d2 == D (need < number tied).
 // Up to 32 tied members are ranked in registers; more fall back to
@@ -233,7 +227,7 @@ __device__ int tie_threshold(const Candidates& C, bool motion, unsigned D, int n
             int dx, dy;
             c += (!motion || word_motion(w)) && cand_d2(C.pos[j], dx, dy) == D && word_index(w) <= mid;
         }
-        if (warp_sum_i(c) >= need)
+        if ((int)__reduce_add_sync(kFull, c) >= need)
             hi = mid;
         else
             lo = mid + 1;
@@ -241,112 +235,129 @@ __device__ int tie_threshold(const Candidates& C, bool motion, unsigned D, int n
     return lo;
 }
 
-// The k-th smallest d2 of both neighbourhoods, all candidates (k_geo) and
-// the motion seeds among them (k_motion), by bisections that share their
-// passes over the candidates: the smallest D with at least k members
-// within D.  hiA / hiM are distances that at least k members are within
-// (0 skips that set).  each(f) calls f(d2, motion) for every candidate of
-// the lane.
-template <class Each>
-__device__ void bisect_both(Each each, int kg, int km, unsigned hiA, unsigned hiM, unsigned& DA, unsigned& DM) {
-    unsigned loA = 0, loM = 0;
-    while (loA < hiA || loM < hiM) {
-        const unsigned midA = loA + ((hiA - loA) >> 1), midM = loM + ((hiM - loM) >> 1);
-        int ca = 0, cm = 0;
-        each([&](unsigned d2, unsigned mot) {
-            ca += d2 <= midA;
-            cm += mot & (d2 <= midM);
-        });
-        ca = warp_sum_i(ca);
-        cm = warp_sum_i(cm);
-        if (loA < hiA) {
-            if (ca >= kg)
-                hiA = midA;
-            else
-                loA = midA + 1;
-        }
-        if (loM < hiM) {
-            if (cm >= km)
-                hiM = midM;
-            else
-                loM = midM + 1;
-        }
-    }
-    DA = loA;
-    DM = loM;
-}
+// Bracket of the k-th smallest distance of a set: fewer than k members are nearer
+// than lo, at least k within hi; `full`: exactly k are within hi, which need not be
+// a member's distance itself.
+struct Bracket {
+    unsigned lo, hi;
+    bool full;
+};
 
-// Runs f(each) with each(g) calling g(d2, motion) for the lane's candidates:
-// from keys held in registers when the candidates fit (bit 31 = motion; the
-// filler 0x7fffffff is farther than any bound), else from shared memory.
+// Runs f(each) with each(g) calling g(d2, motion key) for the lane's candidates,
+// the motion key being d2 for a motion seed, past 2^31 for another; from keys held
+// in registers when the candidates fit, else from shared memory.
 template <class F>
 __device__ __forceinline__ void with_keys(const Candidates& C, int lane, F f) {
     if (C.m <= 32 * kRegKeys) {
-        unsigned key[kRegKeys];
-#pragma unroll
-        for (int t = 0; t < kRegKeys; ++t) {
+        unsigned key[kRegKeys];  // bit 31: no motion seed; the filler is farther than any bound
+        const bool second = C.m > 16 * kRegKeys;
+        auto load = [&](int t) {
             const int j = lane + 32 * t;
-            key[t] = 0x7fffffffu;
+            key[t] = 0xffffffffu;
             if (j < C.m) {
                 int dx, dy;
-                key[t] = cand_d2(C.pos[j], dx, dy) | ((unsigned)word_motion(C.word[j]) << 31);
+                key[t] = cand_d2(C.pos[j], dx, dy) | ((unsigned)!word_motion(C.word[j]) << 31);
             }
-        }
+        };
+#pragma unroll
+        for (int t = 0; t < kRegKeys / 2; ++t) load(t);
+        if (second)
+#pragma unroll
+            for (int t = kRegKeys / 2; t < kRegKeys; ++t) load(t);
         f([&](auto g) {
 #pragma unroll
-            for (int t = 0; t < kRegKeys; ++t) g(key[t] & 0x7fffffffu, key[t] >> 31);
+            for (int t = 0; t < kRegKeys / 2; ++t) g(key[t] & 0x7fffffffu, key[t]);
+            if (second)
+#pragma unroll
+                for (int t = kRegKeys / 2; t < kRegKeys; ++t) g(key[t] & 0x7fffffffu, key[t]);
         });
     } else {
         f([&](auto g) {
             for (int j = lane; j < C.m; j += 32) {
                 int dx, dy;
-                g(cand_d2(C.pos[j], dx, dy), (unsigned)word_motion(C.word[j]));
+                const unsigned d2 = cand_d2(C.pos[j], dx, dy);
+                g(d2, d2 | ((unsigned)!word_motion(C.word[j]) << 31));
             }
         });
     }
 }
 
-// The k-th smallest distances DA, DM of both sets (hiA / hiM: bounds that
-// at least k members are within; 0 skips a set) and the counts of members
-// below and at them (warp-reduced).  One routine serves the tightening of
-// the ring bound and the final selection, so that its code exists once.
-__device__ __noinline__ void kth_and_counts(const Candidates& C, int kg, int km, unsigned hiA, unsigned hiM,
-                                            int lane, unsigned& DA, unsigned& DM, int (&cnt)[4]) {
-    int ba = 0, ea = 0, bm = 0, em = 0;
+// Narrows the brackets of both sets, all candidates (k_geo) and the motion seeds
+// among them (k_motion), by bisections that share their passes over the candidates,
+// until they are full or at most hi >> shift wide (shift 31: lo = hi), and then, if
+// asked for, counts the members below and at the distances that are not full
+// (cnt[0..1] and cnt[2..3], zeros for a full one).  A set with lo = hi is left
+// alone.  The counts of both sets share a word (at most 6400 candidates) and one
+// reduction.  A dense field has about 200 candidates a seed, 7 of 16 keys per lane,
+// and ends full after 5 or 6 passes from a bracket whose lower end is the nearest
+// seed that the further rings can hold (10 from zero, and 10 more for the ring bound
+// to the last integer): k_interp_models 309 M -> 226 M warp instructions, 714 -> 659
+// us at 1242 x 375.  One routine serves the tightening of the ring bound and the final
+// selection, so that its code exists once.
+__device__ __noinline__ void narrow_both(const Candidates& C, int kg, int km, Bracket& A, Bracket& M, int shift,
+                                         int lane, int* cnt) {
+    A.full = M.full = false;
     with_keys(C, lane, [&](auto each) {
-        bisect_both(each, kg, km, hiA, hiM, DA, DM);
-        each([&](unsigned d2, unsigned mot) {
-            ba += d2 < DA;
-            ea += d2 == DA;
-            bm += mot & (d2 < DM);
-            em += mot & (d2 == DM);
-        });
+        for (;;) {
+            const bool ga = !A.full && A.hi - A.lo > (A.hi >> shift), gm = !M.full && M.hi - M.lo > (M.hi >> shift);
+            if (!ga && !gm) break;
+            const unsigned midA = A.lo + ((A.hi - A.lo) >> 1), midM = M.lo + ((M.hi - M.lo) >> 1);
+            unsigned c = 0;
+            each([&](unsigned d2, unsigned mot) {
+                if (d2 <= midA) c += 1u;
+                if (mot <= midM) c += 1u << 16;
+            });
+            c = __reduce_add_sync(kFull, c);
+            const int ca = c & 0xffffu, cm = c >> 16;
+            auto step = [](Bracket& B, unsigned mid, int count, int k) {
+                if (count < k) {
+                    B.lo = mid + 1;
+                } else {
+                    B.hi = mid;
+                    B.full = count == k;
+                }
+            };
+            if (ga) step(A, midA, ca, kg);
+            if (gm) step(M, midM, cm, km);
+        }
+        if (!cnt) return;
+        unsigned below = 0, at = 0;
+        if (!A.full || !M.full) {
+            each([&](unsigned d2, unsigned mot) {
+                if (d2 < A.hi) below += 1u;
+                if (d2 == A.hi) at += 1u;
+                if (mot < M.hi) below += 1u << 16;
+                if (mot == M.hi) at += 1u << 16;
+            });
+            below = __reduce_add_sync(kFull, below);
+            at = __reduce_add_sync(kFull, at);
+        }
+        cnt[0] = A.full ? 0 : (int)(below & 0xffffu);
+        cnt[1] = A.full ? 0 : (int)(at & 0xffffu);
+        cnt[2] = M.full ? 0 : (int)(below >> 16);
+        cnt[3] = M.full ? 0 : (int)(at >> 16);
     });
-    cnt[0] = warp_sum_i(ba);
-    cnt[1] = warp_sum_i(ea);
-    cnt[2] = warp_sum_i(bm);
-    cnt[3] = warp_sum_i(em);
 }
 
 // Thresholds of the k smallest (d2, index) keys of both neighbourhoods.
-// `fa`/`fm` are the sizes of the two sets, `far_a`/`far_m` distances that
-// at least k of their members are within.
-__device__ void select_both(const Candidates& C, int kg, int km, int fa, int fm, unsigned far_a, unsigned far_m,
-                            int n, int* scratch, int lane, Threshold& A, Threshold& M) {
+// `fa`/`fm` are the sizes of the two sets, BA / BM brackets of their k-th distances.
+__device__ void select_both(const Candidates& C, int kg, int km, int fa, int fm, Bracket BA, Bracket BM, int n,
+                            int* scratch, int lane, Threshold& A, Threshold& M) {
     A = Threshold{0xffffffffu, 0x7fffffff};
     M = Threshold{0xffffffffu, 0x7fffffff};
     const bool sa = fa > kg, sm = fm > km;
     if (!sa && !sm) return;
-    unsigned DA, DM;
     int cnt[4];
-    kth_and_counts(C, kg, km, sa ? far_a : 0, sm ? far_m : 0, lane, DA, DM, cnt);
+    if (!sa) BA.lo = BA.hi;
+    if (!sm) BM.lo = BM.hi;
+    narrow_both(C, kg, km, BA, BM, 31, lane, cnt);
     if (sa) {
-        A.D = DA;
-        if (kg - cnt[0] < cnt[1]) A.I = tie_threshold(C, false, DA, kg - cnt[0], cnt[1], n, scratch, lane);
+        A.D = BA.hi;
+        if (!BA.full && kg - cnt[0] < cnt[1]) A.I = tie_threshold(C, false, A.D, kg - cnt[0], cnt[1], n, scratch, lane);
     }
     if (sm) {
-        M.D = DM;
-        if (km - cnt[2] < cnt[3]) M.I = tie_threshold(C, true, DM, km - cnt[2], cnt[3], n, scratch, lane);
+        M.D = BM.hi;
+        if (!BM.full && km - cnt[2] < cnt[3]) M.I = tie_threshold(C, true, M.D, km - cnt[2], cnt[3], n, scratch, lane);
     }
 }
 
@@ -427,8 +438,8 @@ __device__ __forceinline__ bool select_neighbours(const InterpJob& J, int si, in
     // k members; a set's bound is the largest distance found when it got
     // them, and from then on a seed is kept only if it is within the bound
     // of a set it belongs to (so that sparse motion seeds do not drag every
-    // seed in).  Then the k-th smallest distances of the candidates replace
-    // the bounds, and the further rings that can still hold a member within
+    // seed in).  Then distances little above the k-th smallest of the candidates
+    // replace the bounds, and the further rings that can still hold a member within
     // a bound are scanned.
     int fill = 0;                                          // candidates kept
     int fa = 0, fm = 0;                                    // ... of which motion seeds: fm
@@ -443,11 +454,10 @@ __device__ __forceinline__ bool select_neighbours(const InterpJob& J, int si, in
         const Candidates Cc{pos, word, fill};
         unsigned DA = bound_a, DM = bound_m;
         if (fa >= kg || fm >= km) {
-            int cnt[4];
-            unsigned da, dm;
-            kth_and_counts(Cc, kg, km, fa >= kg ? far_a : 0, fm >= km ? far_m : 0, lane, da, dm, cnt);
-            if (fa >= kg) DA = min(DA, da);
-            if (fm >= km) DM = min(DM, dm);
+            Bracket A{0u, fa >= kg ? far_a : 0u}, M{0u, fm >= km ? far_m : 0u};
+            narrow_both(Cc, kg, km, A, M, 31, lane, nullptr);
+            if (fa >= kg) DA = min(DA, A.hi);
+            if (fm >= km) DM = min(DM, M.hi);
         }
         int kept = 0, kmot = 0;
         for (int base = 0; base < fill; base += 32) {
@@ -516,13 +526,8 @@ __device__ __forceinline__ bool select_neighbours(const InterpJob& J, int si, in
             fa += __popc(has);
             fm += __popc(mot);
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            ma = max(ma, __shfl_xor_sync(kFull, ma, o));
-            mm = max(mm, __shfl_xor_sync(kFull, mm, o));
-        }
-        far_a = max(far_a, ma);
-        far_m = max(far_m, mm);
+        far_a = max(far_a, __reduce_max_sync(kFull, ma));
+        far_m = max(far_m, __reduce_max_sync(kFull, mm));
         if (bound_a == 0xffffffffu && fa >= kg) bound_a = far_a;
         if (bound_m == 0xffffffffu && fm >= km) bound_m = far_m;
     };
@@ -530,10 +535,16 @@ __device__ __forceinline__ bool select_neighbours(const InterpJob& J, int si, in
     for (; q <= rmax && (fa < kg || fm < km); ++q) scan(q);
     __syncwarp();
     if (fill > J.slots) return false;
+    unsigned lo_a = 0, lo_m = 0;  // the k-th distances are at least these
     if (fa >= kg && fm >= km) {
         const Candidates C1{pos, word, fill};
-        int cnt[4];
-        kth_and_counts(C1, kg, km, bound_a, bound_m, lane, bound_a, bound_m, cnt);
+        Bracket A{0u, bound_a}, M{0u, bound_m};
+        narrow_both(C1, kg, km, A, M, kTighten, lane, nullptr);
+        bound_a = A.hi;
+        bound_m = M.hi;
+        const unsigned near = (unsigned)(max(3 * q - 2, 0) * max(3 * q - 2, 0));  // the further rings' seeds
+        lo_a = min(A.lo, near);
+        lo_m = min(M.lo, near);
         for (; q <= rmax; ++q) {
             const long long b = 3 * q - 2;
             if (b * b > (long long)max(bound_a, bound_m)) break;
@@ -544,7 +555,8 @@ __device__ __forceinline__ bool select_neighbours(const InterpJob& J, int si, in
     const Candidates C{pos, word, fill};
     if (C.m > J.slots) return false;
     Threshold TA, TM;
-    select_both(C, kg, km, fa, fm, min(bound_a, far_a), min(bound_m, far_m), n, scratch, lane, TA, TM);
+    select_both(C, kg, km, fa, fm, Bracket{lo_a, min(bound_a, far_a)}, Bracket{lo_m, min(bound_m, far_m)}, n, scratch,
+                lane, TA, TM);
 
     // the members of both neighbourhoods, compacted into lists
     na = nm = 0;
