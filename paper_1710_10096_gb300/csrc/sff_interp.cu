@@ -49,18 +49,24 @@ namespace sff {
 namespace {
 
 constexpr int kBlock = 3;            // sparsification block of Sec. 3.2
-constexpr int kModelWarps = 2;       // warps (seeds) per CTA of k_interp_models
+constexpr int kModelWarps = 1;       // warps per CTA of k_interp_models
 constexpr int kSeedsPerWarp = 2;     // seeds whose sums share a warp's instructions (16 lanes each)
 constexpr int kMaxK = 1024;          // largest k_geo / k_motion
 constexpr int kRegKeys = 16;         // candidate keys per lane held in registers during selection (half are, up to 256)
 constexpr int kTighten = 4;          // the ring bound is within 1/16 of the k-th distance so far
 
-// Candidate slots per seed: the rings up to the bound of the k-th nearest
-// hold about 4/pi times k seeds plus a margin of whole rings; 6 k + 256
-// leaves room for uneven seed density (with k = 160, a lone seed in the
-// middle of a 480 x 480 px hole in a dense seed lattice takes 833).
+// Candidate slots per seed: the rings up to the bound of the k-th nearest hold about
+// 4/pi times k seeds plus a margin of whole rings; 4 k + 192 leaves room for uneven
+// seed density (with k = 160, a lone seed in the middle of a 480 x 480 px hole in a
+// dense seed lattice meets 833).  What does not fit is compacted to the members of
+// both sets so far, k_geo + k_motion and those tied at the larger distance (a circle
+// within an image of 16384 px has at most 288 lattice points), and a batch of 32 more.
+// With 6 k + 256 an SM held 16 warps instead of 20: 659 -> 622 us, and 612 with one
+// warp per CTA, whose resources are free as soon as it ends.
 __host__ __device__ __forceinline__ int candidate_slots(int kg, int km) {
-    return ((6 * (kg > km ? kg : km) + 256) + 31) & ~31;
+    const int k = kg > km ? kg : km, whole = kg + km + 352;
+    const int slots = 6 * k + 256 < whole ? 6 * k + 256 : whole > 4 * k + 192 ? whole : 4 * k + 192;
+    return (slots + 31) & ~31;
 }
 constexpr int kModelDoubles = 18;    // plane 3, [A | t] 12, centre 3
 constexpr int kPointDoubles = 8;     // x0 3, x1 3, d0, pad
@@ -287,7 +293,7 @@ __device__ __forceinline__ void with_keys(const Candidates& C, int lane, F f) {
 // until they are full or at most hi >> shift wide (shift 31: lo = hi), and then, if
 // asked for, counts the members below and at the distances that are not full
 // (cnt[0..1] and cnt[2..3], zeros for a full one).  A set with lo = hi is left
-// alone.  The counts of both sets share a word (at most 6400 candidates) and one
+// alone.  The counts of both sets share a word (at most 4352 candidates) and one
 // reduction.  A dense field has about 200 candidates a seed, 7 of 16 keys per lane,
 // and ends full after 5 or 6 passes from a bracket whose lower end is the nearest
 // seed that the further rings can hold (10 from zero, and 10 more for the ring bound
@@ -589,7 +595,7 @@ __device__ __forceinline__ bool select_neighbours(const InterpJob& J, int si, in
 // additions; 174 instead of 221 FP64 instructions per seed.  1242 x 375, default
 // neighbourhoods: 778 -> 714 us (with the disparity fill's seeds 989 -> 879); four
 // seeds per warp 887: their lists leave 12 warps per SM.
-__global__ void __launch_bounds__(kModelWarps * 32, 8) k_interp_models(InterpJob J) {
+__global__ void __launch_bounds__(kModelWarps * 32, 20) k_interp_models(InterpJob J) {
     constexpr int SP = kSeedsPerWarp, W = 32 / SP;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
