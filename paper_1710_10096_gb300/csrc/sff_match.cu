@@ -144,7 +144,6 @@ constexpr unsigned kInfBits = 0x7f800000u;   // +inf
 constexpr int kMaxFiniteBits = 0x7f7fffff;   // largest finite float
 
 __host__ __device__ __forceinline__ int tc_rows(int gq) { return (gq + kTcRows - 1) / kTcRows * kTcRows; }
-__host__ __device__ __forceinline__ int tc_cand_rows(int gq) { return (gq + kTcCand - 1) / kTcCand * kTcCand; }
 
 // Writes the augmented bf16 rows of the reference (role 0: queries) and
 // temporal (role 1: candidates) coarsest-grid points; rows past gq are zero.
@@ -154,7 +153,7 @@ __global__ void k_gather_grid(const __grid_constant__ Fields F, int n) {
     dependent_start();
     const Field& A = pick(F);
     const int role = blockIdx.y;
-    const int rows = role ? tc_cand_rows(A.gq) : tc_rows(A.gq);
+    const int rows = tc_rows(A.gq);
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (role >= 2) {
         // roles 2, 3: compact int8 records of the stereo and cross images
@@ -198,8 +197,8 @@ __global__ void k_gather_grid(const __grid_constant__ Fields F, int n) {
         w[k] = *reinterpret_cast<const uint32_t*>(&h);
     }
     uint8_t* base = A.tk + (role ? (size_t)tc_rows(A.gq) * (kTcK * 2) : 0);
-    const int tile = role ? kTcCand : kTcRows;
-    const size_t off = (size_t)(r / tile) * tile * (kTcK * 2) + (size_t)kg * tile * 16 + ((r % tile) >> 3) * 128 + (r & 7) * 16;
+    const int tile = role ? kTcCand : kTcRows, start = r / tile * tile, held = min(tile, rows - start);
+    const size_t off = (size_t)start * (kTcK * 2) + (size_t)kg * held * 16 + ((r - start) >> 3) * 128 + (r & 7) * 16;
     *reinterpret_cast<uint4*>(base + off) = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
@@ -366,8 +365,16 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_knn_tc(const __grid_constant_
                     (*fail ||
                      !(ok = mbar_wait(&bar_empty[s], (unsigned)((u - kTcStages) / kTcStages) & 1u, wait_ns))))
                     break;
-                mbar_expect_tx(&bar_a[s], kTcTileBytes);
-                bulk_copy_g2s(sA + s * kTcTileBytes, gC + (size_t)(u % nt) * kTcTileBytes, kTcTileBytes, &bar_a[s]);
+                const uint8_t* from = gC + (size_t)(u % nt) * kTcTileBytes;
+                if (tc_rows(gq) - u % nt * kTcCand >= kTcCand) {
+                    mbar_expect_tx(&bar_a[s], kTcTileBytes);
+                    bulk_copy_g2s(sA + s * kTcTileBytes, from, kTcTileBytes, &bar_a[s]);
+                } else {  // half a tile: the scans drop the other columns, whatever they hold
+                    mbar_expect_tx(&bar_a[s], kTcTileBytes / 2);
+                    for (int kg = 0; kg < kTcK / 8; ++kg)
+                        bulk_copy_g2s(sA + s * kTcTileBytes + kg * kTcTileGroup, from + kg * (kTcTileGroup / 2),
+                                      kTcTileGroup / 2, &bar_a[s]);
+                }
             }
             if (!ok) {
                 *fail = 1;
@@ -2571,7 +2578,7 @@ FieldScratch field_scratch(int w, int h, const sff_params& p) {
     FieldScratch f;
     f.best8 = 0;
     f.tk = f.best8 + align256((size_t)gq * 8 * sizeof(int2));
-    f.rec = f.tk + align256(((size_t)tc_rows(gq) + tc_cand_rows(gq)) * kTcK * 2);
+    f.rec = f.tk + align256((size_t)2 * tc_rows(gq) * kTcK * 2);
     f.rec_n = f.rec + align256((size_t)2 * gq * kFeat);
     f.field = f.rec_n + align256((size_t)2 * gq * sizeof(int));
     f.cost = f.field + align256((size_t)w * h * 8);
@@ -2706,7 +2713,7 @@ int run_fields(const FieldSpec* spec, int nf, const sff_params& P, const sff_tun
             mgq = std::max(mgq, F.f[k].gq);
         }
         if (s == S - 1) {
-            dim3 g0((tc_cand_rows(mgq) * 8 + 255) / 256, 4, nf);
+            dim3 g0((tc_rows(mgq) * 8 + 255) / 256, 4, nf);
             SFF_LAUNCH_DEPENDENT(k_gather_grid, g0, 256, 0, st, F, n);
             if (!knn_smem_ready()) return SFF_ERR_CUDA;
             if (fork_hook) {
@@ -2924,7 +2931,7 @@ int run_field_sift(const FieldSpec& fs, const float* const* phi, const sff_param
                         plane_of(fs.crs, s, S, w, h), w, h, fs.mirror ? -1 : 1};
             A.gw = gw;
             A.gh = gh;
-            dim3 g0((tc_cand_rows(A.gq) * 8 + 255) / 256, 4, 1);
+            dim3 g0((tc_rows(A.gq) * 8 + 255) / 256, 4, 1);
             SFF_LAUNCH(k_gather_grid, g0, 256, 0, st, F, N);
             if (!knn_smem_ready()) return SFF_ERR_CUDA;
             dim3 g1((A.gq + kTcRows - 1) / kTcRows, 1, 1);
