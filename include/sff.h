@@ -452,8 +452,9 @@ int sff_sift_features(const uint8_t* const* rgb_dev4, int32_t pitch_bytes, int32
  * (temporal, stereo, cross) rank order winning.  phi_*_dev: [S][H][W][4]
  * float of the views in the field's roles.  cost_dev receives each float
  * cost as its int32 bit pattern (non-negative floats order like their bit
- * patterns; SFF_EMPTY_COST stays the empty marker).  Workspace as
- * sff_match_views. */
+ * patterns; SFF_EMPTY_COST stays the empty marker).  Workspace of
+ * sff_workspace_bytes(); in a smaller one that is enough for sff_match_views,
+ * 64 bytes per pixel are allocated and freed in stream order on each call. */
 int sff_match_views_sift(const uint8_t* pyr_ref_dev, const uint8_t* pyr_temporal_dev,
                          const uint8_t* pyr_stereo_dev, const uint8_t* pyr_cross_dev, const float* phi_ref_dev,
                          const float* phi_temporal_dev, const float* phi_stereo_dev, const float* phi_cross_dev,

@@ -48,6 +48,8 @@ extern "C" size_t sff_workspace_bytes(int32_t width, int32_t height, const sff_p
     size_t m = sff::match_ws_bytes(width, height, *params);
     size_t f = sff::filter_ws_bytes(width, height);
     size_t s = sff::seeds_ws_bytes(width, height);
+    size_t t = sff::sift_match_ws_bytes(width, height, *params);
+    if (t > b) b = t;
     if (m > b) b = m;
     if (f > b) b = f;
     if (s > b) b = s;

@@ -322,6 +322,7 @@ int check_size(int w, int h);
 int check_params(const sff_params* p);
 size_t features_ws_bytes(int w, int h, const sff_params& p);
 size_t match_ws_bytes(int w, int h, const sff_params& p);
+size_t sift_match_ws_bytes(int w, int h, const sff_params& p);
 size_t filter_ws_bytes(int w, int h);
 size_t seeds_ws_bytes(int w, int h);
 int launch_status();

@@ -2599,10 +2599,13 @@ size_t sift_pack_bytes(int w, int h, const sff_params& p) {
     return n > 1 ? align256((size_t)4 * h * ((w + n - 1) / n * n) * 16) : 0;
 }
 
-// Workspace of the matching calls: the scratch of two fields (sff_match_quad)
-// or of one and the repacked phi.
-size_t match_ws_bytes(int w, int h, const sff_params& p) {
-    return field_ws_bytes(w, h, p) + std::max(field_ws_bytes(w, h, p), sift_pack_bytes(w, h, p));
+// Workspace that the matching calls need: the scratch of two fields
+// (sff_match_quad).
+size_t match_ws_bytes(int w, int h, const sff_params& p) { return 2 * field_ws_bytes(w, h, p); }
+
+// Workspace of sff_match_views_sift with room for the repacked phi.
+size_t sift_match_ws_bytes(int w, int h, const sff_params& p) {
+    return field_ws_bytes(w, h, p) + sift_pack_bytes(w, h, p);
 }
 
 // Opts k_knn_tc into its dynamic shared memory, once per device.
@@ -2881,7 +2884,7 @@ int run_fields(const FieldSpec* spec, int nf, const sff_params& P, const sff_tun
 // in run_fields, then initialisation, inheritance, half-steps and random
 // search in the kernels above.  phi[4]: [S][H][W] float4 of the views in the
 // field's roles (reference, temporal, stereo, cross).
-int run_field_sift(const FieldSpec& fs, const float* const* phi, const sff_params& P, cudaStream_t st) {
+int run_field_sift(const FieldSpec& fs, const float* const* phi, const sff_params& P, void* pack, cudaStream_t st) {
     const int S = P.num_scales, I = P.iterations, w = fs.width, h = fs.height;
     static const int kDirs[4][2] = {{1, 1}, {-1, -1}, {1, -1}, {-1, 1}};
     static Fields F;
@@ -2920,7 +2923,7 @@ int run_field_sift(const FieldSpec& fs, const float* const* phi, const sff_param
         SV.sigma = fs.mirror ? -1 : 1;
         SV.m = (w + N - 1) / N;
         SV.pitch = N * SV.m;
-        SP.packed = reinterpret_cast<float4*>(ws + sc.total);
+        SP.packed = reinterpret_cast<float4*>(pack);
         for (int k = 0; k < 4; ++k) {
             SP.v[k] = reinterpret_cast<const float4*>(phi[k]) + off;
             SV.v[k] = N > 1 ? SP.packed + (size_t)k * h * SV.pitch : SP.v[k];
@@ -3158,5 +3161,18 @@ extern "C" int sff_match_views_sift(const uint8_t* pyr_ref_dev, const uint8_t* p
     if (workspace_bytes < match_ws_bytes(width, height, *params)) return SFF_ERR_WORKSPACE;
     FieldSpec f{pyr_ref_dev, pyr_temporal_dev, pyr_stereo_dev, pyr_cross_dev, field_dev, cost_dev, mirror,
                 width, height, seed, workspace};
-    return run_field_sift(f, phi, *params, (cudaStream_t)stream);
+    // a workspace of two fields' scratch is enough: the repacked phi is then
+    // allocated and freed in stream order
+    const cudaStream_t st = (cudaStream_t)stream;
+    void *pack = reinterpret_cast<char*>(workspace) + field_ws_bytes(width, height, *params), *own = nullptr;
+    if (workspace_bytes < sift_match_ws_bytes(width, height, *params)) {
+        if (cudaMallocAsync(&own, sift_pack_bytes(width, height, *params), st) != cudaSuccess) {
+            cudaGetLastError();
+            return SFF_ERR_WORKSPACE;
+        }
+        pack = own;
+    }
+    const int rc = run_field_sift(f, phi, *params, pack, st);
+    if (own && cudaFreeAsync(own, st) != cudaSuccess && rc == SFF_OK) return SFF_ERR_CUDA;
+    return rc;
 }

@@ -141,3 +141,50 @@ def test_sift_fields_at_tile_edges(w, h, S, knn_t, knn_e):
         wf, wc = oracle.match_views_sift(*[feats[k] for k in order], *[phis[k] for k in order], w, h, mirror, 77, op)
         assert np.array_equal(cost.cpu().numpy(), wc)
         assert np.array_equal(field.cpu().numpy(), wf)
+
+
+@pytest.mark.parametrize("w,h", [(64, 40), (37, 23)])
+def test_workspace_of_two_fields_gives_the_same_field(w, h):
+    """A workspace without room for the repacked phi: the scratch of the WHT
+    matching calls, 39 to 64 bytes per pixel at four scales, is enough for both."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1710_10096_gb300 as sff
+    sff.build()
+    p = sff.default_params(num_scales=4)
+    dev = [torch.as_tensor(np.ascontiguousarray(im)).cuda() for im in scenegen.random_images(w, h, seed=5, n=4)]
+    full = torch.empty(sff.workspace_bytes(w, h, p), dtype=torch.uint8, device="cuda")
+    pyr = [torch.empty(sff.pyramid_bytes(w, h, p), dtype=torch.uint8, device="cuda") for _ in range(4)]
+    for im, q in zip(dev, pyr):
+        sff.features(im, q, full, p)
+    phis = [torch.empty((4, h, w, 4), dtype=torch.float32, device="cuda") for _ in range(4)]
+    sff.sift_features(dev, phis, torch.empty(sff.sift_workspace_bytes(w, h), dtype=torch.uint8, device="cuda"), p)
+
+    def field(call, ws):
+        f = torch.empty((h, w, 4), dtype=torch.int16, device="cuda")
+        c = torch.empty((h, w), dtype=torch.int32, device="cuda")
+        call(f, c, ws)
+        torch.cuda.synchronize()
+        return f, c
+
+    def sift(f, c, ws):
+        sff.match_views_sift(*pyr, *phis, w, h, 0, 7, f, c, ws, p)
+
+    def wht(f, c, ws):
+        sff.match_views(*pyr, w, h, 0, 7, f, c, ws, p)
+
+    # the smallest workspace that sff_match_views takes
+    lo, hi = 0, full.numel()
+    while lo < hi:
+        mid = (lo + hi) // 2 // 256 * 256
+        try:
+            field(wht, full[:mid])
+            hi = mid
+        except sff.SffError:
+            lo = mid + 256
+    assert lo < full.numel()
+    for a, b in zip(field(sift, full), field(sift, full[:lo].clone())):
+        assert torch.equal(a, b)
+    with pytest.raises(sff.SffError):
+        field(sift, full[: lo - 256])
