@@ -508,10 +508,11 @@ size_t sff_interp_workspace_bytes(int32_t width, int32_t height, int32_t capacit
  * during the call.  The seeds must lie in the image with at most one seed per
  * 3x3 block anchored at (0, 0), as sff_emit_seeds writes them.
  * Errors found on the GPU (a second seed in one block, a seed outside the
- * image, or more than 6 * max(k_geo, k_motion) + 224 neighbour candidates of
- * one seed tied at the k-th distances, which the candidate buffer's
- * compaction cannot reduce) set bits of a status word in the workspace (read
- * it with sff_interp_status) and the field is all zeros. */
+ * image, or, where 6 * max(k_geo, k_motion) + 256 < k_geo + k_motion + 544, so
+ * many neighbour candidates of one seed tied at the k-th distances that its
+ * members and they do not fit 6 * max(k_geo, k_motion) + 224 slots) set bits of
+ * a status word in the workspace (read it with sff_interp_status) and the field
+ * is all zeros. */
 int sff_interpolate(const sff_seed* seeds_dev, const int32_t* count_dev, int32_t capacity, int32_t width,
                     int32_t height, const sff_interp_params* params, float* field_dev, void* workspace,
                     size_t workspace_bytes, void* stream);

@@ -59,12 +59,14 @@ constexpr int kTighten = 4;          // the ring bound is within 1/16 of the k-t
 // 4/pi times k seeds plus a margin of whole rings; 4 k + 192 leaves room for uneven
 // seed density (with k = 160, a lone seed in the middle of a 480 x 480 px hole in a
 // dense seed lattice meets 833).  What does not fit is compacted to the members of
-// both sets so far, k_geo + k_motion and those tied at the larger distance (a circle
-// within an image of 16384 px has at most 288 lattice points), and a batch of 32 more.
-// With 6 k + 256 an SM held 16 warps instead of 20: 659 -> 622 us, and 612 with one
-// warp per CTA, whose resources are free as soon as it ends.
+// both sets so far: at most k_geo - 1 + k_motion - 1 and those tied at either k-th
+// distance, 256 each (the most lattice points on a circle that fit an image of 16384
+// x 16384 px, counted), and a batch of 32 more.  `whole` slots always hold these; for
+// small k 6 k + 256 slots are fewer, and candidates that do not fit raise
+// kErrOverflow.  With 6 k + 256 at k = 160 an SM held 16 warps instead of 20: 659 ->
+// 622 us, and 612 with one warp per CTA, whose resources are free as soon as it ends.
 __host__ __device__ __forceinline__ int candidate_slots(int kg, int km) {
-    const int k = kg > km ? kg : km, whole = kg + km + 352;
+    const int k = kg > km ? kg : km, whole = kg + km + 2 * 256 + 32;
     const int slots = 6 * k + 256 < whole ? 6 * k + 256 : whole > 4 * k + 192 ? whole : 4 * k + 192;
     return (slots + 31) & ~31;
 }
@@ -456,6 +458,7 @@ __device__ __forceinline__ bool select_neighbours(const InterpJob& J, int si, in
     // k-th smallest distances of the candidates so far bound the final ones
     // from above (more candidates only lower them), so the candidates beyond
     // them are no members and are dropped, keeping the others in scan order.
+    // far_a and far_m have to cover every candidate counted in fa and fm.
     auto compact = [&]() {
         const Candidates Cc{pos, word, fill};
         unsigned DA = bound_a, DM = bound_m;
@@ -515,6 +518,9 @@ __device__ __forceinline__ bool select_neighbours(const InterpJob& J, int si, in
                 }
             }
             if (fill + __popc(__ballot_sync(kFull, w >= 0)) > J.slots) {
+                // fa and fm count this ring's seeds already: a set may owe its k-th to them
+                far_a = max(far_a, __reduce_max_sync(kFull, ma));
+                far_m = max(far_m, __reduce_max_sync(kFull, mm));
                 compact();
                 if (w >= 0 && !(d2 <= bound_a || (word_motion(w) && d2 <= bound_m))) w = -1;
             }
