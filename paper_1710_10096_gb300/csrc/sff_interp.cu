@@ -50,6 +50,7 @@ namespace {
 
 constexpr int kBlock = 3;            // sparsification block of Sec. 3.2
 constexpr int kModelWarps = 1;       // warps per CTA of k_interp_models
+constexpr int kModelResident = 20;   // ... and CTAs per SM that its registers allow
 constexpr int kSeedsPerWarp = 2;     // seeds whose sums share a warp's instructions (16 lanes each)
 constexpr int kMaxK = 1024;          // largest k_geo / k_motion
 constexpr int kRegKeys = 16;         // candidate keys per lane held in registers during selection (half are, up to 256)
@@ -76,6 +77,7 @@ constexpr int kSumDoubles = 32;      // plane sums 9, motion N 10 and R 12, pad
 constexpr int kWeightTable = 1 << 16;
 constexpr unsigned kErrSeed = 1u, kErrOverflow = 2u;
 constexpr unsigned kFull = 0xffffffffu;
+constexpr int kSms = 152, kSmemPerSm = 228 * 1024, kSmemPerCta = 1024;  // shared memory of an SM, and reserved per CTA
 
 // Map word of a block: (seed index << 5) | (motion << 4) | (ox << 2) | oy,
 // (ox, oy) the seed's offset inside its block; -1 for an empty block.
@@ -93,9 +95,11 @@ struct InterpJob {
     double* sums;      // [capacity][kSumDoubles] normal equations
     int* motion;       // [capacity] motion neighbours
     unsigned* status;  // error bits
+    int* lone_max;     // k_interp_models takes one seed per warp up to this many (see there)
     sff_interp_params p;
     double fb, inv_f;  // focal * baseline, 1 / focal
     int slots;         // candidate slots per warp of k_interp_models
+    int resident;      // warps of k_interp_models that the GPU holds at once
 };
 
 __device__ __forceinline__ int seed_count(const InterpJob& J) { return min(*J.count, J.capacity); }
@@ -108,7 +112,12 @@ __global__ void k_interp_clear(InterpJob J) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < J.gbw * J.gbh) J.map[i] = -1;
     if (i < kWeightTable) J.wt[i] = exp(-J.p.alpha * sqrt((double)i) / J.p.dist_unit);
-    if (i == 0) *J.status = 0u;
+    if (i == 0) {
+        const int n = seed_count(J);
+        *J.status = 0u;
+        const bool lone = n <= J.resident || (n > 2 * J.resident && n <= J.resident * 10 / 3) || 2 * n < J.gbw * J.gbh;
+        *J.lone_max = lone ? n : -1;
+    }
 }
 
 // Pinhole triangulation: Z = f B / d, X = (x - cx) Z / f, Y = (y - cy) Z / f.
@@ -601,12 +610,29 @@ __device__ __forceinline__ bool select_neighbours(const InterpJob& J, int si, in
 // additions; 174 instead of 221 FP64 instructions per seed.  1242 x 375, default
 // neighbourhoods: 778 -> 714 us (with the disparity fill's seeds 989 -> 879); four
 // seeds per warp 887: their lists leave 12 warps per SM.
-__global__ void __launch_bounds__(kModelWarps * 32, 20) k_interp_models(InterpJob J) {
+// Two each only where that is the better split, in us the call with two / one each
+// (n seeds; R warps resident, SMs x 20 = 3040 at the default k):
+//   - one each up to R, where every seed has a warp of its own at once (n = 368 102 /
+//     75, 2885 122 / 104);
+//   - two each up to 2 R, one round of the GPU instead of two (3691 126 / 135, 5105 145
+//     / 150);
+//   - one each again up to 10 R / 3, where the second round of two each is short (6774
+//     209 / 189, 10009 257 / 249), and two each from there on (10856 226 / 240, 36976
+//     632 / 684);
+//   - but one each at any number of sparse seeds, fewer than half of the blocks: their
+//     selections, which scan more rings, then outweigh the sums, and differ more from
+//     warp to warp (4693 on 39195 blocks 352 / 313, 15110 on 51750 533 / 461, 59975 on
+//     122574 1287 / 1306; 16012 on 30000, above half, 402 / 393).
+__global__ void __launch_bounds__(kModelWarps * 32, kModelResident) k_interp_models(InterpJob J) {
     constexpr int SP = kSeedsPerWarp, W = 32 / SP;
+    static_assert(SP == 2, "a lone seed's sums are in two halves");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int s0 = (blockIdx.x * kModelWarps + wid) * SP;
     const int n = seed_count(J);
+    // one seed, its sums over all lanes (the line as a word of its own: with the rule's
+    // comparisons here the kernel took 1 % more)
+    const bool lone = n <= *J.lone_max;
+    const int s0 = (blockIdx.x * kModelWarps + wid) * (lone ? 1 : SP);
     if (s0 >= n) return;  // warp-uniform
     const int kg = J.p.k_geo, km = J.p.k_motion;
     unsigned char* mine = smem_raw + (size_t)wid * warp_smem_bytes(J.slots, kg, km);
@@ -614,11 +640,13 @@ __global__ void __launch_bounds__(kModelWarps * 32, 20) k_interp_models(InterpJo
     int* word = reinterpret_cast<int*>(mine + (size_t)J.slots * 4);
     uint2* lists = reinterpret_cast<uint2*>(mine + (size_t)J.slots * 8);
     int* scratch = reinterpret_cast<int*>(lists + SP * (kg + km));
-    const int sub = lane / W, l = lane % W, si = s0 + sub;  // this lane's seed
+    const int sub = lone ? 0 : lane / W, l = lane % W, si = s0 + sub;  // this lane's seed
+    const int first = lone ? lane : l, step = lone ? 32 : W;          // its neighbours
+    const auto halves = [&](double& v) { v += __shfl_xor_sync(kFull, v, W); };
     int na = 0, nm = 0;
 #pragma unroll 1
     for (int k = 0; k < SP; ++k) {
-        if (s0 + k >= n) break;
+        if (s0 + k >= n || (lone && k > 0)) break;
         int a, m;
         uint2* la = lists + k * (kg + km);
         if (!select_neighbours(J, s0 + k, n, pos, word, scratch, la, la + kg, a, m, lane)) {
@@ -638,7 +666,7 @@ __global__ void __launch_bounds__(kModelWarps * 32, 20) k_interp_models(InterpJo
     double g[16];
 #pragma unroll
     for (int k = 0; k < 16; ++k) g[k] = 0.0;
-    for (int t = l; t < na; t += W) {
+    for (int t = first; t < na; t += step) {
         const uint2 c = la[t];
         int dx, dy;
         const unsigned d2 = cand_d2(c.x, dx, dy);
@@ -656,7 +684,7 @@ __global__ void __launch_bounds__(kModelWarps * 32, 20) k_interp_models(InterpJo
         g[7] += w1 * d;
         g[8] += wt * d;
     }
-    for (int t = l; t < nm; t += W) {
+    for (int t = first; t < nm; t += step) {
         const uint2 c = lm[t];
         int dx, dy;
         const unsigned d2 = cand_d2(c.x, dx, dy);
@@ -669,6 +697,7 @@ __global__ void __launch_bounds__(kModelWarps * 32, 20) k_interp_models(InterpJo
     }
     __syncwarp();
     reduce_scatter<16, W>(g, lane);
+    if (lone) halves(g[0]);
     auto value = [&](int k) { return __shfl_sync(kFull, g[0], sub * W + k); };  // on lane k of the group
     double cen[3] = {0.0, 0.0, 0.0};
     {
@@ -686,7 +715,7 @@ __global__ void __launch_bounds__(kModelWarps * 32, 20) k_interp_models(InterpJo
     double a[kSums];
 #pragma unroll
     for (int k = 0; k < kSums; ++k) a[k] = 0.0;
-    for (int t = l; t < nm; t += W) {
+    for (int t = first; t < nm; t += step) {
         const uint2 c = lm[t];
         int dx, dy;
         const unsigned d2 = cand_d2(c.x, dx, dy);
@@ -706,9 +735,13 @@ __global__ void __launch_bounds__(kModelWarps * 32, 20) k_interp_models(InterpJo
     }
     __syncwarp();
     reduce_scatter<kSums, W>(a, lane);
+    if (lone) {
+#pragma unroll
+        for (int i = 0; i < kSums / W; ++i) halves(a[i]);
+    }
 
     // the sums go to k_interp_solve: plane sums first, then N and R
-    if (si >= n) return;
+    if (si >= n || (lone && lane >= W)) return;
     double* sums = J.sums + (size_t)si * kSumDoubles;
     if (l < 9) sums[l] = g[0];
 #pragma unroll
@@ -991,21 +1024,26 @@ extern "C" int sff_interpolate(const sff_seed* seeds_dev, const int32_t* count_d
     J.sums = reinterpret_cast<double*>(ws + L.sums);
     J.motion = reinterpret_cast<int*>(ws + L.motion);
     J.status = reinterpret_cast<unsigned*>(ws + L.status);
+    J.lone_max = reinterpret_cast<int*>(J.status + 1);
     J.p = *params;
     J.fb = params->focal * params->baseline;
     J.inv_f = 1.0 / params->focal;
     J.slots = candidate_slots(params->k_geo, params->k_motion);
+    const size_t smem = kModelWarps * warp_smem_bytes(J.slots, J.p.k_geo, J.p.k_motion);
+    J.resident = kModelWarps * kSms * min(kModelResident, (int)(kSmemPerSm / (smem + kSmemPerCta)));
     cudaStream_t st = (cudaStream_t)stream;
     const int clear = max(J.gbw * J.gbh, kWeightTable);
     SFF_LAUNCH(k_interp_clear, dim3((clear + 255) / 256), 256, 0, st, J);
     if (capacity > 0) {
         SFF_LAUNCH(k_interp_prep, dim3((capacity + 255) / 256), 256, 0, st, J);
-        const size_t smem = kModelWarps * warp_smem_bytes(J.slots, J.p.k_geo, J.p.k_motion);
         if (smem > 48 * 1024 &&
             cudaFuncSetAttribute(k_interp_models, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
             return SFF_ERR_CUDA;
-        constexpr int kPer = kModelWarps * kSeedsPerWarp;
-        SFF_LAUNCH(k_interp_models, dim3((capacity + kPer - 1) / kPer), kModelWarps * 32, smem, st, J);
+        // enough warps for either split; those without a seed leave at once
+        const int lone = min(capacity, max(J.resident * 10 / 3, J.gbw * J.gbh / 2));
+        const int warps = max((capacity + kSeedsPerWarp - 1) / kSeedsPerWarp, lone);
+        const int blocks = (warps + kModelWarps - 1) / kModelWarps;
+        SFF_LAUNCH(k_interp_models, dim3(blocks), kModelWarps * 32, smem, st, J);
         SFF_LAUNCH(k_interp_solve, dim3((capacity + 63) / 64, 2), 64, 0, st, J);
     }
     int2* col = reinterpret_cast<int2*>(ws + L.nearest);
