@@ -432,7 +432,8 @@ int sff_emit_seeds_noalloc(const int16_t* fwd_dev, const int32_t* fwd_cost_dev,
 /* Scratch of sff_sift_features: about 2052 bytes per pixel up to 2^21 pixels,
  * 516 above; 0 for invalid sizes.  With the descriptors of every scale in it
  * the coarser scales' are computed while the axes are, on a second stream of
- * the library (one per device and caller stream); 516 bytes per pixel are
+ * the library (one per device and caller stream, and for cudaStreamPerThread
+ * one per device and thread); 516 bytes per pixel are
  * enough for any image (the scales then follow one another, same results). */
 size_t sff_sift_workspace_bytes(int32_t width, int32_t height);
 

@@ -665,31 +665,57 @@ int scratch_scales(int w, int h) { return (size_t)w * h <= kOverlapPixels ? SFF_
 struct AxesStream {
     cudaStream_t s = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
-    std::mutex mu;  // held from a call's fork to its join: threads may share the handle (cudaStreamPerThread)
+    std::mutex mu;  // held from a call's fork to its join: threads may share the caller's stream
+
+    bool make() {
+        int lo = 0, hi = 0;
+        if (cudaDeviceGetStreamPriorityRange(&lo, &hi) == cudaSuccess &&
+            cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, hi) == cudaSuccess &&
+            cudaEventCreateWithFlags(&fork, cudaEventDisableTiming) == cudaSuccess &&
+            cudaEventCreateWithFlags(&join, cudaEventDisableTiming) == cudaSuccess)
+            return true;
+        release();
+        cudaGetLastError();
+        return false;
+    }
+    void release() {
+        if (join) cudaEventDestroy(join);
+        if (fork) cudaEventDestroy(fork);
+        if (s) cudaStreamDestroy(s);
+    }
 };
 constexpr size_t kMaxAxesStreams = 64;  // further caller streams run everything in order
 std::mutex g_axes_mu;
 std::map<std::pair<int, cudaStream_t>, AxesStream> g_axes;
 
-AxesStream* axes_stream(cudaStream_t st) {
-    int dev = 0, lo = 0, hi = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
-    std::lock_guard<std::mutex> lk(g_axes_mu);
-    const auto it = g_axes.find({dev, st});
-    if (it != g_axes.end()) return &it->second;
-    if (g_axes.size() >= kMaxAxesStreams) return nullptr;
-    AxesStream& a = g_axes[{dev, st}];
-    if (cudaDeviceGetStreamPriorityRange(&lo, &hi) != cudaSuccess ||
-        cudaStreamCreateWithPriority(&a.s, cudaStreamNonBlocking, hi) != cudaSuccess ||
-        cudaEventCreateWithFlags(&a.fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&a.join, cudaEventDisableTiming) != cudaSuccess) {
-        if (a.fork) cudaEventDestroy(a.fork);
-        if (a.s) cudaStreamDestroy(a.s);
-        g_axes.erase({dev, st});
-        cudaGetLastError();
-        return nullptr;
+// cudaStreamPerThread names another stream in each thread, so its side streams (by
+// device) belong to the thread and end with it.  One for all threads would stay part
+// of a capture in one of them while another's call forks to it.
+struct ThreadAxes {
+    std::map<int, AxesStream> by_device;
+    ~ThreadAxes() {
+        for (auto& e : by_device) e.second.release();
     }
-    return &a;
+};
+thread_local ThreadAxes t_axes;
+
+template <class Map, class Key>
+AxesStream* made_axes(Map& m, const Key& key) {
+    const auto it = m.find(key);
+    if (it != m.end()) return &it->second;
+    if (m.size() >= kMaxAxesStreams) return nullptr;
+    AxesStream& a = m[key];
+    if (a.make()) return &a;
+    m.erase(key);
+    return nullptr;
+}
+
+AxesStream* axes_stream(cudaStream_t st) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    if (st == cudaStreamPerThread) return made_axes(t_axes.by_device, dev);
+    std::lock_guard<std::mutex> lk(g_axes_mu);
+    return made_axes(g_axes, std::make_pair(dev, st));
 }
 
 }  // namespace
