@@ -149,7 +149,8 @@ typedef struct sff_tuning {
                               * 0, or 32x16 with 3, or 32x8 with 7; 0 or 1 */
     int32_t overlap;         /* 1: in sff_run_batch, the features of the scales below the
                               * coarsest are computed on a second stream of the library (one
-                              * per device and caller stream), forked once the coarsest grid
+                              * per device and caller stream, and for cudaStreamPerThread one
+                              * per device and thread), forked once the coarsest grid
                               * is gathered, while the K-NN and the coarse scales match; each
                               * scale's inheritance waits for its features.  0: every launch
                               * on the caller's stream.  Same results; under stream capture

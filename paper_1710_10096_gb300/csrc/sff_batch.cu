@@ -35,28 +35,54 @@ struct SideStream {
     cudaStream_t s = nullptr;
     cudaEvent_t fork = nullptr;
     cudaEvent_t ready[SFF_MAX_SCALES] = {};
+
+    bool make() {
+        bool ok = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess &&
+                  cudaEventCreateWithFlags(&fork, cudaEventDisableTiming) == cudaSuccess;
+        for (int k = 0; ok && k < SFF_MAX_SCALES; ++k)
+            ok = cudaEventCreateWithFlags(&ready[k], cudaEventDisableTiming) == cudaSuccess;
+        if (ok) return true;
+        release();
+        cudaGetLastError();
+        return false;
+    }
+    void release() {
+        for (cudaEvent_t e : ready)
+            if (e) cudaEventDestroy(e);
+        if (fork) cudaEventDestroy(fork);
+        if (s) cudaStreamDestroy(s);
+    }
 };
 
 std::mutex g_side_mu;
 std::map<std::pair<int, cudaStream_t>, SideStream> g_side;
 
+// cudaStreamPerThread names another stream in each thread, so its sets (by device)
+// belong to the thread and end with it: threads sharing one would reuse its events at
+// once, and fork to a stream that is part of another thread's capture.
+struct ThreadSides {
+    std::map<int, SideStream> by_device;
+    ~ThreadSides() {
+        for (auto& e : by_device) e.second.release();
+    }
+};
+thread_local ThreadSides t_sides;
+
+template <class Map, class Key>
+const SideStream* made_side(Map& m, const Key& key) {
+    const auto it = m.find(key);
+    if (it != m.end()) return &it->second;
+    SideStream ss;
+    return ss.make() ? &m.emplace(key, ss).first->second : nullptr;
+}
+
 // The set of the current device and `st`, or nullptr when it cannot be made.
 const SideStream* side_stream(cudaStream_t st) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    if (st == cudaStreamPerThread) return made_side(t_sides.by_device, dev);
     std::lock_guard<std::mutex> lk(g_side_mu);
-    auto it = g_side.find({dev, st});
-    if (it != g_side.end()) return &it->second;
-    SideStream ss;
-    bool ok = cudaStreamCreateWithFlags(&ss.s, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaEventCreateWithFlags(&ss.fork, cudaEventDisableTiming) == cudaSuccess;
-    for (int k = 0; ok && k < SFF_MAX_SCALES; ++k)
-        ok = cudaEventCreateWithFlags(&ss.ready[k], cudaEventDisableTiming) == cudaSuccess;
-    if (!ok) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    return &g_side.emplace(std::make_pair(dev, st), ss).first->second;
+    return made_side(g_side, std::make_pair(dev, st));
 }
 
 // The feature overlap of one sff_run_batch call (sff_tuning.overlap).

@@ -94,3 +94,18 @@ def test_sift_features(env):
     _beside_a_capture(torch, *calls)
     for o in outs[1:]:
         assert all(torch.equal(a, b) for a, b in zip(outs[0], o))
+
+
+def test_run_batch(env):
+    torch, sff = env
+    q = scenegen.make_quad("planes", 161, 83, 6)
+    dev = [torch.as_tensor(im).cuda() for im in q.images()]
+    ms = [sff.QuadMatcher(q.width, q.height) for _ in range(3)]
+    for m in ms:
+        m.seeds.zero_()
+    ms[0].run(*dev, seed=3)
+    torch.cuda.synchronize()
+    _beside_a_capture(torch, *[lambda m=m: m.run(*dev, seed=3, stream=PerThread()) for m in ms[1:]])
+    for m in ms[1:]:
+        for what in ("fwd", "fwd_cost", "inv", "inv_cost", "keep", "cerr", "seeds", "count"):
+            assert torch.equal(getattr(ms[0], what), getattr(m, what)), what
