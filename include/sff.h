@@ -139,7 +139,9 @@ typedef struct sff_tuning {
                               * (2,0,32x8,0), (1,1,32x16,0), (1,1,32x8,0), (1,1,16x8,0),
                               * (1,1,8x8,0), (2,1,32x8,0), (2,1,16x8,0), (2,1,8x8,0),
                               * (1,4,16x8,0), (1,4,8x8,0), (2,4,8x8,0); bit 0 clear, and no
-                              * bit shared with pdl or alternate_order; 0..14.  A
+                              * bit shared with pdl or alternate_order; 0..14.  Such a
+                              * launch waits until all its CTAs can be resident at once, so
+                              * it runs beside less of other streams' work.  A
                               * barrier wait that runs out (1 s) raises SFF_ERR_TIMEOUT in
                               * sff_device_status. */
     int32_t tma;             /* 1: at scale 0 each CTA of the iteration kernel stages its

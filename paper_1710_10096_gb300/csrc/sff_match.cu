@@ -2523,10 +2523,14 @@ bool default_tuning(const sff_tuning& t) {
 // tuning leaves everything to the library; with any other, scale 0 takes the tuned
 // variant, a coarser scale its entry when one is given, and the schedule is the
 // tuning's.  The library's schedule (us the stage, other choice / this one):
-//   - in small stages the scales below the slot limit are fused into one
-//     cooperative launch each (512 x 160 478 / 461, 640 x 192 590 / 569; 900 x 300
-//     906 / 898); in larger ones the features still run beside them, whose CTAs
-//     the grid barriers wait for (1024 x 436 1324 / 1260, 1242 x 375 1399 / 1300);
+//   - in small stages the scales whose tiles (128 points) are no more than the SMs are
+//     fused into one cooperative launch each (256 x 80 373 / 351).  Such a launch waits
+//     until all its CTAs are resident at once, so it keeps other streams' kernels and
+//     its own stage's features from running beside it: with larger grids and stages,
+//     four streams of quads took longer (us a quad, every scale below the slot limit
+//     fused / this rule; 400 x 130 279 / 237, 640 x 192 430 / 384, 900 x 300 1042 /
+//     846), more than one stream gained (400 x 130 441 / 451, 640 x 192 543 / 561, 900
+//     x 300 914 / 908);
 //   - the others are dependent launches, which hide the launches' gaps (1242 x 375
 //     1732 / 1630 before the other changes), but not scales 2 and 3 of the
 //     largest stages, where the waiting CTAs take the features' place (1917 x 1083
@@ -2536,13 +2540,13 @@ bool default_tuning(const sff_tuning& t) {
 //     grid exceed half of L2, every other launch backwards (together 1395 / 1349
 //     and, 1917 x 1083, 6324 / 5901).
 constexpr double kAlternateBytes = 64e6;
-constexpr long kFuseStagePixPerSm = 4096, kDependentStagePixPerSm = 16384;
+constexpr long kFusePixPerSm = 128, kFuseStagePixPerSm = 768, kDependentStagePixPerSm = 16384;
 
 ScalePlan plan_scale(const sff_tuning& t, bool derive, bool capturing, int s, long px, long px0) {
     ScalePlan p;
     if (derive) {
         p.v = derived_variant(px);
-        p.fuse = s > 0 && p.v->slots > 0 && px0 / kSmCount < kFuseStagePixPerSm;
+        p.fuse = s > 0 && p.v->slots > 0 && px / kSmCount < kFusePixPerSm && px0 / kSmCount < kFuseStagePixPerSm;
         if (s == 0 && p.v->slots > 0) p.v = find_variant(1, 0, 32, 8, 0);  // 256 x 80: 597 / 524 us
         p.pdl = !p.fuse && !capturing && (s < 2 || px0 / kSmCount < kDependentStagePixPerSm);
         p.alternate = !p.fuse && 2.0 * kFeat * (double)px > kAlternateBytes;
