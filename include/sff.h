@@ -100,9 +100,11 @@ typedef struct sff_params {
  * s >= 1 takes coarse[s - 1] = {lanes, slots, tile_x, tile_y, min_ctas}; all zero means
  * derived from the grid pixels per SM over all fields of the launch: (1, 4, 16, 8,
  * 0) below 200, (1, 0, 32, 8, 7) from 1280 to 1792, else (1, 0, 32, 8, 0).
- * A tuning equal to sff_default_tuning's leaves every choice of the iterations to
- * the library, scale 0 and the schedules (pair_fields, alternate_order, pdl, fuse)
- * included: derived from the grid sizes in the same way.
+ * A tuning that differs from sff_default_tuning's in features_form and overlap at
+ * most leaves every choice of the iterations to the library, scale 0 and the
+ * schedules (pair_fields, alternate_order, pdl, fuse) included: derived from the
+ * grid sizes in the same way.  Any coarse entry (of a scale that is not run, with
+ * one scale) makes the default's other values explicit.
  * sff_tuning_supported() checks a setting. */
 typedef struct sff_tuning {
     int32_t lanes_per_pixel; /* threads that share one pixel's feature loads */

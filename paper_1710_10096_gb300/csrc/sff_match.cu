@@ -2513,14 +2513,18 @@ const IterVariant* derived_variant(long px) {
     return find_variant(1, 0, 32, 8, per >= kPixPerSmWaveLo && per < kPixPerSmWaveHi ? 7 : 0);
 }
 
-bool default_tuning(const sff_tuning& t) {
+// Whether the tuning leaves the iterations to the library: every field that describes
+// them is the default.  features_form and overlap do not.
+bool derives_iterations(const sff_tuning& t) {
     sff_tuning d;
     sff_default_tuning(&d);
+    d.features_form = t.features_form;
+    d.overlap = t.overlap;
     return memcmp(&t, &d, sizeof t) == 0;
 }
 
-// Scale s over px grid pixels of the launch's fields, px0 at scale 0.  The default
-// tuning leaves everything to the library; with any other, scale 0 takes the tuned
+// Scale s over px grid pixels of the launch's fields, px0 at scale 0.  `derive`:
+// everything is left to the library; else scale 0 takes the tuned
 // variant, a coarser scale its entry when one is given, and the schedule is the
 // tuning's.  The library's schedule (us the stage, other choice / this one):
 //   - in small stages the scales whose tiles (128 points) are no more than the SMs are
@@ -2632,7 +2636,7 @@ bool knn_smem_ready() {
 int run_fields(const FieldSpec* spec, int nf, const sff_params& P, const sff_tuning& T, cudaStream_t st,
                bool sequential, const cudaEvent_t* scale_ready, const ForkHook* fork_hook) {
     if (!tuning_valid(T) || nf < 1 || nf > kMaxFields) return SFF_ERR_ARG;
-    const bool derive = default_tuning(T);
+    const bool derive = derives_iterations(T);
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     const bool capturing = cudaStreamIsCapturing(st, &capture) == cudaSuccess && capture != cudaStreamCaptureStatusNone;
     const int S = P.num_scales, I = P.iterations;

@@ -35,3 +35,22 @@ def _fused_scales(w, h, tuning=None):
 ])
 def test_fused_scales_leave_room_for_other_streams(w, h, fused):
     assert _fused_scales(w, h) == fused
+
+
+@pytest.mark.parametrize("field,value,fused", [
+    ("overlap", 0, {1, 2, 3}), ("features_form", 1, {1, 2, 3}), ("features_form", 2, {1, 2, 3}),
+    # fields of the iterations: their setting as given
+    ("group_mb", 64, set()), ("pair_fields", 1, set()), ("alternate_order", 1, set()), ("pdl", 1, set()),
+])
+def test_only_iteration_fields_end_the_derived_schedule(field, value, fused):
+    import paper_1710_10096_gb300 as sff
+    sff.build()
+    t = sff.default_tuning()
+    setattr(t, field, value)
+    assert _fused_scales(256, 80, t) == fused
+
+
+def test_a_coarse_entry_makes_the_default_values_explicit():
+    import paper_1710_10096_gb300 as sff
+    sff.build()
+    assert _fused_scales(256, 80, sff.make_tuning(1, 32, 16, 0, [(1, 0, 32, 16)])) == set()
