@@ -2537,14 +2537,15 @@ bool derives_iterations(const sff_tuning& t) {
 //     x 300 914 / 908);
 //   - the others are dependent launches, which hide the launches' gaps (1242 x 375
 //     1732 / 1630 before the other changes), but not scales 2 and 3 of the
-//     largest stages, where the waiting CTAs take the features' place (1917 x 1083
-//     5446 / 5311), nor in a captured graph, whose gaps are short (the batch 23.4 /
-//     20.9 ms);
+//     largest stages, where the waiting CTAs take the features' place (with them / without:
+//     1242 x 375, 6128 points a SM, 1286 / 1329; 1500 x 700, 13815, 2668 / 2688; 1600 x
+//     800, 16842, 3259 / 3224; 1917 x 1083, 27317, 5329 / 5184), nor in a captured
+//     graph, whose gaps are short (the batch 23.4 / 20.9 ms);
 //   - a quad's two fields side by side and, where the four images' records of the
 //     grid exceed half of L2, every other launch backwards (together 1395 / 1349
 //     and, 1917 x 1083, 6324 / 5901).
 constexpr double kAlternateBytes = 64e6;
-constexpr long kFusePixPerSm = 128, kFuseStagePixPerSm = 768, kDependentStagePixPerSm = 16384;
+constexpr long kFusePixPerSm = 128, kFuseStagePixPerSm = 768, kDependentStagePixPerSm = 15000;
 
 ScalePlan plan_scale(const sff_tuning& t, bool derive, bool capturing, int s, long px, long px0) {
     ScalePlan p;
