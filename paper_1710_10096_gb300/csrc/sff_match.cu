@@ -1961,23 +1961,40 @@ __device__ __forceinline__ float root_in_range(float x) {
     return __fmaf_rn(__fmaf_rn(-g, g, x), __fmul_rn(0.5f, y), g);
 }
 
-// The sum of Eq. 1 for any values, one thread, by sqrt.rn (0 for 0).
+// The distances of column q - 3 of a candidate's window for any values, by sqrt.rn (0
+// for 0): row j's at d[21 j + 3 q].  Inlined: as a call it cost the common path 1.3 %.
 template <int N>
-__device__ float sift_cost_any(const SiftViews& S, int px, int py, const Vec4& a) {
-    auto get = [&](int k, int x, int y) {
-        return __ldg(S.v[k] + (size_t)clampi(y, 0, S.h - 1) * S.pitch + sift_slot<N>(clampi(x, 0, S.w - 1), S.m));
-    };
-    auto root = [](float d) { return d == 0.0f ? 0.0f : __fsqrt_rn(d); };
-    float c = 0.0f;
+__device__ __forceinline__ void sift_column_any(const SiftViews& S, float* d, int q, int px, int py, const Vec4& a) {
+    const int x = px + (q - 3) * N;
+    const int s0 = sift_slot<N>(clampi(x, 0, S.w - 1), S.m), s1 = sift_slot<N>(clampi(x + a.u, 0, S.w - 1), S.m),
+              s2 = sift_slot<N>(clampi(x - S.sigma * a.d0, 0, S.w - 1), S.m),
+              s3 = sift_slot<N>(clampi(x + a.u - S.sigma * a.d1, 0, S.w - 1), S.m);
+    auto root = [](float v) { return v == 0.0f ? 0.0f : __fsqrt_rn(v); };
 #pragma unroll 1
-    for (int k = 0; k < 49; ++k) {
-        const int x = px + (k % 7 - 3) * N, y = py + (k / 7 - 3) * N;
-        const float4 f = get(0, x, y);
-        c = __fadd_rn(c, root(sift_dist2(f, get(1, x + a.u, y + a.v))));
-        c = __fadd_rn(c, root(sift_dist2(f, get(2, x - S.sigma * a.d0, y))));
-        c = __fadd_rn(c, root(sift_dist2(f, get(3, x + a.u - S.sigma * a.d1, y + a.v))));
+    for (int j = 0; j < 7; ++j) {
+        const int y = py + (j - 3) * N;
+        const size_t r = (size_t)clampi(y, 0, S.h - 1) * S.pitch, t = (size_t)clampi(y + a.v, 0, S.h - 1) * S.pitch;
+        const float4 f = __ldg(S.v[0] + r + s0);
+        d[21 * j + 3 * q] = root(sift_dist2(f, __ldg(S.v[1] + t + s1)));
+        d[21 * j + 3 * q + 1] = root(sift_dist2(f, __ldg(S.v[2] + r + s2)));
+        d[21 * j + 3 * q + 2] = root(sift_dist2(f, __ldg(S.v[3] + t + s3)));
     }
-    return c;
+}
+
+constexpr int kSiftStride = 148;  // 147 distances, rows of whole 16 bytes
+
+// The sum of a candidate's 147 distances, in index order.
+template <int U>
+__device__ __forceinline__ float sift_sum(const float* buf) {
+    const float4* d = reinterpret_cast<const float4*>(buf);
+    float c = 0.0f;
+#pragma unroll U
+    for (int k = 0; k < 36; ++k) {
+        const float4 v = d[k];
+        c = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(c, v.x), v.y), v.z), v.w);
+    }
+    const float4 v = d[36];
+    return __fadd_rn(__fadd_rn(__fadd_rn(c, v.x), v.y), v.z);
 }
 
 // Eq. 1 of up to 8 candidates by one warp: 8 lanes per candidate, lane q taking
@@ -1988,9 +2005,11 @@ __device__ float sift_cost_any(const SiftViews& S, int px, int py, const Vec4& a
 // adds them in the definition's order.  at(k, px, py, vec): candidate k < n, the
 // same for the 8 lanes; n is warp-uniform.  Lane k < n returns candidate k's cost
 // as the float's bit pattern.  A candidate with a squared distance below the fast
-// root's range (a zero among them), or a sum that may hold one above it (then it
-// is at least 2^50 or no number), is evaluated again by the general form.
-constexpr int kSiftStride = 148;  // 147 distances, rows of whole 16 bytes
+// root's range (a zero among them: flat areas that the views share), or a sum that may
+// hold one above it (then it is at least 2^50 or no number), is scored again by the
+// general form, 8 lanes per candidate too: both fields of a 1242 x 375 quad whose upper
+// 30 % are saturated took 27.7 ms with one lane each, 13.4 so (20.4 with every root by
+// sqrt.rn); without flat areas 9.12 and 9.14.
 template <int N, class At>
 __device__ __forceinline__ int sift_costs(const SiftViews& S, float* buf, int lane, int n, At at) {
     const int g = lane >> 3, q = lane & 7, col = (min(q, 6) - 3) * N;
@@ -2028,24 +2047,22 @@ __device__ __forceinline__ int sift_costs(const SiftViews& S, float* buf, int la
         for (int k = 0; k < 4; ++k) slow |= (unsigned)(((low >> (8 * k)) & 0xffu) != 0) << (k0 + k);
     }
     __syncwarp();
-    float c = 0.0f;
-    if (lane < n) {
-        const float4* d = reinterpret_cast<const float4*>(buf + lane * kSiftStride);
-#pragma unroll 6
-        for (int k = 0; k < 36; ++k) {
-            const float4 v = d[k];
-            c = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(c, v.x), v.y), v.z), v.w);
-        }
-        const float4 v = d[36];
-        c = __fadd_rn(__fadd_rn(__fadd_rn(c, v.x), v.y), v.z);
-        if (((slow >> lane) & 1u) || !(c < kRootSumMax)) {
+    float c = lane < n ? sift_sum<6>(buf + lane * kSiftStride) : 0.0f;
+    __syncwarp();
+    slow |= __ballot_sync(0xffffffffu, lane < n && !(c < kRootSumMax));
+    if (__builtin_expect(slow != 0, 0)) {
+#pragma unroll 1
+        for (int k = g; k < n; k += 4) {
+            if (!((slow >> k) & 1u) || q == 7) continue;
             int px, py;
             Vec4 a;
-            at(lane, px, py, a);
-            c = sift_cost_any<N>(S, px, py, a);
+            at(k, px, py, a);
+            sift_column_any<N>(S, buf + k * kSiftStride, q, px, py, a);
         }
+        __syncwarp();
+        if ((slow >> lane) & 1u) c = sift_sum<2>(buf + lane * kSiftStride);
+        __syncwarp();
     }
-    __syncwarp();
     return __float_as_int(c);
 }
 
