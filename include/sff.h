@@ -459,8 +459,8 @@ int sff_sift_features(const uint8_t* const* rgb_dev4, int32_t pitch_bytes, int32
  * float of the views in the field's roles.  cost_dev receives each float
  * cost as its int32 bit pattern (non-negative floats order like their bit
  * patterns; SFF_EMPTY_COST stays the empty marker).  Workspace of
- * sff_workspace_bytes(); in a smaller one that is enough for sff_match_views,
- * 64 bytes per pixel are allocated and freed in stream order on each call. */
+ * sff_workspace_bytes(); a smaller one that is enough for sff_match_views will do
+ * (same results, slower: phi is then read in the caller's order). */
 int sff_match_views_sift(const uint8_t* pyr_ref_dev, const uint8_t* pyr_temporal_dev,
                          const uint8_t* pyr_stereo_dev, const uint8_t* pyr_cross_dev, const float* phi_ref_dev,
                          const float* phi_temporal_dev, const float* phi_stereo_dev, const float* phi_cross_dev,

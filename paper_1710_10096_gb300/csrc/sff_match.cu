@@ -1918,22 +1918,21 @@ __global__ void __launch_bounds__(256) k_random_search(const __grid_constant__ F
 // window row are then 112 contiguous bytes, one or two lines; in the caller's
 // order they lie in up to 7.  (Planes of 8 and 4 bytes in classes mod 2 n, made for
 // one candidate per lane, take 4 lines a row here: 9.4 against 8.9 ms for both
-// fields of a 1242 x 375 quad.)
+// fields of a 1242 x 375 quad.)  Without room for the repacked rows the caller's are
+// read as they lie: 9.86 against 9.12 ms.
 struct SiftViews {
     const float4* v[4];  // reference, temporal, stereo, cross
     int w, h, n, sigma;
-    int m;      // columns per residue class
-    int pitch;  // n m: elements per row
+    int mask, shift;  // n - 1 and log2 n; both 0 for the caller's order
+    int m;            // columns per residue class
+    int pitch;        // elements per row
 };
 struct SiftPhi {
     const float4* v[4];
     float4* packed;  // 4 x [h][pitch]
 };
 
-template <int N>
-__device__ __forceinline__ int sift_slot(int x, int m) {
-    return (x & (N - 1)) * m + x / N;
-}
+__device__ __forceinline__ int sift_slot(const SiftViews& S, int x) { return (x & S.mask) * S.m + (x >> S.shift); }
 
 template <int N>
 __global__ void k_sift_pack(SiftPhi P, SiftViews S) {
@@ -1966,9 +1965,9 @@ __device__ __forceinline__ float root_in_range(float x) {
 template <int N>
 __device__ __forceinline__ void sift_column_any(const SiftViews& S, float* d, int q, int px, int py, const Vec4& a) {
     const int x = px + (q - 3) * N;
-    const int s0 = sift_slot<N>(clampi(x, 0, S.w - 1), S.m), s1 = sift_slot<N>(clampi(x + a.u, 0, S.w - 1), S.m),
-              s2 = sift_slot<N>(clampi(x - S.sigma * a.d0, 0, S.w - 1), S.m),
-              s3 = sift_slot<N>(clampi(x + a.u - S.sigma * a.d1, 0, S.w - 1), S.m);
+    const int s0 = sift_slot(S, clampi(x, 0, S.w - 1)), s1 = sift_slot(S, clampi(x + a.u, 0, S.w - 1)),
+              s2 = sift_slot(S, clampi(x - S.sigma * a.d0, 0, S.w - 1)),
+              s3 = sift_slot(S, clampi(x + a.u - S.sigma * a.d1, 0, S.w - 1));
     auto root = [](float v) { return v == 0.0f ? 0.0f : __fsqrt_rn(v); };
 #pragma unroll 1
     for (int j = 0; j < 7; ++j) {
@@ -2021,9 +2020,9 @@ __device__ __forceinline__ int sift_costs(const SiftViews& S, float* buf, int la
             Vec4 a;
             at(k0 + g, px, py, a);
             const int x = px + col;
-            const int s0 = sift_slot<N>(clampi(x, 0, S.w - 1), S.m), s1 = sift_slot<N>(clampi(x + a.u, 0, S.w - 1), S.m),
-                      s2 = sift_slot<N>(clampi(x - S.sigma * a.d0, 0, S.w - 1), S.m),
-                      s3 = sift_slot<N>(clampi(x + a.u - S.sigma * a.d1, 0, S.w - 1), S.m);
+            const int s0 = sift_slot(S, clampi(x, 0, S.w - 1)), s1 = sift_slot(S, clampi(x + a.u, 0, S.w - 1)),
+                      s2 = sift_slot(S, clampi(x - S.sigma * a.d0, 0, S.w - 1)),
+                      s3 = sift_slot(S, clampi(x + a.u - S.sigma * a.d1, 0, S.w - 1));
             float* d = buf + (k0 + g) * kSiftStride + 3 * q;
 #pragma unroll
             for (int j = 0; j < 7; ++j) {
@@ -2909,7 +2908,8 @@ int run_fields(const FieldSpec* spec, int nf, const sff_params& P, const sff_tun
 // One field with the paper's own cost: the WHT K-NN of the coarsest scale as
 // in run_fields, then initialisation, inheritance, half-steps and random
 // search in the kernels above.  phi[4]: [S][H][W] float4 of the views in the
-// field's roles (reference, temporal, stereo, cross).
+// field's roles (reference, temporal, stereo, cross).  pack: room for the repacked
+// phi (sift_pack_bytes), or nullptr.
 int run_field_sift(const FieldSpec& fs, const float* const* phi, const sff_params& P, void* pack, cudaStream_t st) {
     const int S = P.num_scales, I = P.iterations, w = fs.width, h = fs.height;
     static const int kDirs[4][2] = {{1, 1}, {-1, -1}, {1, -1}, {-1, 1}};
@@ -2947,14 +2947,17 @@ int run_field_sift(const FieldSpec& fs, const float* const* phi, const sff_param
         SV.h = h;
         SV.n = N;
         SV.sigma = fs.mirror ? -1 : 1;
-        SV.m = (w + N - 1) / N;
-        SV.pitch = N * SV.m;
+        const bool packed = N > 1 && pack;
+        SV.mask = packed ? N - 1 : 0;
+        SV.shift = packed ? s : 0;
+        SV.m = packed ? gw : w;
+        SV.pitch = packed ? N * gw : w;
         SP.packed = reinterpret_cast<float4*>(pack);
         for (int k = 0; k < 4; ++k) {
             SP.v[k] = reinterpret_cast<const float4*>(phi[k]) + off;
-            SV.v[k] = N > 1 ? SP.packed + (size_t)k * h * SV.pitch : SP.v[k];
+            SV.v[k] = packed ? SP.packed + (size_t)k * h * SV.pitch : SP.v[k];
         }
-        if (N > 1) SFF_LAUNCH(k_sift_pack<N>, dim3((SV.pitch + 255) / 256, h, 4), 256, 0, st, SP, SV);
+        if (packed) SFF_LAUNCH(k_sift_pack<N>, dim3((SV.pitch + 255) / 256, h, 4), 256, 0, st, SP, SV);
         if (s == S - 1) {
             A.V = Views{plane_of(fs.ref, s, S, w, h), plane_of(fs.tmp, s, S, w, h), plane_of(fs.ste, s, S, w, h),
                         plane_of(fs.crs, s, S, w, h), w, h, fs.mirror ? -1 : 1};
@@ -3187,18 +3190,8 @@ extern "C" int sff_match_views_sift(const uint8_t* pyr_ref_dev, const uint8_t* p
     if (workspace_bytes < match_ws_bytes(width, height, *params)) return SFF_ERR_WORKSPACE;
     FieldSpec f{pyr_ref_dev, pyr_temporal_dev, pyr_stereo_dev, pyr_cross_dev, field_dev, cost_dev, mirror,
                 width, height, seed, workspace};
-    // a workspace of two fields' scratch is enough: the repacked phi is then
-    // allocated and freed in stream order
-    const cudaStream_t st = (cudaStream_t)stream;
-    void *pack = reinterpret_cast<char*>(workspace) + field_ws_bytes(width, height, *params), *own = nullptr;
-    if (workspace_bytes < sift_match_ws_bytes(width, height, *params)) {
-        if (cudaMallocAsync(&own, sift_pack_bytes(width, height, *params), st) != cudaSuccess) {
-            cudaGetLastError();
-            return SFF_ERR_WORKSPACE;
-        }
-        pack = own;
-    }
-    const int rc = run_field_sift(f, phi, *params, pack, st);
-    if (own && cudaFreeAsync(own, st) != cudaSuccess && rc == SFF_OK) return SFF_ERR_CUDA;
-    return rc;
+    // a workspace of two fields' scratch is enough: the phi is then not repacked
+    const bool room = workspace_bytes >= sift_match_ws_bytes(width, height, *params);
+    void* pack = reinterpret_cast<char*>(workspace) + field_ws_bytes(width, height, *params);
+    return run_field_sift(f, phi, *params, room ? pack : nullptr, (cudaStream_t)stream);
 }
