@@ -395,7 +395,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_knn_tc(const __grid_constant_
         // ---- MMAs (one thread)
         if (lane == 0) {
             int committed = 0;
-            const int withhold = g_withhold_step < 0 ? -1 : g_withhold_step / (kTcCand / 128);  // in 128-candidate visits
+            // counted in visits of 128 candidates, two of a pass at a time here
+            const int visits = (gq + 127) / 128, at = g_withhold_step;
+            const int withhold = at < 0 || at >= 2 * visits ? -1 : at / visits * nt + at % visits / 2;
             bool ok = mbar_wait(bar_q, 0, wait_ns);
             const uint32_t qaddr = smem_addr(sQ);
             for (int u = 0; ok && u < steps; ++u) {
