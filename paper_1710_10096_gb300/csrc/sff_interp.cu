@@ -36,7 +36,7 @@
 //
 // k_interp_clear:  empty map, status, weight table.
 // k_interp_prep:   map words and triangulated points of every seed.
-// k_interp_models: one warp per seed: one pass over rings of blocks collects
+// k_interp_models: one warp per one or two seeds: one pass over rings of blocks collects
 //                  the candidates of both neighbourhoods, bisection selects
 //                  them, the normal equations accumulate in double precision.
 // k_interp_columns: per pixel column the closest seed in that column, for
@@ -50,8 +50,9 @@ namespace {
 
 constexpr int kBlock = 3;            // sparsification block of Sec. 3.2
 constexpr int kModelWarps = 1;       // warps per CTA of k_interp_models
-constexpr int kModelResident = 20;   // ... and CTAs per SM that its registers allow
-constexpr int kSeedsPerWarp = 2;     // seeds whose sums share a warp's instructions (16 lanes each)
+constexpr int kModelResident = 20;   // ... and CTAs per SM that its registers allow,
+constexpr int kModelResidentLone = 12;  // in the form of one seed per warp
+constexpr int kMinResidentPairs = 15;  // two seeds per warp only if this many fit an SM
 constexpr int kMaxK = 1024;          // largest k_geo / k_motion
 constexpr int kRegKeys = 16;         // candidate keys per lane held in registers during selection (half are, up to 256)
 constexpr int kTighten = 4;          // the ring bound is within 1/16 of the k-th distance so far
@@ -436,8 +437,8 @@ __device__ __forceinline__ void solve4(const Factor4& F, double (&b)[4]) {
 // Shared memory of one warp of k_interp_models: candidate positions and map words
 // (J.slots each), the neighbour lists of its seeds (k_geo, k_motion position and
 // word pairs each), 32 ints of scratch.
-__host__ __device__ __forceinline__ size_t warp_smem_bytes(int slots, int kg, int km) {
-    return (size_t)slots * 8 + (size_t)kSeedsPerWarp * (kg + km) * 8 + 128;
+__host__ __device__ __forceinline__ size_t warp_smem_bytes(int slots, int kg, int km, int seeds) {
+    return (size_t)slots * 8 + (size_t)seeds * (kg + km) * 8 + 128;
 }
 
 // The two neighbourhoods of seed si into la[kg] and lm[km]; false when the
@@ -602,7 +603,7 @@ __device__ __forceinline__ bool select_neighbours(const InterpJob& J, int si, in
     return na <= kg && nm <= km;  // at most k members are selected
 }
 
-// One warp per two seeds: the whole warp selects each seed's neighbourhoods in
+// One warp per two seeds (SP = 2): the whole warp selects each seed's neighbourhoods in
 // turn, then the sums of both run side by side, 16 lanes per seed.  An FP64
 // instruction holds its sub-partition's pipe for 64 clocks whatever its active
 // lanes, so what counts is the number of warp instructions: with 32 lanes per seed
@@ -623,19 +624,25 @@ __device__ __forceinline__ bool select_neighbours(const InterpJob& J, int si, in
 //     selections, which scan more rings, then outweigh the sums, and differ more from
 //     warp to warp (4693 on 39195 blocks 352 / 313, 15110 on 51750 533 / 461, 59975 on
 //     122574 1287 / 1306; 16012 on 30000, above half, 402 / 393).
-__global__ void __launch_bounds__(kModelWarps * 32, kModelResident) k_interp_models(InterpJob J) {
-    constexpr int SP = kSeedsPerWarp, W = 32 / SP;
-    static_assert(SP == 2, "a lone seed's sums are in two halves");
+// With larger neighbourhoods the second seed's lists cost more warps than the shared
+// instructions save: SP = 1, one seed per warp at any number, where fewer than 15 warps
+// of two would fit an SM (37749 seeds, us two / one: k 200/100, 16 warps, 951 / 960;
+// 250/125, 13 warps, 1172 / 1120; 400/300 2167 / 1957; 1024/1024 13791 / 9911).
+template <int SP>
+__global__ void __launch_bounds__(kModelWarps * 32, SP == 2 ? kModelResident : kModelResidentLone)
+    k_interp_models(InterpJob J) {
+    constexpr int W = 16;  // lanes per seed of two, and half the lanes of a lone one's
+    static_assert(SP == 1 || SP == 2, "seeds per warp");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int n = seed_count(J);
     // one seed, its sums over all lanes (the line as a word of its own: with the rule's
     // comparisons here the kernel took 1 % more)
-    const bool lone = n <= *J.lone_max;
+    const bool lone = SP == 1 || n <= *J.lone_max;
     const int s0 = (blockIdx.x * kModelWarps + wid) * (lone ? 1 : SP);
     if (s0 >= n) return;  // warp-uniform
     const int kg = J.p.k_geo, km = J.p.k_motion;
-    unsigned char* mine = smem_raw + (size_t)wid * warp_smem_bytes(J.slots, kg, km);
+    unsigned char* mine = smem_raw + (size_t)wid * warp_smem_bytes(J.slots, kg, km, SP);
     uint32_t* pos = reinterpret_cast<uint32_t*>(mine);
     int* word = reinterpret_cast<int*>(mine + (size_t)J.slots * 4);
     uint2* lists = reinterpret_cast<uint2*>(mine + (size_t)J.slots * 8);
@@ -1029,21 +1036,25 @@ extern "C" int sff_interpolate(const sff_seed* seeds_dev, const int32_t* count_d
     J.fb = params->focal * params->baseline;
     J.inv_f = 1.0 / params->focal;
     J.slots = candidate_slots(params->k_geo, params->k_motion);
-    const size_t smem = kModelWarps * warp_smem_bytes(J.slots, J.p.k_geo, J.p.k_motion);
-    J.resident = kModelWarps * kSms * min(kModelResident, (int)(kSmemPerSm / (smem + kSmemPerCta)));
+    const size_t pair_smem = kModelWarps * warp_smem_bytes(J.slots, J.p.k_geo, J.p.k_motion, 2);
+    const int per_sm = kModelWarps * min(kModelResident, (int)(kSmemPerSm / (pair_smem + kSmemPerCta)));
+    const bool pairs = per_sm >= kMinResidentPairs;
+    J.resident = kSms * per_sm;
     cudaStream_t st = (cudaStream_t)stream;
     const int clear = max(J.gbw * J.gbh, kWeightTable);
     SFF_LAUNCH(k_interp_clear, dim3((clear + 255) / 256), 256, 0, st, J);
     if (capacity > 0) {
         SFF_LAUNCH(k_interp_prep, dim3((capacity + 255) / 256), 256, 0, st, J);
+        void (*const k_interp_models)(InterpJob) = pairs ? sff::k_interp_models<2> : sff::k_interp_models<1>;
+        const size_t smem =
+            pairs ? pair_smem : kModelWarps * warp_smem_bytes(J.slots, J.p.k_geo, J.p.k_motion, 1);
         if (smem > 48 * 1024 &&
             cudaFuncSetAttribute(k_interp_models, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
             return SFF_ERR_CUDA;
-        // enough warps for either split; those without a seed leave at once
+        // pairs: enough warps for either split; those without a seed leave at once
         const int lone = min(capacity, max(J.resident * 10 / 3, J.gbw * J.gbh / 2));
-        const int warps = max((capacity + kSeedsPerWarp - 1) / kSeedsPerWarp, lone);
-        const int blocks = (warps + kModelWarps - 1) / kModelWarps;
-        SFF_LAUNCH(k_interp_models, dim3(blocks), kModelWarps * 32, smem, st, J);
+        const int warps = pairs ? max((capacity + 1) / 2, lone) : capacity;
+        SFF_LAUNCH(k_interp_models, dim3((warps + kModelWarps - 1) / kModelWarps), kModelWarps * 32, smem, st, J);
         SFF_LAUNCH(k_interp_solve, dim3((capacity + 63) / 64, 2), 64, 0, st, J);
     }
     int2* col = reinterpret_cast<int2*>(ws + L.nearest);

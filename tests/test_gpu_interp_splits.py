@@ -54,3 +54,31 @@ def test_counts_at_the_splits(w, h, count):
     want, _ = oracle.interpolate_pixels(sd, p, pix, models=oracle.seed_models(sd, p, which=closest))
     assert {0, 1, count - 2, count - 1} <= set(closest.tolist())
     np.testing.assert_allclose(field.cpu().numpy()[pix[:, 1], pix[:, 0]], want, rtol=1e-5, atol=1e-3)
+
+
+@pytest.mark.parametrize("kg,km", [(200, 100), (240, 120), (250, 125), (400, 300), (1024, 1024), (7, 1024)])
+@pytest.mark.parametrize("count", [1, 33, 4001])
+def test_neighbourhoods_at_the_split(kg, km, count):
+    # two seeds per warp up to 220 / 110 neighbours, one each above
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import oracle
+    import paper_1710_10096_gb300 as sff
+    sff.build()
+    oracle.build()
+    oracle.set_threads(os.cpu_count() or 1)
+    w, h = 265, 200
+    gt, occ, f, b = scenegen.ground_truth("planes", w, h, 3)
+    s = scenegen.sparse_seeds(gt, np.zeros_like(occ), seed=5, keep=1.0, noise=0.3)
+    s = s[np.sort(np.random.default_rng(kg + count).permutation(len(s))[:count])]
+    s["d1"][1::3] = 0  # geometry only
+    raw = torch.as_tensor(np.frombuffer(np.ascontiguousarray(s).tobytes(), np.uint8).copy()).cuda()
+    field = torch.empty((h, w, 4), dtype=torch.float32, device="cuda")
+    ws = torch.empty(sff.interp_workspace_bytes(w, h, count), dtype=torch.uint8, device="cuda")
+    sff.interpolate(raw, torch.tensor([count], dtype=torch.int32, device="cuda"), count, w, h,
+                    sff.default_interp_params(w, h, f, b, k_geo=kg, k_motion=km), field, ws)
+    torch.cuda.synchronize()
+    assert sff.interp_status(ws, w, h, count) == 0
+    want = oracle.interpolate(s, w, h, oracle.interp_params(w, h, f, b, k_geo=kg, k_motion=km))
+    np.testing.assert_allclose(field.cpu().numpy(), want, rtol=1e-5, atol=1e-3)
