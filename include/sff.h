@@ -586,7 +586,9 @@ int sff_profile_enable(int32_t on);
 int sff_profile_collect(sff_kernel_time* out, int32_t capacity, int32_t* n_out);
 
 /* Number of device-side bounded waits (on the completion of the library's own
- * asynchronous copies and tensor-core operations) that gave up since the last
+ * asynchronous copies and tensor-core operations, on other CTAs of a fused scale
+ * and on other rows of a sequential sweep; those of sff_features_tc and
+ * sff_sift_features are in sff_device_status alone) that gave up since the last
  * reset; nonzero means a result is invalid.  reset also clears the drain count
  * below.  Synchronises the current device.  Host pointer. */
 int sff_device_timeouts(uint32_t* out, int32_t reset);
@@ -613,10 +615,12 @@ int sff_int_peak(int32_t kind, double* ops_per_s, void* stream);
  * conditions that kernels of this library raised on the current device since
  * the last reset:
  *   SFF_ERR_TIMEOUT   a bounded device wait gave up (the temporal K-NN's
- *                     waits on its bulk copies and MMAs): the fields, and
- *                     everything computed from them, of the calls since the
- *                     last reset are invalid (their pixels may be empty,
- *                     never out of bounds);
+ *                     waits on its bulk copies and MMAs, a fused scale's grid
+ *                     barrier, the sequential sweep's waits between rows, the
+ *                     MMA waits of sff_features_tc and sff_sift_features): the
+ *                     features or fields, and everything computed from them,
+ *                     of the calls since the last reset are invalid (a field's
+ *                     pixels may be empty, never out of bounds);
  *   SFF_ERR_CAPACITY  otherwise, if sff_emit_seeds / sff_emit_seeds_geo /
  *                     sff_run_batch found more seeds than a seed buffer's
  *                     capacity: the first `capacity` seeds were written and

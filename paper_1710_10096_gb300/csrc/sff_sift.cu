@@ -651,7 +651,7 @@ SiftLayout sift_layout(int w, int h, int scales) {
 }
 
 // The scratch that sff_sift_workspace_bytes asks for holds every scale's
-// descriptors up to this size (2 KB per pixel, 5.6 GiB at most), so that the
+// descriptors up to this size (2 KB per pixel, 4.0 GiB at most), so that the
 // coarser scales' can be computed while the axes are; a larger image's holds
 // one scale's.
 constexpr size_t kOverlapPixels = (size_t)1 << 21;
